@@ -94,6 +94,7 @@ struct dlma_ctx {
   uint64_t memcap = 0;
   uint64_t work_bytes = 0;      // bytes currently held in work buffers
   double timing[kTimingSlots] = {0};
+  cudaEvent_t ev[2] = {nullptr, nullptr};   // timing events of the operator calls
   // stencil block shape (sites x right-hand sides) per precision, chosen by autotune_hop
   int hop_sx[3] = {64, 64, 64}, hop_sy[3] = {4, 4, 4}, hop_tuned[3] = {0, 0, 0};
   int hop_l18[3] = {0, 0, 0};   // FP32: read 18-real links instead of rebuilding row 2
@@ -215,12 +216,17 @@ template <class T> dlma_status workT(dlma_ctx* ctx, int slot, size_t count, T** 
 //   FP64  double2 [12][Vh]
 //   FP32  float4  [6][Vh]      (complex components 2q, 2q+1 in one float4)
 //   FP16S uint4   [3][Vh]      (complex components 4q..4q+3) + float scale [Vh]
+// A FP64 field may also stand for a caller's canonical array (lay), which only the
+// stencil's split form reads and writes in place: half = one parity, complex
+// [V/2][4][3] per right-hand side; full = the sites of one parity inside [V][4][3].
+enum { kLayInternal = 0, kLayHalf = 1, kLayFull = 2 };
 struct Field {
   void* data = nullptr;
   float* scale = nullptr;
   int prec = DLMA_FP64;
   int nrhs = 0;
   int Vh = 0;
+  int lay = kLayInternal;
 };
 
 __host__ __device__ inline size_t field_units_per_rhs(int prec, int Vh) {
@@ -270,7 +276,16 @@ struct HopOp {
 };
 dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Field* own, Field& out,
                        int* nblocks_out = nullptr);
-int hop_grid_x(dlma_ctx* ctx, int prec);
+// site tiles of a hop launch over the whole parity (= partial sums per right-hand side)
+int hop_grid_x(dlma_ctx* ctx, int prec, int nrhs);
+// whether hop launches on nrhs right-hand sides take the split form (hop_split.cuh).
+// k_hop needs 87 us per FP64 Schur application for any number of (even site, rhs) pairs
+// up to 19456 (one warp per SM sub-partition); the split form 20 us up to 1024 pairs, 31
+// at 3072, 49 at 6144, 80 at 12288 and 120 at 19456 (4^3 x 8 to 10^3 x 18 alike)
+constexpr int kHopSplitPairs = 12500;
+inline bool hop_split(const dlma_ctx* ctx, int prec, int nrhs) {
+  return prec == DLMA_FP64 && (size_t)ctx->g.Vh * nrhs < (size_t)kHopSplitPairs;
+}
 
 // Schur operator on even fields: out = Dhat in (dagger: gamma5 Dhat gamma5), tmp: odd work field
 dlma_status schur_apply(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, int dagger,

@@ -394,6 +394,8 @@ static void free_all(dlma_ctx* ctx) {
   if (ctx->dirac_V) cudaFree(ctx->dirac_V);
   for (int i = 0; i < WS_COUNT; i++)
     if (ctx->wb[i].p) cudaFree(ctx->wb[i].p);
+  for (cudaEvent_t e : ctx->ev)
+    if (e) cudaEventDestroy(e);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
   if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
 }

@@ -14,6 +14,7 @@
 #include "common.cuh"
 
 #include "fieldio.cuh"
+#include "hop_split.cuh"
 
 // link U_mu(x) for x of parity p at compressed index i
 template <int P>
@@ -483,8 +484,8 @@ static inline void hop_block(dlma_ctx* ctx, int prec, int& sx, int& sy) {
   sy = ctx->hop_sy[prec];
 }
 
-// number of site tiles of a hop launch (= partial sums per right-hand side)
-int hop_grid_x(dlma_ctx* ctx, int prec) {
+int hop_grid_x(dlma_ctx* ctx, int prec, int nrhs) {
+  if (hop_split(ctx, prec, nrhs)) return (ctx->g.Vh + kSplitSites - 1) / kSplitSites;
   int sx, sy;
   hop_block(ctx, prec, sx, sy);
   return (ctx->g.Vh + sx - 1) / sx;
@@ -522,9 +523,58 @@ static void dispatch_cgu(dim3 grid, dim3 blk, cudaStream_t st, const HopArgs& a)
   k_hop<P, 1, false, true, 2, false, true, true, L18, true><<<grid, blk, 0, st>>>(a);
 }
 
+// the split form of launch_hop (FP64; any combination of terms but the DOT epilogue)
+static dlma_status launch_hop_split(dlma_ctx* ctx, const HopOp& op, const Field& in, const Field* own, Field& out,
+                                    int* nblocks_out) {
+  const size_t Vh = ctx->g.Vh;
+  if (op.own >= 2 && op.kout) return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil with two site matrices");
+  auto view = [&](const Field& f) {
+    SplitView v;
+    v.p = (double2*)f.data;
+    v.lay = f.lay;
+    v.rhs = (f.lay == kLayFull ? 24 : 12) * Vh;
+    return v;
+  };
+  SplitArgs a;
+  a.g = ctx->g;
+  a.p_out = op.p_out;
+  a.nrhs = out.nrhs;
+  a.site0 = op.nsites >= 0 ? op.site0 : 0;
+  a.nsites = op.nsites >= 0 ? op.nsites : ctx->g.Vh;
+  if (a.nsites == 0) return DLMA_OK;
+  a.ntiles = (a.nsites + kSplitSites - 1) / kSplitSites;
+  a.in = view(in);
+  if (own) a.own = view(*own);
+  a.out = view(out);
+  a.U = ctx->U64;
+  a.Kown = (op.own == 3 ? ctx->Ci64 : ctx->C64) + op.p_out * 36 * Vh;
+  a.Kout = (op.kout == 2 ? ctx->C64 : ctx->Ci64) + op.p_out * 36 * Vh;
+  a.s = op.s;
+  a.hop = op.hop;
+  a.g5_in = op.g5_in;
+  a.g5_hop = op.g5_hop;
+  a.own_op = op.own >= 2 ? 2 : op.own;
+  a.kout = op.kout != 0;
+  a.active = op.active;
+  a.nbr = ctx->nbr_tab;
+  a.norm_part = op.norm_part;
+  a.cg_x = (double2*)op.cg_x;
+  a.cg_r = (double2*)op.cg_r;
+  a.cg_p = (const double2*)op.cg_p;
+  a.cg_alpha = op.cg_alpha;
+  k_hop_split<<<(unsigned)((size_t)a.ntiles * a.nrhs), 16 * kSplitSites, 0, ctx->stream>>>(a);
+  CHECK_LAUNCH();
+  if (nblocks_out) *nblocks_out = a.ntiles;
+  return DLMA_OK;
+}
+
 dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Field* own, Field& out,
                        int* nblocks_out) {
   const int P = out.prec;
+  if (op.nsites >= 0 && (op.norm_part || op.dot_part || op.cg_x || op.nsites > ctx->g.Vh || op.site0 < 0 ||
+                         op.site0 >= ctx->g.Vh))
+    return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil site range");
+  if (!op.dot_part && hop_split(ctx, P, out.nrhs)) return launch_hop_split(ctx, op, in, own, out, nblocks_out);
   HopArgs a;
   a.g = ctx->g;
   a.bc_t = ctx->bc_t;
@@ -579,9 +629,6 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   const bool cgu = op.cg_x != nullptr && op.hop;
   const bool dot = op.dot_part != nullptr && op.hop && op.own == 2 && !op.kout && !op.g5_hop;
   const int nr = (P == DLMA_FP32 && !cgu) ? ctx->hop_nr[P] : 1;
-  if (op.nsites >= 0 && (op.norm_part || op.dot_part || op.cg_x || op.nsites > ctx->g.Vh || op.site0 < 0 ||
-                         op.site0 >= ctx->g.Vh))
-    return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil site range");
   a.site0 = op.nsites >= 0 ? op.site0 : 0;
   a.nsites = op.nsites >= 0 ? op.nsites : ctx->g.Vh;
   if (a.nsites == 0) return DLMA_OK;
@@ -630,7 +677,8 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
 // sides per thread), then for each chunk size of the block order, and keep the
 // fastest for this precision.
 dlma_status autotune_hop(dlma_ctx* ctx, int prec, const Field& in, Field& tmp, Field& out) {
-  if (ctx->hop_tuned[prec]) return DLMA_OK;
+  // the split form has no shape to tune, and its batches say nothing about larger ones
+  if (ctx->hop_tuned[prec] || hop_split(ctx, prec, in.nrhs)) return DLMA_OK;
   static const int cand[][2] = {{32, 8}, {64, 4}, {128, 2}, {256, 1}, {32, 4}, {64, 2}, {32, 2}};
   cudaEvent_t e0, e1;
   CU(cudaEventCreate(&e0));
@@ -848,6 +896,20 @@ static dlma_status check_ready(dlma_ctx* ctx) {
   return DLMA_OK;
 }
 
+// a caller's canonical FP64 array as a field of the split stencil
+static Field canonical(dlma_ctx* ctx, const double* p, int nrhs, int lay) {
+  Field f;
+  f.data = (void*)p;
+  f.nrhs = nrhs;
+  f.Vh = ctx->g.Vh;
+  f.lay = lay;
+  return f;
+}
+// (overlapping input and output go through the packed copies)
+static bool disjoint(const double* a, const double* b, size_t bytes) {
+  return (const char*)a + bytes <= (const char*)b || (const char*)b + bytes <= (const char*)a;
+}
+
 extern "C" dlma_status dlma_apply_Dw(dlma_ctx* ctx, const double* in, double* out, int nrhs, dlma_prec prec,
                                      dlma_mem mem) {
   TRY(check_ready(ctx));
@@ -858,6 +920,16 @@ extern "C" dlma_status dlma_apply_Dw(dlma_ctx* ctx, const double* in, double* ou
   TRY(copy_in(ctx, WS_IN, in, bytes, mem, &din));
   double* dout = out;
   if (mem == DLMA_MEM_HOST) TRY(workT(ctx, WS_OUT, bytes / 8, &dout));
+  if (hop_split(ctx, prec, nrhs) && disjoint(din, dout, bytes)) {   // in place on the canonical arrays
+    const Field fi = canonical(ctx, din, nrhs, kLayFull);
+    Field fr = canonical(ctx, dout, nrhs, kLayFull);
+    HopOp op;
+    op.own = 2;
+    for (op.p_out = 0; op.p_out < 2; op.p_out++) TRY(launch_hop(ctx, op, fi, &fi, fr));
+    if (mem == DLMA_MEM_HOST) TRY(copy_out(ctx, out, dout, bytes, mem));
+    CU(cudaStreamSynchronize(ctx->stream));
+    return DLMA_OK;
+  }
   Field fe, fo, re, ro;
   TRY(field_alloc(ctx, WS_T0, prec, nrhs, &fe));
   TRY(field_alloc(ctx, WS_T1, prec, nrhs, &fo));
@@ -898,28 +970,32 @@ extern "C" dlma_status dlma_apply_schur(dlma_ctx* ctx, const double* in, double*
   TRY(copy_in(ctx, WS_IN, in, bytes, mem, &din));
   double* dout = out;
   if (mem == DLMA_MEM_HOST) TRY(workT(ctx, WS_OUT, bytes / 8, &dout));
+  // few pairs: the split stencil reads and writes the canonical arrays themselves
+  const bool direct = hop_split(ctx, prec, nrhs) && disjoint(din, dout, bytes);
   Field fe, tmp, res;
-  TRY(field_alloc(ctx, WS_T0, prec, nrhs, &fe));
   TRY(field_alloc(ctx, WS_T1, prec, nrhs, &tmp));
-  TRY(field_alloc(ctx, WS_T2, prec, nrhs, &res));
-  TRY(pack_parity(ctx, din, 0, 0, fe));
-  TRY(autotune_hop(ctx, prec, fe, tmp, res));
-  EvTimer ev;
-  CU(cudaEventCreate(&ev.a));
-  CU(cudaEventCreate(&ev.b));
-  CU(cudaEventRecord(ev.a, ctx->stream));
+  if (direct) {
+    fe = canonical(ctx, din, nrhs, kLayHalf);
+    res = canonical(ctx, dout, nrhs, kLayHalf);
+  } else {
+    TRY(field_alloc(ctx, WS_T0, prec, nrhs, &fe));
+    TRY(field_alloc(ctx, WS_T2, prec, nrhs, &res));
+    TRY(pack_parity(ctx, din, 0, 0, fe));
+    TRY(autotune_hop(ctx, prec, fe, tmp, res));
+  }
+  for (cudaEvent_t& e : ctx->ev)
+    if (!e) CU(cudaEventCreate(&e));
+  CU(cudaEventRecord(ctx->ev[0], ctx->stream));
   TRY(schur_apply(ctx, fe, tmp, res, dagger ? 1 : 0, nullptr, nullptr));
-  CU(cudaEventRecord(ev.b, ctx->stream));
-  TRY(unpack_parity(ctx, res, 0, 0, dout));
+  CU(cudaEventRecord(ctx->ev[1], ctx->stream));
+  if (!direct) TRY(unpack_parity(ctx, res, 0, 0, dout));
   if (mem == DLMA_MEM_HOST) TRY(copy_out(ctx, out, dout, bytes, mem));
   CU(cudaStreamSynchronize(ctx->stream));
   float ms = 0;
-  cudaEventElapsedTime(&ms, ev.a, ev.b);
+  cudaEventElapsedTime(&ms, ctx->ev[0], ctx->ev[1]);
   for (int i = 0; i < kTimingSlots; i++) ctx->timing[i] = 0;
   ctx->timing[0] = ms;
   ctx->timing[1] = ms;
   ctx->timing[2] = 2;
-  cudaEventDestroy(ev.a);
-  cudaEventDestroy(ev.b);
   return DLMA_OK;
 }

@@ -722,7 +722,7 @@ template <int PB, int PS>
 static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since, double delta2) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
-  const int nbh = hop_grid_x(ctx, PS);
+  const int nbh = hop_grid_x(ctx, PS, nrhs);
   // q = Dhat p ; |q|^2 partials
   TRY(schur_apply(ctx, B.ps, B.tmp, B.q, 0, B.sc.active, B.part));
   k_cg_alpha<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.part, nbh, nrhs, B.sc);
@@ -826,7 +826,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
     TRY(field_alloc(ctx, WS_BI_S, PB, nrhs, &B.sl));
     TRY(field_alloc(ctx, WS_BI_R0, PB, nrhs, &B.r0));
   }
-  const int nbmax = (Vh + 31) / 32 + 8;
+  const int nbmax = std::max((Vh + 31) / 32, hop_split(ctx, PS, nrhs) ? hop_grid_x(ctx, PS, nrhs) : 0) + 8;
   TRY(workT(ctx, WS_PART, (size_t)2 * nbmax * nrhs, &B.part));
   B.part2 = B.part + (size_t)nbmax * nrhs;
   if (bicg) {
@@ -1185,7 +1185,7 @@ template <int P>
 static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since, double delta2) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
-  const int nbh = hop_grid_x(ctx, P);
+  const int nbh = hop_grid_x(ctx, P, nrhs);
   const int nw = (nrhs + 3) / 4;
   // v = Dhat p (into q) with the partials of (r0, v)
   TRY(schur_apply_dot(ctx, B.pl, B.tmp, B.q, B.sc.active, B.r0, B.cpart, nullptr));
