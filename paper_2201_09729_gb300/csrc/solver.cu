@@ -30,6 +30,7 @@ struct CgScal {
   double* alpha;
   double* beta;
   double* stop2;   // |r|^2 that triggers the next reliable update
+  double* rr0;     // |r|^2 right after the last update
   double* rnorm;   // FP64 Schur residual norm per rhs (at the last update)
   double* bnorm;   // |b| per rhs (full lattice)
   double* scale;   // s_j = |bhat_j|: the low-precision system solves for x / s_j
@@ -77,7 +78,7 @@ __global__ void k_cg_alpha(const double* part, int nb, int nrhs, CgScal sc) {
 }
 
 // beta_j; pause for a reliable update when |r|^2 fell below stop2 or after max_since iterations
-__global__ void k_cg_beta(const double* part, int nb, int nrhs, CgScal sc, int max_since, double delta2) {
+__global__ void k_cg_beta(const double* part, int nb, int nrhs, CgScal sc, int max_since) {
   const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   if (j >= nrhs || !sc.active[j]) return;
   const int lane = threadIdx.x & 31;
@@ -96,7 +97,7 @@ __global__ void k_cg_beta(const double* part, int nb, int nrhs, CgScal sc, int m
     // p update (k_pause), so the search direction stays consistent with r.  An
     // exhausted recursion (|r| = 0 or an overflowing beta) also asks for the FP64 check.
     else if (rrn <= sc.stop2[j] || sc.since[j] >= max_since || !(rrn > 0) || !isfinite(bt) ||
-             rrn * delta2 > 1e4 * sc.stop2[j])    // |r|^2 grew 1e4 x above its value at the last update
+             rrn > 1e4 * sc.rr0[j])               // |r|^2 grew 1e4 x above its value at the last update
       sc.ru[j] = 1;
   }
 }
@@ -358,8 +359,20 @@ __global__ void k_ru_check(int nrhs, CgScal sc, double tol) {
   sc.upd[j] = 1;
 }
 
+// reduction of the iterated residual at which the next reliable update is due: delta,
+// or less when the tolerance is nearer than that.  A cycle of delta that starts just
+// above the tolerance would iterate a whole cycle too far (FP64 CGNE to 1e-12 on
+// 4^3 x 8, delta 1e-6: 104 iterations against 78); at least a factor 10, so that a cycle
+// that did its work is never taken for a stalled one.  margin: how far the iterated
+// residual has to drop for the Schur residual to drop by the factor that is missing
+__device__ __forceinline__ double next_stop(const CgScal& sc, int j, double delta, double tol, double margin) {
+  const double need = tol * sc.bnorm[j] / sc.rnorm[j];
+  const double f = fmax(delta, fmin(0.1, margin * need));
+  return f * f;
+}
+
 // resume the updated rhs with the recomputed normal-equation residual
-__global__ void k_resume(int nrhs, CgScal sc, double delta2) {
+__global__ void k_resume(int nrhs, CgScal sc, double delta, double tol) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nrhs || !sc.upd[j]) return;
   const double rr = sc.rrnew[j];
@@ -371,8 +384,9 @@ __global__ void k_resume(int nrhs, CgScal sc, double delta2) {
     sc.alive[j] = 0;
     return;
   }
-  sc.rr[j] = rr;
-  sc.stop2[j] = delta2 * rr;
+  sc.rr[j] = sc.rr0[j] = rr;
+  // the normal-equation residual Dhat^dag r falls ahead of r: aim further
+  sc.stop2[j] = next_stop(sc, j, delta, tol, 0.1) * rr;
   sc.active[j] = 1;
 }
 
@@ -539,7 +553,7 @@ __global__ void __launch_bounds__(BX) k_bi_xr(int Vh, int nrhs, void* x, void* r
 
 // rho_new = (r0, r), |r|^2; beta = (rho_new / rho) (alpha / omega); reliable-update triggers
 __global__ void k_bi_beta(const double2* cpart, const double* npart, int nb, int nrhs, CgScal sc, BiScal bs,
-                          int max_since, double delta2) {
+                          int max_since) {
   const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   if (j >= nrhs || !sc.active[j]) return;
   const int lane = threadIdx.x & 31;
@@ -563,7 +577,7 @@ __global__ void k_bi_beta(const double2* cpart, const double* npart, int nb, int
     sc.since[j] += 1;
     if (!isfinite(n)) { sc.active[j] = 0; sc.count[1] = 1; }
     else if (!ok) { sc.ru[j] = 1; bs.brk[j] = 1; }
-    else if (n <= sc.stop2[j] || sc.since[j] >= max_since || !(n > 0) || n * delta2 > 1e4 * sc.stop2[j])
+    else if (n <= sc.stop2[j] || sc.since[j] >= max_since || !(n > 0) || n > 1e4 * sc.rr0[j])
       sc.ru[j] = 1;                        // the pause takes effect after the p update (k_pause)
   }
 }
@@ -653,7 +667,7 @@ __global__ void __launch_bounds__(BX) k_bi_restore(int Vh, int nrhs, const doubl
 
 // resume the updated rhs: rho = (r0, r), |r|^2 from the partials; restart flags consumed
 __global__ void k_bi_resume(const double2* cpart, const double* npart, int nb, int nrhs, CgScal sc, BiScal bs,
-                            double delta2) {
+                            double delta, double tol) {
   const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   if (j >= nrhs || !sc.upd[j]) return;
   const int lane = threadIdx.x & 31;
@@ -678,8 +692,8 @@ __global__ void k_bi_resume(const double2* cpart, const double* npart, int nb, i
       return;
     }
     bs.rho[j] = d;
-    sc.rr[j] = n;
-    sc.stop2[j] = delta2 * n;
+    sc.rr[j] = sc.rr0[j] = n;
+    sc.stop2[j] = next_stop(sc, j, delta, tol, 0.2) * n;
     sc.active[j] = 1;
   }
 }
@@ -719,7 +733,7 @@ static dlma_status rowsum(dlma_ctx* ctx, const double* part, int nb, int nrhs, d
 }
 
 template <int PB, int PS>
-static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since, double delta2) {
+static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
   const int nbh = hop_grid_x(ctx, PS, nrhs);
@@ -729,7 +743,7 @@ static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int ma
   CHECK_LAUNCH();
   // z = Dhat^dag q with the update x += alpha p, r -= alpha z fused into its epilogue
   TRY(schur_dag_cgupdate(ctx, B.q, B.tmp, B.sc.active, B.xl, B.rl, B.pl, B.sc.alpha, B.part2));
-  k_cg_beta<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.part2, nbh, nrhs, B.sc, max_since, delta2);
+  k_cg_beta<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.part2, nbh, nrhs, B.sc, max_since);
   CHECK_LAUNCH();
   k_update_p<PB, PS><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.rl.data, B.pl.data, B.ps.data, B.ps.scale, B.sc);
   CHECK_LAUNCH();
@@ -744,7 +758,7 @@ static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int ma
 // defect-correction restart, used with the FP16 stencil whose rounding makes the
 // kept search direction inconsistent with the recomputed residual)
 template <int PB, int PS>
-static dlma_status reliable_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta2,
+static dlma_status reliable_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta,
                                    bool first, bool restart = false) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
@@ -791,7 +805,7 @@ static dlma_status reliable_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double
       CHECK_LAUNCH();
     }
   }
-  k_resume<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc, delta2);
+  k_resume<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc, delta, tol_target);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
@@ -834,7 +848,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
     B.cpart2 = B.cpart + (size_t)nbmax * nrhs;
   }
   double* sd;
-  TRY(workT(ctx, WS_SCAL, (size_t)10 * nrhs + 64, &sd));
+  TRY(workT(ctx, WS_SCAL, (size_t)11 * nrhs + 64, &sd));
   B.sc.rr = sd;
   B.sc.alpha = sd + nrhs;
   B.sc.beta = sd + 2 * nrhs;
@@ -844,6 +858,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   B.sc.scale = sd + 6 * nrhs;
   B.sc.rrnew = sd + 7 * nrhs;
   B.tmpd = sd + 8 * nrhs;     // 2 nrhs scratch
+  B.sc.rr0 = sd + 10 * nrhs;
   TRY(workT(ctx, WS_T0, (size_t)nrhs + 16, &B.sc.rbest));
   int* si;
   TRY(workT(ctx, WS_ACT, (size_t)16 * nrhs + 32, &si));
@@ -1164,12 +1179,11 @@ static dlma_status solve_batch(dlma_ctx* ctx, const double* b_dev, double* x_dev
   SolveBufs B;
   TRY((solve_setup<PB, PS>(ctx, B, b_dev, nrhs, false)));
   const double tol_target = 0.5 * tol;
-  const double delta2 = delta * delta;
   // the first "update" sets r_l = Dhat^dag (bhat / s) and p = r_l
   dlma_status st = iterate(
-      ctx, B, nrhs, max_inner, [&]() { return inner_iteration<PB, PS>(ctx, B, nrhs, max_since, delta2); },
+      ctx, B, nrhs, max_inner, [&]() { return inner_iteration<PB, PS>(ctx, B, nrhs, max_since); },
       [&](bool first) {
-        return reliable_update<PB, PS>(ctx, B, nrhs, tol_target, delta2, first, !first && PS == DLMA_FP16S);
+        return reliable_update<PB, PS>(ctx, B, nrhs, tol_target, delta, first, !first && PS == DLMA_FP16S);
       });
   if (st != DLMA_OK && st != DLMA_ERR_NOT_CONVERGED && st != DLMA_ERR_TIMEOUT) return st;
   return solve_finish<PB>(ctx, B, x_dev, nrhs, tol, info, st);
@@ -1182,7 +1196,7 @@ static dlma_status solve_batch(dlma_ctx* ctx, const double* b_dev, double* x_dev
 // p = r + beta (p - omega v).  Two operator applications per iteration, the inner
 // products in the stencil's and the vector kernels' epilogues.
 template <int P>
-static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since, double delta2) {
+static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
   const int nbh = hop_grid_x(ctx, P, nrhs);
@@ -1200,7 +1214,7 @@ static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max
   k_bi_xr<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.xl.data, B.rl.data, B.pl.data, B.sl.data, B.z.data, B.r0.data,
                                          B.sc, B.bs, B.cpart2, B.part2);
   CHECK_LAUNCH();
-  k_bi_beta<<<nw, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, max_since, delta2);
+  k_bi_beta<<<nw, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, max_since);
   CHECK_LAUNCH();
   k_bi_p<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.rl.data, B.pl.data, B.q.data, B.sc, B.bs);
   CHECK_LAUNCH();
@@ -1213,7 +1227,7 @@ static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max
 // FP64; the converged retire; the rest continue with r_l = r64 / s and rho = (r0, r_l),
 // restarting r0 = p = r_l on the first update, after a breakdown or on stagnation.
 template <int P>
-static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta2, bool first) {
+static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta, bool first) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
   const int* ru = B.sc.ru;
@@ -1261,7 +1275,8 @@ static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol
   k_bi_restore<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.r64.data, B.sc.scale, B.rl.data, B.r0.data,
                                                B.pl.data, upd, B.rmask, B.cpart2, B.part2);
   CHECK_LAUNCH();
-  k_bi_resume<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, delta2);
+  k_bi_resume<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, delta,
+                                                            tol_target);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
@@ -1272,10 +1287,9 @@ static dlma_status solve_batch_bicg(dlma_ctx* ctx, const double* b_dev, double* 
   SolveBufs B;
   TRY((solve_setup<P, P>(ctx, B, b_dev, nrhs, true)));
   const double tol_target = 0.5 * tol;
-  const double delta2 = delta * delta;
   dlma_status st = iterate(
-      ctx, B, nrhs, max_inner, [&]() { return bicg_iteration<P>(ctx, B, nrhs, max_since, delta2); },
-      [&](bool first) { return bicg_update<P>(ctx, B, nrhs, tol_target, delta2, first); });
+      ctx, B, nrhs, max_inner, [&]() { return bicg_iteration<P>(ctx, B, nrhs, max_since); },
+      [&](bool first) { return bicg_update<P>(ctx, B, nrhs, tol_target, delta, first); });
   if (st != DLMA_OK && st != DLMA_ERR_NOT_CONVERGED && st != DLMA_ERR_TIMEOUT) return st;
   return solve_finish<P>(ctx, B, x_dev, nrhs, tol, info, st);
 }
