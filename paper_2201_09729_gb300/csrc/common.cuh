@@ -170,7 +170,7 @@ enum WorkSlot {
   WS_EIG_X, WS_EIG_Y, WS_EIG_Y2, WS_EIG_W, WS_EIG_G, WS_EIG_PART, WS_EIG_S, WS_EIG_AUX,
   WS_PROJ_V, WS_PROJ_PART, WS_PROJ_C, WS_CON, WS_CON2, WS_SRC, WS_SOL, WS_ETA,
   WS_BI_S, WS_BI_R0, WS_BI_PART, WS_BI_SCAL, WS_RETRY_B, WS_RETRY_X,
-  WS_TC_A, WS_TC_B, WS_TC_E, WS_SUPPORT,
+  WS_TC_A, WS_TC_B, WS_TC_E, WS_TC_P, WS_SUPPORT,
   WS_COUNT
 };
 
