@@ -176,7 +176,7 @@ dlma_status dlma_solve(dlma_ctx* ctx, const double* b, double* x, int nrhs, doub
  * (the default) iterates BiCGStab on the Schur system Dhat x_e = bhat with
  * FP32 vectors and the same FP64 reliable updates (residual replacement when
  * |r| has dropped by 3e-4 since the last update, DLMA_BICG_DELTA in the
- * environment overriding the factor; restart of the shadow residual after a
+ * environment overriding the factor; restart of the search direction after a
  * breakdown or a stagnating update).  The iteration aims at tol / 2; once a
  * right-hand side's FP64 residual is below 1e-3 (tol / 2) / 1.2e-7 times |b|,
  * its next update subtracts the FP32 operator's image of the FP32 solution

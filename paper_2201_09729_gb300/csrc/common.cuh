@@ -27,6 +27,9 @@ template <class R> __host__ __device__ __forceinline__ Cx<R> operator*(R s, Cx<R
 template <class R> __host__ __device__ __forceinline__ Cx<R> conj(Cx<R> a) { return cx<R>(a.re, -a.im); }
 // i * a
 template <class R> __host__ __device__ __forceinline__ Cx<R> mul_i(Cx<R> a) { return cx<R>(-a.im, a.re); }
+// a + i b, a - i b
+template <class R> __host__ __device__ __forceinline__ Cx<R> add_i(Cx<R> a, Cx<R> b) { return cx<R>(a.re - b.im, a.im + b.re); }
+template <class R> __host__ __device__ __forceinline__ Cx<R> sub_i(Cx<R> a, Cx<R> b) { return cx<R>(a.re + b.im, a.im - b.re); }
 // a += b * c
 template <class R> __host__ __device__ __forceinline__ void fma_acc(Cx<R>& a, Cx<R> b, Cx<R> c) {
   a.re = fma(b.re, c.re, a.re); a.re = fma(-b.im, c.im, a.re);
@@ -38,6 +41,40 @@ template <class R> __host__ __device__ __forceinline__ void fma_conj_acc(Cx<R>& 
   a.im = fma(b.re, c.im, a.im); a.im = fma(-b.im, c.re, a.im);
 }
 template <class R> __host__ __device__ __forceinline__ R norm2(Cx<R> a) { return a.re * a.re + a.im * a.im; }
+
+// Two FP32 values in one 64-bit register pair: the same component of two right-hand
+// sides, processed by one packed instruction.
+struct __align__(8) f2 {
+  float x, y;
+  f2() = default;
+  __host__ __device__ __forceinline__ constexpr f2(float a, float b) : x(a), y(b) {}
+  __host__ __device__ __forceinline__ constexpr explicit f2(float a) : x(a), y(a) {}
+  __host__ __device__ __forceinline__ constexpr explicit f2(double a) : x((float)a), y((float)a) {}
+  __host__ __device__ __forceinline__ constexpr explicit f2(int a) : x((float)a), y((float)a) {}
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ float2 f2_raw(f2 a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ f2 f2_of(float2 a) { return f2(a.x, a.y); }
+__device__ __forceinline__ f2 fma(f2 a, f2 b, f2 c) { return f2_of(__ffma2_rn(f2_raw(a), f2_raw(b), f2_raw(c))); }
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2_of(__fadd2_rn(f2_raw(a), f2_raw(b))); }
+__device__ __forceinline__ f2 operator*(f2 a, f2 b) { return f2_of(__fmul2_rn(f2_raw(a), f2_raw(b))); }
+__device__ __forceinline__ f2 operator-(f2 a, f2 b) { return fma(b, f2(-1.f), a); }
+__device__ __forceinline__ f2 operator-(f2 a) { return a * f2(-1.f); }
+__device__ __forceinline__ f2 operator*(float a, f2 b) { return f2(a) * b; }
+// a += b * c and a += conj(b) * c for a scalar b shared by the pair
+__device__ __forceinline__ void fma_acc(Cx<f2>& a, Cx<float> b, Cx<f2> c) {
+  a.re = fma(f2(b.re), c.re, a.re); a.re = fma(f2(-b.im), c.im, a.re);
+  a.im = fma(f2(b.re), c.im, a.im); a.im = fma(f2(b.im), c.re, a.im);
+}
+__device__ __forceinline__ void fma_conj_acc(Cx<f2>& a, Cx<float> b, Cx<f2> c) {
+  a.re = fma(f2(b.re), c.re, a.re); a.re = fma(f2(b.im), c.im, a.re);
+  a.im = fma(f2(b.re), c.im, a.im); a.im = fma(f2(-b.im), c.re, a.im);
+}
+__device__ __forceinline__ Cx<f2> operator*(float s, Cx<f2> a) { return cx<f2>(f2(s) * a.re, f2(s) * a.im); }
+__device__ __forceinline__ Cx<f2> operator*(Cx<float> b, Cx<f2> c) {
+  return cx<f2>(fma(f2(-b.im), c.im, f2(b.re) * c.re), fma(f2(b.im), c.re, f2(b.re) * c.im));
+}
+#endif
 
 // ---------------------------------------------------------------------------
 // lattice geometry: even-odd compressed index <-> coordinates.
@@ -96,10 +133,11 @@ struct dlma_ctx {
   double timing[kTimingSlots] = {0};
   cudaEvent_t ev[2] = {nullptr, nullptr};   // timing events of the operator calls
   // stencil block shape (sites x right-hand sides) per precision, chosen by autotune_hop
-  int hop_sx[3] = {64, 64, 64}, hop_sy[3] = {4, 4, 4}, hop_tuned[3] = {0, 0, 0};
-  int hop_l18[3] = {0, 0, 0};   // FP32: read 18-real links instead of rebuilding row 2
-  int hop_chunk[3] = {64, 64, 64};   // right-hand sides per chunk of the stencil's block order
-  int hop_nr[3] = {1, 1, 1};    // FP32: right-hand sides per thread (1 or 2)
+  // (the fourth entry: FP32 in pairs of right-hand sides, kFP32x2)
+  int hop_sx[4] = {64, 64, 64, 64}, hop_sy[4] = {4, 4, 4, 4}, hop_tuned[4] = {0, 0, 0, 0};
+  int hop_l18[4] = {0, 0, 0, 0};   // FP32: read 18-real links instead of rebuilding row 2
+  int hop_chunk[4] = {64, 64, 64, 64};   // right-hand sides per chunk of the stencil's block order
+  int hop_nr[4] = {1, 1, 1, 1};    // FP32: right-hand sides per thread (1 or 2)
   // the Laplacian eigensolver's FP64 phase computes its Gram matrices and rotations
   // in double-float (dfloat.cuh) for tol >= 1e-11; DLMA_DF_EIGS=0 at context
   // creation keeps FP64 arithmetic
@@ -169,7 +207,7 @@ enum WorkSlot {
   WS_SCAL, WS_PART, WS_ACT, WS_ITERS,
   WS_EIG_X, WS_EIG_Y, WS_EIG_Y2, WS_EIG_W, WS_EIG_G, WS_EIG_PART, WS_EIG_S, WS_EIG_AUX,
   WS_PROJ_V, WS_PROJ_PART, WS_PROJ_C, WS_CON, WS_CON2, WS_SRC, WS_SOL, WS_ETA,
-  WS_BI_S, WS_BI_R0, WS_BI_PART, WS_BI_SCAL, WS_RETRY_B, WS_RETRY_X,
+  WS_BI_S, WS_BI_R0, WS_BI_W0, WS_BI_PART, WS_BI_SCAL, WS_RETRY_B, WS_RETRY_X,
   WS_TC_A, WS_TC_B, WS_TC_E, WS_TC_P, WS_SUPPORT,
   WS_COUNT
 };
@@ -216,6 +254,8 @@ template <class T> dlma_status workT(dlma_ctx* ctx, int slot, size_t count, T** 
 //   FP64  double2 [12][Vh]
 //   FP32  float4  [6][Vh]      (complex components 2q, 2q+1 in one float4)
 //   FP16S uint4   [3][Vh]      (complex components 4q..4q+3) + float scale [Vh]
+// and per pair of right-hand sides (2 j, 2 j + 1; an odd last one has an empty partner)
+//   kFP32x2 float4 [12][Vh]    (re, re', im, im' of one component)
 // A FP64 field may also stand for a caller's canonical array (lay), which only the
 // stencil's split form reads and writes in place: half = one parity, complex
 // [V/2][4][3] per right-hand side; full = the sites of one parity inside [V][4][3].
@@ -229,12 +269,19 @@ struct Field {
   int lay = kLayInternal;
 };
 
+constexpr int kFP32x2 = 3;
+// vectors of a field: pairs for kFP32x2, right-hand sides otherwise
+__host__ __device__ inline int field_vectors(int prec, int nrhs) { return prec == kFP32x2 ? (nrhs + 1) / 2 : nrhs; }
+// 16-byte units and bytes per vector
 __host__ __device__ inline size_t field_units_per_rhs(int prec, int Vh) {
-  return prec == DLMA_FP64 ? (size_t)12 * Vh : prec == DLMA_FP32 ? (size_t)6 * Vh : (size_t)3 * Vh;
+  return prec == DLMA_FP64 || prec == kFP32x2 ? (size_t)12 * Vh : prec == DLMA_FP32 ? (size_t)6 * Vh : (size_t)3 * Vh;
 }
 inline size_t field_bytes_per_rhs(int prec, int Vh) {
-  return prec == DLMA_FP64 ? (size_t)12 * Vh * 16 : prec == DLMA_FP32 ? (size_t)6 * Vh * 16
+  return prec == DLMA_FP64 || prec == kFP32x2 ? (size_t)12 * Vh * 16 : prec == DLMA_FP32 ? (size_t)6 * Vh * 16
                                                                       : (size_t)3 * Vh * 16 + (size_t)Vh * 4;
+}
+inline size_t field_bytes(int prec, int Vh, int nrhs) {
+  return field_bytes_per_rhs(prec, Vh) * (size_t)field_vectors(prec, nrhs);
 }
 dlma_status field_alloc(dlma_ctx* ctx, int slot, int prec, int nrhs, Field* f);
 
@@ -266,9 +313,17 @@ struct HopOp {
   const void* cg_p = nullptr;
   const double* cg_alpha = nullptr;
   // DOT epilogue (Schur step B, no gamma_5 on the hop): per (rhs, site tile)
-  // partial of sum conj(w) out into dot_part; w is a field in the output precision
-  const struct Field* dot_w = nullptr;
+  // partial of sum conj(own) out into dot_part
   double2* dot_part = nullptr;
+  // BIS epilogue (Schur step B): s = r - alpha out per right-hand side, stored besides
+  // out, with the partials of sum conj(w0) s (dot_part) and sum conj(r0) s (dot_part2);
+  // w0 and r0 are one FP32 vector each, shared by the right-hand sides
+  const void* bis_r = nullptr;
+  void* bis_s = nullptr;
+  const void* bis_w0 = nullptr;
+  const void* bis_r0 = nullptr;
+  const double2* bis_alpha = nullptr;
+  double2* dot_part2 = nullptr;
   // output sites: the compressed indices site0 .. site0 + nsites - 1 (cyclic modulo
   // V/2; nsites < 0: all).  Whole timeslices are contiguous ranges, so a source
   // supported on few timeslices needs few sites; no partial sums with a range.
@@ -291,10 +346,9 @@ inline bool hop_split(const dlma_ctx* ctx, int prec, int nrhs) {
 dlma_status schur_apply(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, int dagger,
                         const int* active, double* norm_part);
 dlma_status autotune_hop(dlma_ctx* ctx, int prec, const Field& in, Field& tmp, Field& out);
-// out = Dhat in with the partials of sum conj(w) out (dot_part, double2) and, if
-// norm_part is set, |out|^2 per (rhs, site tile)
-dlma_status schur_apply_dot(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, const int* active,
-                            const Field& w, double2* dot_part, double* norm_part);
+// out = Dhat in with the epilogue that `epi` asks for (its dot_part / norm_part / bis_* members)
+dlma_status schur_apply_epi(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, const int* active,
+                            const HopOp& epi);
 // z = Dhat^dag q fused with the CG update x += alpha p, r -= alpha z (x, r, p in the
 // vector precision); partial |r|^2 per (rhs, site tile) into part
 dlma_status schur_dag_cgupdate(dlma_ctx* ctx, const Field& q, Field& tmp, const int* active, Field& x, Field& r,

@@ -46,7 +46,7 @@ dlma_status work(dlma_ctx* ctx, int slot, size_t bytes, void** out) {
 dlma_status field_alloc(dlma_ctx* ctx, int slot, int prec, int nrhs, Field* f) {
   size_t per = field_bytes_per_rhs(prec, ctx->g.Vh);
   void* p;
-  TRY(work(ctx, slot, per * nrhs + 256, &p));
+  TRY(work(ctx, slot, per * field_vectors(prec, nrhs) + 256, &p));
   f->data = p;
   f->prec = prec;
   f->nrhs = nrhs;

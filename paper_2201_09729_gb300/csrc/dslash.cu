@@ -19,10 +19,10 @@
 // link U_mu(x) for x of parity p at compressed index i
 template <int P>
 __device__ __forceinline__ void load_link(const void* __restrict__ Ua, const void* __restrict__ Ub, int p, int mu,
-                                          int i, int Vh, Cx<typename PT<P>::R> U[3][3], bool l18) {
-  typedef typename PT<P>::R R;
+                                          int i, int Vh, Cx<typename PT<P>::S> U[3][3], bool l18) {
+  typedef typename PT<P>::S R;
   size_t base = (size_t)(p * 4 + mu);
-  if (P == DLMA_FP32 && l18) {   // all 18 reals stored: no reconstruction
+  if ((P == DLMA_FP32 || P == kFP32x2) && l18) {   // all 18 reals stored: no reconstruction
     const float4* u = (const float4*)Ua;
 #pragma unroll
     for (int q = 0; q < 5; q++) {
@@ -41,7 +41,7 @@ __device__ __forceinline__ void load_link(const void* __restrict__ Ua, const voi
     }
     return;
   }
-  if (P == DLMA_FP32) {
+  if (P == DLMA_FP32 || P == kFP32x2) {
     const float4* u = (const float4*)Ua;
 #pragma unroll
     for (int q = 0; q < 3; q++) {
@@ -68,8 +68,8 @@ __device__ __forceinline__ void load_link(const void* __restrict__ Ua, const voi
 // one chirality block (36 packed reals) of a clover-type field at parity-offset base
 template <int P>
 __device__ __forceinline__ void load_clover_block(const void* __restrict__ C, int i, int Vh, int ch,
-                                                  typename PT<P>::R a[36]) {
-  typedef typename PT<P>::R R;
+                                                  typename PT<P>::S a[36]) {
+  typedef typename PT<P>::S R;
   if (P == DLMA_FP64) {
     const double2* c = (const double2*)C;
 #pragma unroll
@@ -78,7 +78,7 @@ __device__ __forceinline__ void load_clover_block(const void* __restrict__ C, in
       a[2 * q] = (R)v.x;
       a[2 * q + 1] = (R)v.y;
     }
-  } else if (P == DLMA_FP32) {
+  } else if (P == DLMA_FP32 || P == kFP32x2) {
     const float4* c = (const float4*)C;
 #pragma unroll
     for (int q = 0; q < 9; q++) {
@@ -113,12 +113,12 @@ __device__ __forceinline__ void load_clover_block(const void* __restrict__ C, in
 // (their register cap: 85 registers at 3, 128 at 2).
 // Right-hand sides per chunk of the block order (see k_hop): chosen per precision
 // by the autotuner among {16, 32, 64, 128} (ctx->hop_chunk).
-constexpr int hop_minb(int P, int NR) { return P == DLMA_FP64 ? 2 : (NR > 1 ? 2 : 3); }
+constexpr int hop_minb(int P, int NR) { return P == DLMA_FP64 || P == kFP32x2 ? 2 : (NR > 1 ? 2 : 3); }
 
 // ---------------------------------------------------------------------------
 struct HopArgs {
   Geom g;
-  int bc_t, p_out, nrhs;
+  int bc_t, p_out, nrhs, nvec;         // nvec: vectors (pairs for kFP32x2)
   const void* in; const float* in_scale; size_t in_stride;
   const void* own; const float* own_scale; size_t own_stride;
   void* out; float* out_scale; size_t out_stride;
@@ -136,12 +136,15 @@ struct HopArgs {
   // block order (1D grid): chunks of right-hand-side groups (slowest), site tiles,
   // groups within the chunk (fastest)
   int ntiles, ngroups, gpc;
-  // DOT epilogue: per (rhs, tile) partial of sum conj(w) out (complex) next to |out|^2
-  const void* dot_w; const float* dot_w_scale; double2* dot_part;
+  // DOT epilogue: per (rhs, tile) partial of sum conj(own) out (complex) next to |out|^2
+  double2* dot_part;
+  // BIS epilogue: see HopOp
+  const void* bis_r; void* bis_s; const void* bis_w0; const void* bis_r0; const double2* bis_alpha;
+  double2* dot_part2;
 };
 
-template <class R>
-__device__ __forceinline__ void su3_mul(const Cx<R> U[3][3], const Cx<R> h[3], Cx<R> w[3]) {
+template <class S, class R>
+__device__ __forceinline__ void su3_mul(const Cx<S> U[3][3], const Cx<R> h[3], Cx<R> w[3]) {
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     Cx<R> s = U[a][0] * h[0];
@@ -150,11 +153,11 @@ __device__ __forceinline__ void su3_mul(const Cx<R> U[3][3], const Cx<R> h[3], C
     w[a] = s;
   }
 }
-template <class R>
-__device__ __forceinline__ void su3_dag_mul(const Cx<R> U[3][3], const Cx<R> h[3], Cx<R> w[3]) {
+template <class S, class R>
+__device__ __forceinline__ void su3_dag_mul(const Cx<S> U[3][3], const Cx<R> h[3], Cx<R> w[3]) {
 #pragma unroll
   for (int a = 0; a < 3; a++) {
-    Cx<R> s = cx<R>(0, 0);
+    Cx<R> s = cx<R>((R)0, (R)0);
     fma_conj_acc(s, U[0][a], h[0]);
     fma_conj_acc(s, U[1][a], h[1]);
     fma_conj_acc(s, U[2][a], h[2]);
@@ -167,14 +170,21 @@ template <int P>
 __device__ __forceinline__ void load_chiral(const void* __restrict__ base, const float* __restrict__ scale, int Vh,
                                             int i, int ch, Cx<typename PT<P>::R> v[6]) {
   typedef typename PT<P>::R R;
-  if (P == DLMA_FP64) {
+  if constexpr (P == kFP32x2) {
+    const float4* b = (const float4*)base;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+      const float4 e = __ldg(b + (size_t)(6 * ch + k) * Vh + i);
+      v[k] = cx<R>(f2(e.x, e.y), f2(e.z, e.w));
+    }
+  } else if constexpr (P == DLMA_FP64) {
     const double2* b = (const double2*)base;
 #pragma unroll
     for (int k = 0; k < 6; k++) {
       const double2 e = __ldg(b + (size_t)(6 * ch + k) * Vh + i);
       v[k] = cx<R>((R)e.x, (R)e.y);
     }
-  } else if (P == DLMA_FP32) {
+  } else if constexpr (P == DLMA_FP32) {
     const float4* b = (const float4*)base;
 #pragma unroll
     for (int q = 0; q < 3; q++) {
@@ -191,8 +201,8 @@ __device__ __forceinline__ void load_chiral(const void* __restrict__ base, const
 
 // out = A in for one 6 x 6 hermitian chirality block (36 packed reals: diagonal, then
 // the strictly lower triangle row by row)
-template <class R>
-__device__ __forceinline__ void clover_block_mul(const R a[36], const Cx<R> in[6], Cx<R> out[6]) {
+template <class S, class R>
+__device__ __forceinline__ void clover_block_mul(const S a[36], const Cx<R> in[6], Cx<R> out[6]) {
 #pragma unroll
   for (int r = 0; r < 6; r++) out[r] = a[r] * in[r];
   int k = 6;
@@ -200,7 +210,7 @@ __device__ __forceinline__ void clover_block_mul(const R a[36], const Cx<R> in[6
   for (int r = 1; r < 6; r++)
 #pragma unroll
     for (int c = 0; c < r; c++) {
-      const Cx<R> l = cx<R>(a[k], a[k + 1]);
+      const Cx<S> l = cx<S>(a[k], a[k + 1]);
       k += 2;
       fma_acc(out[r], l, in[c]);
       fma_conj_acc(out[c], l, in[r]);
@@ -251,9 +261,11 @@ __device__ __forceinline__ R cg_update(void* __restrict__ x, void* __restrict__ 
 }
 
 template <int P, int NR, bool G5IN, bool G5HOP, int OWN, bool KOUT, bool HOP, bool NORM, bool L18, bool CGU = false,
-          bool DOT = false>
+          bool DOT = false, bool BIS = false>
 __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
   typedef typename PT<P>::R R;
+  typedef typename PT<P>::S S;
+  constexpr int LN = PT<P>::lanes;   // right-hand sides per vector j
   // Block order: the right-hand sides of a chunk (gpc groups, about 32 rhs) run back
   // to back on a site tile, so its links and clover come from DRAM once per chunk
   // and from L2 otherwise; the chunk sweeps all tiles before the next chunk starts,
@@ -274,7 +286,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
   for (int q = NR - 1; q >= 0; q--) {
     jq[q] = j0 + q;
-    vq[q] = il < a.nsites && jq[q] < a.nrhs && (!a.active || a.active[jq[q]] != 0);
+    vq[q] = il < a.nsites && jq[q] < a.nvec && vec_on<P>(jq[q], a.nrhs, a.active);
     if (vq[q]) { valid = true; jany = jq[q]; }
   }
   // loads of an idle slot read a live right-hand side of this thread (always in bounds)
@@ -282,9 +294,10 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
   for (int q = 0; q < NR; q++) jl[q] = vq[q] ? jq[q] : jany;
   R nrm[NR];   // |out|^2 per thread in the stencil precision; block partials in FP64
-  R dre[NR], dim[NR];   // DOT: sum conj(w) out
+  R dre[NR], dim[NR];   // DOT: sum conj(own) out; BIS: sum conj(w0) s
+  R ere[NR], eim[NR];   // BIS: sum conj(r0) s
 #pragma unroll
-  for (int q = 0; q < NR; q++) nrm[q] = dre[q] = dim[q] = 0;
+  for (int q = 0; q < NR; q++) nrm[q] = dre[q] = dim[q] = ere[q] = eim[q] = (R)0;
   if (valid) {
     Spinor<R> res[NR];
 #pragma unroll
@@ -292,7 +305,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
       for (int s = 0; s < 4; s++)
 #pragma unroll
-        for (int c = 0; c < 3; c++) res[q].c[s][c] = cx<R>(0, 0);
+        for (int c = 0; c < 3; c++) res[q].c[s][c] = cx<R>((R)0, (R)0);
     if (HOP) {
       const int4 q0 = __ldg(a.nbr + ((size_t)a.p_out * 2 + 0) * g.Vh + i);
       const int4 q1 = __ldg(a.nbr + ((size_t)a.p_out * 2 + 1) * g.Vh + i);
@@ -303,10 +316,10 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
         for (int dir = 0; dir < 2; dir++) {
           const int raw = nb8[2 * mu + dir];
           const int n = mu == 0 ? (raw & 0x7fffffff) : raw;   // only time neighbours carry the phase bit
-          Cx<R> U[3][3];
+          Cx<S> U[3][3];
           // forward: U_mu(x) at this site; backward: U_mu(x - mu) at the neighbour
           load_link<P>(a.Ua, a.Ub, dir == 0 ? a.p_out : 1 - a.p_out, mu, dir == 0 ? i : n, g.Vh, U, L18);
-          const R ph = raw < 0 ? (R)-1 : (R)1;    // antiperiodic time phase (bit 31, mu = 0 only)
+          const S ph = raw < 0 ? (S)-1 : (S)1;    // antiperiodic time phase (bit 31, mu = 0 only)
 #pragma unroll
           for (int q = 0; q < NR; q++) {
             Spinor<R> ps = load_spinor<P>((const char*)a.in + (size_t)jl[q] * a.in_stride,
@@ -321,14 +334,14 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
               const Cx<R> u0 = ps.c[0][c], u1 = ps.c[1][c], d0 = ps.c[2][c], d1 = ps.c[3][c];
               if (dir == 0) {           // (1 - g_mu)
                 if (mu == 0) { h0[c] = u0 + d0; h1[c] = u1 + d1; }
-                else if (mu == 1) { h0[c] = u0 + mul_i(d1); h1[c] = u1 + mul_i(d0); }
+                else if (mu == 1) { h0[c] = add_i(u0, d1); h1[c] = add_i(u1, d0); }
                 else if (mu == 2) { h0[c] = u0 + d1; h1[c] = u1 - d0; }
-                else { h0[c] = u0 + mul_i(d0); h1[c] = u1 - mul_i(d1); }
+                else { h0[c] = add_i(u0, d0); h1[c] = sub_i(u1, d1); }
               } else {                  // (1 + g_mu)
                 if (mu == 0) { h0[c] = u0 - d0; h1[c] = u1 - d1; }
-                else if (mu == 1) { h0[c] = u0 - mul_i(d1); h1[c] = u1 - mul_i(d0); }
+                else if (mu == 1) { h0[c] = sub_i(u0, d1); h1[c] = sub_i(u1, d0); }
                 else if (mu == 2) { h0[c] = u0 - d1; h1[c] = u1 + d0; }
-                else { h0[c] = u0 - mul_i(d0); h1[c] = u1 + mul_i(d1); }
+                else { h0[c] = sub_i(u0, d0); h1[c] = add_i(u1, d1); }
               }
             }
             if (dir == 0) { su3_mul(U, h0, w0); su3_mul(U, h1, w1); }
@@ -341,27 +354,27 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
               rq.c[1][c] = rq.c[1][c] + x1;
               if (dir == 0) {
                 if (mu == 0) { rq.c[2][c] = rq.c[2][c] + x0; rq.c[3][c] = rq.c[3][c] + x1; }
-                else if (mu == 1) { rq.c[2][c] = rq.c[2][c] - mul_i(x1); rq.c[3][c] = rq.c[3][c] - mul_i(x0); }
+                else if (mu == 1) { rq.c[2][c] = sub_i(rq.c[2][c], x1); rq.c[3][c] = sub_i(rq.c[3][c], x0); }
                 else if (mu == 2) { rq.c[2][c] = rq.c[2][c] - x1; rq.c[3][c] = rq.c[3][c] + x0; }
-                else { rq.c[2][c] = rq.c[2][c] - mul_i(x0); rq.c[3][c] = rq.c[3][c] + mul_i(x1); }
+                else { rq.c[2][c] = sub_i(rq.c[2][c], x0); rq.c[3][c] = add_i(rq.c[3][c], x1); }
               } else {
                 if (mu == 0) { rq.c[2][c] = rq.c[2][c] - x0; rq.c[3][c] = rq.c[3][c] - x1; }
-                else if (mu == 1) { rq.c[2][c] = rq.c[2][c] + mul_i(x1); rq.c[3][c] = rq.c[3][c] + mul_i(x0); }
+                else if (mu == 1) { rq.c[2][c] = add_i(rq.c[2][c], x1); rq.c[3][c] = add_i(rq.c[3][c], x0); }
                 else if (mu == 2) { rq.c[2][c] = rq.c[2][c] + x1; rq.c[3][c] = rq.c[3][c] - x0; }
-                else { rq.c[2][c] = rq.c[2][c] + mul_i(x0); rq.c[3][c] = rq.c[3][c] - mul_i(x1); }
+                else { rq.c[2][c] = add_i(rq.c[2][c], x0); rq.c[3][c] = sub_i(rq.c[3][c], x1); }
               }
             }
           }
         }
       }
-      const R f = (R)(-0.5 * a.s);
+      const S f = (S)(-0.5 * a.s);
 #pragma unroll
       for (int q = 0; q < NR; q++)
 #pragma unroll
         for (int s = 0; s < 4; s++)
 #pragma unroll
           for (int c = 0; c < 3; c++) {
-            const R ff = (G5HOP && s >= 2) ? -f : f;
+            const S ff = (G5HOP && s >= 2) ? -f : f;
             res[q].c[s][c] = ff * res[q].c[s][c];
           }
     }
@@ -371,7 +384,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
       for (int ch = 0; ch < 2; ch++) {
         if (OWN) {
-          R k[36];
+          S k[36];
           if (OWN == 2) load_clover_block<P>(a.Kown, i, g.Vh, ch, k);
 #pragma unroll
           for (int q = 0; q < NR; q++) {
@@ -383,11 +396,15 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
             for (int r = 0; r < 6; r++) {
               Cx<R>& e = res[q].c[2 * ch + r / 3][r % 3];
               e = e + (OWN == 2 ? t[r] : o[r]);
+              if (DOT) {           // the result is complete here (no outer factor)
+                dre[q] = fma(o[r].re, e.re, fma(o[r].im, e.im, dre[q]));
+                dim[q] = fma(o[r].re, e.im, fma(-o[r].im, e.re, dim[q]));
+              }
             }
           }
         }
         if (KOUT) {
-          R k[36];
+          S k[36];
           load_clover_block<P>(a.Kout, i, g.Vh, ch, k);
 #pragma unroll
           for (int q = 0; q < NR; q++) {
@@ -405,7 +422,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
     for (int q = 0; q < NR; q++) {
       if (!vq[q]) continue;
       const int j = jq[q];
-      if (CGU) {
+      if constexpr (CGU) {
         // fused CG update: z (= res) is consumed here and never stored
         constexpr int PB = P == DLMA_FP64 ? DLMA_FP64 : DLMA_FP32;
         const size_t sb = (size_t)j * a.cg_stride;
@@ -418,60 +435,77 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
           for (int s = 0; s < 4; s++)
 #pragma unroll
-            for (int c = 0; c < 3; c++) nrm[q] += norm2(res[q].c[s][c]);
+            for (int c = 0; c < 3; c++) nrm[q] = nrm[q] + norm2(res[q].c[s][c]);
         }
-        if (DOT) {
-          const Spinor<R> w = load_spinor<P>((const char*)a.dot_w + (size_t)j * a.out_stride,
-                                             a.dot_w_scale ? a.dot_w_scale + (size_t)j * g.Vh : nullptr, g.Vh, i);
+        if constexpr (BIS) {
+          const size_t o = (size_t)j * a.out_stride;
+          const double2 a0 = a.bis_alpha[lane_rhs<P>(j, 0, a.nrhs)], a1 = a.bis_alpha[lane_rhs<P>(j, LN - 1, a.nrhs)];
+          const R ar = lane_pack<P>(a0.x, a1.x), ai = lane_pack<P>(a0.y, a1.y);
 #pragma unroll
-          for (int s = 0; s < 4; s++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-              const Cx<R> wv = w.c[s][c], ov = res[q].c[s][c];
-              dre[q] = fma(wv.re, ov.re, fma(wv.im, ov.im, dre[q]));
-              dim[q] = fma(wv.re, ov.im, fma(-wv.im, ov.re, dim[q]));
-            }
+          for (int k = 0; k < 12; k++) {
+            // w0, r0: one vector for all right-hand sides
+            const Cx<S> w = load_comp<DLMA_FP32>(a.bis_w0, g.Vh, i, k), z = load_comp<DLMA_FP32>(a.bis_r0, g.Vh, i, k);
+            const Cx<R> v = res[q].c[k / 3][k % 3];
+            Cx<R> e = load_comp<P>((const char*)a.bis_r + o, g.Vh, i, k);
+            e.re = fma(-ar, v.re, fma(ai, v.im, e.re));
+            e.im = fma(-ar, v.im, fma(-ai, v.re, e.im));
+            store_comp<P>((char*)a.bis_s + o, g.Vh, i, k, e);
+            dre[q] = fma((R)w.re, e.re, fma((R)w.im, e.im, dre[q]));
+            dim[q] = fma((R)w.re, e.im, fma((R)-w.im, e.re, dim[q]));
+            ere[q] = fma((R)z.re, e.re, fma((R)z.im, e.im, ere[q]));
+            eim[q] = fma((R)z.re, e.im, fma((R)-z.im, e.re, eim[q]));
+          }
         }
       }
     }
   }
-  if (NORM || DOT) {
-    // per (rhs, block) partial sums: the warps of one threadIdx.y row share NR rhs
-    __shared__ double red[3][32 * NR];
+  if constexpr (NORM || DOT || BIS) {
+    // per (rhs, block) partial sums: the warps of one threadIdx.y row share NR vectors
+    constexpr int NV = (NORM ? 1 : 0) + (DOT || BIS ? 2 : 0) + (BIS ? 2 : 0);
+    __shared__ double red[NV][32 * NR * LN];
     const int wx = threadIdx.x >> 5, nwx = blockDim.x >> 5;
 #pragma unroll
-    for (int q = 0; q < NR; q++) {
-      R v = nrm[q], vr = dre[q], vi = dim[q];
+    for (int q = 0; q < NR; q++)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        if (NORM) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (DOT) {
-          vr += __shfl_down_sync(0xffffffffu, vr, o);
-          vi += __shfl_down_sync(0xffffffffu, vi, o);
+      for (int l = 0; l < LN; l++) {
+        typedef decltype(lane_get(R(), 0)) F;
+        F v[NV];
+        int n = 0;
+        if (NORM) v[n++] = lane_get(nrm[q], l);
+        if (DOT || BIS) { v[n++] = lane_get(dre[q], l); v[n++] = lane_get(dim[q], l); }
+        if (BIS) { v[n++] = lane_get(ere[q], l); v[n++] = lane_get(eim[q], l); }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int e = 0; e < NV; e++) v[e] += __shfl_down_sync(0xffffffffu, v[e], o);
+        if ((threadIdx.x & 31) == 0) {
+          const int slot = ((threadIdx.y * nwx + wx) * NR + q) * LN + l;
+#pragma unroll
+          for (int e = 0; e < NV; e++) red[e][slot] = (double)v[e];
         }
       }
-      if ((threadIdx.x & 31) == 0) {
-        const int slot = (threadIdx.y * nwx + wx) * NR + q;
-        red[0][slot] = (double)v;
-        red[1][slot] = (double)vr;
-        red[2][slot] = (double)vi;
-      }
-    }
     __syncthreads();
     if (threadIdx.x == 0) {
 #pragma unroll
-      for (int q = 0; q < NR; q++) {
-        if (jq[q] >= a.nrhs) continue;
-        double t = 0, tr = 0, ti = 0;
-        for (int w = 0; w < nwx; w++) {
-          const int slot = (threadIdx.y * nwx + w) * NR + q;
-          t += red[0][slot];
-          tr += red[1][slot];
-          ti += red[2][slot];
+      for (int q = 0; q < NR; q++)
+#pragma unroll
+        for (int l = 0; l < LN; l++) {
+          const int r = jq[q] * LN + l;
+          if (r >= a.nrhs) continue;
+          double t[NV];
+#pragma unroll
+          for (int e = 0; e < NV; e++) t[e] = 0;
+          for (int w = 0; w < nwx; w++) {
+            const int slot = ((threadIdx.y * nwx + w) * NR + q) * LN + l;
+#pragma unroll
+            for (int e = 0; e < NV; e++) t[e] += red[e][slot];
+          }
+          const size_t o = (size_t)r * a.ntiles + tile;
+          int n = 0;
+          if (NORM) a.norm_part[o] = t[n++];
+          if (DOT || BIS) { a.dot_part[o] = make_double2(t[n], t[n + 1]); n += 2; }
+          if (BIS) a.dot_part2[o] = make_double2(t[n], t[n + 1]);
         }
-        if (NORM) a.norm_part[(size_t)jq[q] * a.ntiles + tile] = t;
-        if (DOT) a.dot_part[(size_t)jq[q] * a.ntiles + tile] = make_double2(tr, ti);
-      }
     }
   }
 }
@@ -580,6 +614,7 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   a.bc_t = ctx->bc_t;
   a.p_out = op.p_out;
   a.nrhs = out.nrhs;
+  a.nvec = field_vectors(P, out.nrhs);
   a.in = in.data;
   a.in_scale = in.scale;
   a.in_stride = field_units_per_rhs(P, ctx->g.Vh) * 16;
@@ -599,9 +634,13 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   a.cg_p = op.cg_p;
   a.cg_alpha = op.cg_alpha;
   a.cg_stride = field_units_per_rhs(P == DLMA_FP64 ? DLMA_FP64 : DLMA_FP32, ctx->g.Vh) * 16;
-  a.dot_w = op.dot_w ? op.dot_w->data : nullptr;
-  a.dot_w_scale = op.dot_w ? op.dot_w->scale : nullptr;
   a.dot_part = op.dot_part;
+  a.bis_r = op.bis_r;
+  a.bis_s = op.bis_s;
+  a.bis_w0 = op.bis_w0;
+  a.bis_r0 = op.bis_r0;
+  a.bis_alpha = op.bis_alpha;
+  a.dot_part2 = op.dot_part2;
   const size_t Vh = ctx->g.Vh;
   const int p = op.p_out;
   const void* Kown = nullptr;
@@ -610,7 +649,7 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
     a.Ua = ctx->U64; a.Ub = nullptr;
     Kown = op.own == 3 ? (const void*)(ctx->Ci64 + p * 36 * Vh) : (const void*)(ctx->C64 + p * 36 * Vh);
     Kout = op.kout == 2 ? (const void*)(ctx->C64 + p * 36 * Vh) : (const void*)(ctx->Ci64 + p * 36 * Vh);
-  } else if (P == DLMA_FP32) {
+  } else if (P == DLMA_FP32 || P == kFP32x2) {
     a.l18 = ctx->hop_l18[P];
     a.Ua = a.l18 ? (const void*)ctx->U32f : (const void*)ctx->U32;
     a.Ub = nullptr;
@@ -627,14 +666,18 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   hop_block(ctx, P, sx, sy);
   dim3 blk(sx, sy);
   const bool cgu = op.cg_x != nullptr && op.hop;
-  const bool dot = op.dot_part != nullptr && op.hop && op.own == 2 && !op.kout && !op.g5_hop;
-  const int nr = (P == DLMA_FP32 && !cgu) ? ctx->hop_nr[P] : 1;
+  const bool epi = op.dot_part != nullptr && op.hop && op.own == 2 && !op.kout && !op.g5_hop;
+  const bool bis = epi && op.bis_r != nullptr, dot = epi && !bis;
+  if (bis && (op.norm_part || (P != DLMA_FP32 && P != kFP32x2)))
+    return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil epilogue");
+  const int nr = (P == DLMA_FP32 && !cgu && !epi) ? ctx->hop_nr[P] : 1;
   a.site0 = op.nsites >= 0 ? op.site0 : 0;
   a.nsites = op.nsites >= 0 ? op.nsites : ctx->g.Vh;
   if (a.nsites == 0) return DLMA_OK;
   a.ntiles = (a.nsites + sx - 1) / sx;
-  a.ngroups = (out.nrhs + sy * nr - 1) / (sy * nr);
-  a.gpc = std::max(1, std::min(a.ngroups, ctx->hop_chunk[P] / (sy * nr)));
+  const int lanes = P == kFP32x2 ? 2 : 1;
+  a.ngroups = (a.nvec + sy * nr - 1) / (sy * nr);
+  a.gpc = std::max(1, std::min(a.ngroups, ctx->hop_chunk[P] / (sy * nr * lanes)));
   const int nchunks = (a.ngroups + a.gpc - 1) / a.gpc;
   dim3 grid((unsigned)((size_t)nchunks * a.ntiles * a.gpc));
   if (nblocks_out) *nblocks_out = a.ntiles;
@@ -645,16 +688,23 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
 #define LD(PP, NRR, LL) \
   (nrm ? k_hop<PP, NRR, false, false, 2, false, true, true, LL, false, true><<<grid, blk, 0, st>>>(a) \
        : k_hop<PP, NRR, false, false, 2, false, true, false, LL, false, true><<<grid, blk, 0, st>>>(a))
-    if (P == DLMA_FP64) LD(DLMA_FP64, 1, false);
-    else if (P == DLMA_FP32 && nr == 2) { if (a.l18) LD(DLMA_FP32, 2, true); else LD(DLMA_FP32, 2, false); }
-    else if (P == DLMA_FP32) { if (a.l18) LD(DLMA_FP32, 1, true); else LD(DLMA_FP32, 1, false); }
-    else LD(DLMA_FP16S, 1, false);
+    if (P == DLMA_FP32) { if (a.l18) LD(DLMA_FP32, 1, true); else LD(DLMA_FP32, 1, false); }
+    else if (P == kFP32x2) { if (a.l18) LD(kFP32x2, 1, true); else LD(kFP32x2, 1, false); }
+    else return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil epilogue");
 #undef LD
+  } else if (bis) {
+#define LB(PP, LL) k_hop<PP, 1, false, false, 2, false, true, false, LL, false, false, true><<<grid, blk, 0, st>>>(a)
+    if (P == kFP32x2) { if (a.l18) LB(kFP32x2, true); else LB(kFP32x2, false); }
+    else { if (a.l18) LB(DLMA_FP32, true); else LB(DLMA_FP32, false); }
+#undef LB
   } else if (cgu) {
     if (P == DLMA_FP64) dispatch_cgu<DLMA_FP64, false>(grid, blk, st, a);
     else if (P == DLMA_FP32 && a.l18) dispatch_cgu<DLMA_FP32, true>(grid, blk, st, a);
     else if (P == DLMA_FP32) dispatch_cgu<DLMA_FP32, false>(grid, blk, st, a);
     else dispatch_cgu<DLMA_FP16S, false>(grid, blk, st, a);
+  } else if (P == kFP32x2) {
+    if (a.l18) dispatch<kFP32x2, 1, true>(op, grid, blk, st, a);
+    else dispatch<kFP32x2, 1, false>(op, grid, blk, st, a);
   } else if (P == DLMA_FP64) {
     dispatch<DLMA_FP64, 1, false>(op, grid, blk, st, a);
   } else if (P == DLMA_FP32) {
@@ -687,10 +737,11 @@ dlma_status autotune_hop(dlma_ctx* ctx, int prec, const Field& in, Field& tmp, F
   int bx = ctx->hop_sx[prec], by = ctx->hop_sy[prec], bl = 0, bn = 1;
   // FP32: also try 18-real links and two right-hand sides per thread;
   // DLMA_FORCE_LINKS=12 / 18 and DLMA_FORCE_NR=1 / 2 pin the choice (tests)
-  int l0 = 0, l1 = prec == DLMA_FP32 ? 1 : 0;
+  const bool f32 = prec == DLMA_FP32 || prec == kFP32x2;
+  int l0 = 0, l1 = f32 ? 1 : 0;
   int n0 = 1, n1 = prec == DLMA_FP32 ? 2 : 1;
   if (const char* f = getenv("DLMA_FORCE_LINKS")) {
-    if (prec == DLMA_FP32 && atoi(f) == 18) l0 = l1 = 1;
+    if (f32 && atoi(f) == 18) l0 = l1 = 1;
     if (atoi(f) == 12) l0 = l1 = 0;
   }
   if (const char* f = getenv("DLMA_FORCE_NR")) {
@@ -779,23 +830,20 @@ dlma_status schur_dag_cgupdate(dlma_ctx* ctx, const Field& q, Field& tmp, const 
   return DLMA_OK;
 }
 
-dlma_status schur_apply_dot(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, const int* active,
-                            const Field& w, double2* dot_part, double* norm_part) {
+dlma_status schur_apply_epi(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, const int* active,
+                            const HopOp& epi) {
   HopOp A;
   A.p_out = 1;
   A.own = 0;
   A.kout = 3;
   A.active = active;
   TRY(launch_hop(ctx, A, in, nullptr, tmp));
-  HopOp B;
+  HopOp B = epi;
   B.p_out = 0;
   B.own = 2;
   B.kout = 0;
   B.s = -1.0;
   B.active = active;
-  B.norm_part = norm_part;
-  B.dot_w = &w;
-  B.dot_part = dot_part;
   TRY(launch_hop(ctx, B, tmp, &in, out));
   return DLMA_OK;
 }
@@ -823,27 +871,29 @@ dlma_status schur_apply(dlma_ctx* ctx, const Field& in, Field& tmp, Field& out, 
 
 // ---------------------------------------------------------------------------
 // canonical complex128 <-> internal fields
+// vector j of the field <-> its right-hand sides' sites (an empty partner packs as zero)
+__device__ __forceinline__ size_t canonical_site(const Geom& g, int full, int p, int r, int i) {
+  if (!full) return (size_t)r * g.Vh + i;
+  const Coord c = eo_coords(g, p, i);
+  return (size_t)r * g.V + lex_of(g, c.x, c.y, c.z, c.t);
+}
 template <int P>
 __global__ void k_pack(Geom g, const double2* __restrict__ src, int full, int p, int nrhs, void* dst, float* scale) {
   typedef typename PT<P>::R R;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y;
-  if (i >= g.Vh || j >= nrhs) return;
-  size_t site;
-  if (full) {
-    Coord c = eo_coords(g, p, i);
-    site = (size_t)j * g.V + lex_of(g, c.x, c.y, c.z, c.t);
-  } else {
-    site = (size_t)j * g.Vh + i;
-  }
-  const double2* s = src + site * 12;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y;
+  if (i >= g.Vh) return;
+  const double2* s0 = src + canonical_site(g, full, p, lane_rhs<P>(j, 0, nrhs), i) * 12;
+  const bool two = PT<P>::lanes == 2 && 2 * j + 1 < nrhs;
+  const double2* s1 = two ? src + canonical_site(g, full, p, 2 * j + 1, i) * 12 : s0;
   Spinor<R> v;
 #pragma unroll
   for (int k = 0; k < 12; k++) {
-    double2 e = s[k];
-    v.c[k / 3][k % 3] = cx<R>((R)e.x, (R)e.y);
+    const double2 e = s0[k];
+    const double2 f = two ? s1[k] : make_double2(0, 0);
+    v.c[k / 3][k % 3] = cx<R>(lane_pack<P>(e.x, f.x), lane_pack<P>(e.y, f.y));
   }
-  size_t stride = field_units_per_rhs(P, g.Vh) * 16;
+  const size_t stride = field_units_per_rhs(P, g.Vh) * 16;
   store_spinor<P>((char*)dst + j * stride, scale ? scale + (size_t)j * g.Vh : nullptr, g.Vh, i, v);
 }
 
@@ -851,26 +901,26 @@ template <int P>
 __global__ void k_unpack(Geom g, const void* __restrict__ srcf, const float* __restrict__ scale, int full, int p,
                          int nrhs, double2* dst) {
   typedef typename PT<P>::R R;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int j = blockIdx.y;
-  if (i >= g.Vh || j >= nrhs) return;
-  size_t stride = field_units_per_rhs(P, g.Vh) * 16;
-  Spinor<R> v = load_spinor<P>((const char*)srcf + j * stride, scale ? scale + (size_t)j * g.Vh : nullptr, g.Vh, i);
-  size_t site;
-  if (full) {
-    Coord c = eo_coords(g, p, i);
-    site = (size_t)j * g.V + lex_of(g, c.x, c.y, c.z, c.t);
-  } else {
-    site = (size_t)j * g.Vh + i;
-  }
-  double2* d = dst + site * 12;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y;
+  if (i >= g.Vh) return;
+  const size_t stride = field_units_per_rhs(P, g.Vh) * 16;
+  const Spinor<R> v = load_spinor<P>((const char*)srcf + j * stride, scale ? scale + (size_t)j * g.Vh : nullptr, g.Vh, i);
 #pragma unroll
-  for (int k = 0; k < 12; k++) d[k] = make_double2((double)v.c[k / 3][k % 3].re, (double)v.c[k / 3][k % 3].im);
+  for (int l = 0; l < PT<P>::lanes; l++) {
+    const int r = PT<P>::lanes * j + l;
+    if (r >= nrhs) break;
+    double2* d = dst + canonical_site(g, full, p, r, i) * 12;
+#pragma unroll
+    for (int k = 0; k < 12; k++)
+      d[k] = make_double2((double)lane_get(v.c[k / 3][k % 3].re, l), (double)lane_get(v.c[k / 3][k % 3].im, l));
+  }
 }
 
 dlma_status pack_parity(dlma_ctx* ctx, const double* src, int full, int p, Field& f) {
-  dim3 grid((ctx->g.Vh + 127) / 128, f.nrhs);
-  if (f.prec == DLMA_FP64) k_pack<DLMA_FP64><<<grid, 128, 0, ctx->stream>>>(ctx->g, (const double2*)src, full, p, f.nrhs, f.data, f.scale);
+  dim3 grid((ctx->g.Vh + 127) / 128, field_vectors(f.prec, f.nrhs));
+  if (f.prec == kFP32x2) k_pack<kFP32x2><<<grid, 128, 0, ctx->stream>>>(ctx->g, (const double2*)src, full, p, f.nrhs, f.data, f.scale);
+  else if (f.prec == DLMA_FP64) k_pack<DLMA_FP64><<<grid, 128, 0, ctx->stream>>>(ctx->g, (const double2*)src, full, p, f.nrhs, f.data, f.scale);
   else if (f.prec == DLMA_FP32) k_pack<DLMA_FP32><<<grid, 128, 0, ctx->stream>>>(ctx->g, (const double2*)src, full, p, f.nrhs, f.data, f.scale);
   else k_pack<DLMA_FP16S><<<grid, 128, 0, ctx->stream>>>(ctx->g, (const double2*)src, full, p, f.nrhs, f.data, f.scale);
   CHECK_LAUNCH();
@@ -878,8 +928,9 @@ dlma_status pack_parity(dlma_ctx* ctx, const double* src, int full, int p, Field
 }
 
 dlma_status unpack_parity(dlma_ctx* ctx, const Field& f, int full, int p, double* dst) {
-  dim3 grid((ctx->g.Vh + 127) / 128, f.nrhs);
-  if (f.prec == DLMA_FP64) k_unpack<DLMA_FP64><<<grid, 128, 0, ctx->stream>>>(ctx->g, f.data, f.scale, full, p, f.nrhs, (double2*)dst);
+  dim3 grid((ctx->g.Vh + 127) / 128, field_vectors(f.prec, f.nrhs));
+  if (f.prec == kFP32x2) k_unpack<kFP32x2><<<grid, 128, 0, ctx->stream>>>(ctx->g, f.data, f.scale, full, p, f.nrhs, (double2*)dst);
+  else if (f.prec == DLMA_FP64) k_unpack<DLMA_FP64><<<grid, 128, 0, ctx->stream>>>(ctx->g, f.data, f.scale, full, p, f.nrhs, (double2*)dst);
   else if (f.prec == DLMA_FP32) k_unpack<DLMA_FP32><<<grid, 128, 0, ctx->stream>>>(ctx->g, f.data, f.scale, full, p, f.nrhs, (double2*)dst);
   else k_unpack<DLMA_FP16S><<<grid, 128, 0, ctx->stream>>>(ctx->g, f.data, f.scale, full, p, f.nrhs, (double2*)dst);
   CHECK_LAUNCH();
@@ -896,6 +947,8 @@ static dlma_status check_ready(dlma_ctx* ctx) {
   return DLMA_OK;
 }
 
+// the internal form of a batch: FP32 in pairs from two right-hand sides on
+static int field_prec(int prec, int nrhs) { return prec == DLMA_FP32 && nrhs > 1 ? kFP32x2 : prec; }
 // a caller's canonical FP64 array as a field of the split stencil
 static Field canonical(dlma_ctx* ctx, const double* p, int nrhs, int lay) {
   Field f;
@@ -930,13 +983,14 @@ extern "C" dlma_status dlma_apply_Dw(dlma_ctx* ctx, const double* in, double* ou
     CU(cudaStreamSynchronize(ctx->stream));
     return DLMA_OK;
   }
+  const int fp = field_prec(prec, nrhs), nv = field_vectors(fp, nrhs);
   Field fe, fo, re, ro;
-  TRY(field_alloc(ctx, WS_T0, prec, nrhs, &fe));
-  TRY(field_alloc(ctx, WS_T1, prec, nrhs, &fo));
-  TRY(field_alloc(ctx, WS_T2, prec, 2 * nrhs, &re));
+  TRY(field_alloc(ctx, WS_T0, fp, nrhs, &fe));
+  TRY(field_alloc(ctx, WS_T1, fp, nrhs, &fo));
+  TRY(field_alloc(ctx, WS_T2, fp, fp == kFP32x2 ? 4 * nv : 2 * nrhs, &re));
   ro = re;
   ro.nrhs = nrhs;
-  ro.data = (char*)re.data + field_units_per_rhs(prec, ctx->g.Vh) * 16 * nrhs;
+  ro.data = (char*)re.data + field_units_per_rhs(fp, ctx->g.Vh) * 16 * nv;
   if (prec == DLMA_FP16S) ro.scale = re.scale + (size_t)nrhs * ctx->g.Vh;
   re.nrhs = nrhs;
   if (prec == DLMA_FP16S) {
@@ -973,15 +1027,16 @@ extern "C" dlma_status dlma_apply_schur(dlma_ctx* ctx, const double* in, double*
   // few pairs: the split stencil reads and writes the canonical arrays themselves
   const bool direct = hop_split(ctx, prec, nrhs) && disjoint(din, dout, bytes);
   Field fe, tmp, res;
-  TRY(field_alloc(ctx, WS_T1, prec, nrhs, &tmp));
+  const int fp = field_prec(prec, nrhs);
+  TRY(field_alloc(ctx, WS_T1, fp, nrhs, &tmp));
   if (direct) {
     fe = canonical(ctx, din, nrhs, kLayHalf);
     res = canonical(ctx, dout, nrhs, kLayHalf);
   } else {
-    TRY(field_alloc(ctx, WS_T0, prec, nrhs, &fe));
-    TRY(field_alloc(ctx, WS_T2, prec, nrhs, &res));
+    TRY(field_alloc(ctx, WS_T0, fp, nrhs, &fe));
+    TRY(field_alloc(ctx, WS_T2, fp, nrhs, &res));
     TRY(pack_parity(ctx, din, 0, 0, fe));
-    TRY(autotune_hop(ctx, prec, fe, tmp, res));
+    TRY(autotune_hop(ctx, fp, fe, tmp, res));
   }
   for (cudaEvent_t& e : ctx->ev)
     if (!e) CU(cudaEventCreate(&e));

@@ -3,24 +3,56 @@
 #pragma once
 #include "common.cuh"
 
-template <int P> struct PT { typedef float R; };
-template <> struct PT<DLMA_FP64> { typedef double R; };
+// R: vector arithmetic, S: links and clover, lanes: right-hand sides per vector
+template <int P> struct PT { typedef float R; typedef float S; static constexpr int lanes = 1; };
+template <> struct PT<DLMA_FP64> { typedef double R; typedef double S; static constexpr int lanes = 1; };
+template <> struct PT<kFP32x2> { typedef f2 R; typedef float S; static constexpr int lanes = 2; };
 
 template <class R> struct Spinor { Cx<R> c[4][3]; };
+
+// per-rhs values of vector j: one value, or the pair's two (an empty partner reads the first)
+__device__ __forceinline__ float lane_get(f2 v, int q) { return q ? v.y : v.x; }
+__device__ __forceinline__ float lane_get(float v, int) { return v; }
+__device__ __forceinline__ double lane_get(double v, int) { return v; }
+template <int P> __device__ __forceinline__ typename PT<P>::R lane_pack(double a, double b) {
+  if constexpr (P == kFP32x2) return f2((float)a, (float)b);
+  else return (typename PT<P>::R)a;
+}
+// right-hand side of lane q of vector j, and whether it is there and on (mask may be null)
+template <int P> __device__ __forceinline__ int lane_rhs(int j, int q, int nrhs) {
+  const int r = PT<P>::lanes * j + q;
+  return r < nrhs ? r : nrhs - 1;
+}
+template <int P> __device__ __forceinline__ bool lane_on(int j, int q, int nrhs, const int* mask) {
+  const int r = PT<P>::lanes * j + q;
+  return r < nrhs && (!mask || mask[r] != 0);
+}
+template <int P> __device__ __forceinline__ bool vec_on(int j, int nrhs, const int* mask) {
+  bool on = lane_on<P>(j, 0, nrhs, mask);
+  if constexpr (PT<P>::lanes == 2) on = on || lane_on<P>(j, 1, nrhs, mask);
+  return on;
+}
 
 template <int P>
 __device__ __forceinline__ Spinor<typename PT<P>::R> load_spinor(const void* __restrict__ base,
                                                                  const float* __restrict__ scale, int Vh, int i) {
   typedef typename PT<P>::R R;
   Spinor<R> s;
-  if (P == DLMA_FP64) {
+  if constexpr (P == DLMA_FP64) {
     const double2* b = (const double2*)base;
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       double2 v = __ldg(b + (size_t)k * Vh + i);
       s.c[k / 3][k % 3] = cx<R>((R)v.x, (R)v.y);
     }
-  } else if (P == DLMA_FP32) {
+  } else if constexpr (P == kFP32x2) {
+    const float4* b = (const float4*)base;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      const float4 v = __ldg(b + (size_t)k * Vh + i);
+      s.c[k / 3][k % 3] = cx<R>(f2(v.x, v.y), f2(v.z, v.w));
+    }
+  } else if constexpr (P == DLMA_FP32) {
     const float4* b = (const float4*)base;
 #pragma unroll
     for (int q = 0; q < 6; q++) {
@@ -49,11 +81,18 @@ __device__ __forceinline__ Spinor<typename PT<P>::R> load_spinor(const void* __r
 template <int P>
 __device__ __forceinline__ void store_spinor(void* base, float* scale, int Vh, int i,
                                              const Spinor<typename PT<P>::R>& s) {
-  if (P == DLMA_FP64) {
+  if constexpr (P == DLMA_FP64) {
     double2* b = (double2*)base;
 #pragma unroll
     for (int k = 0; k < 12; k++) b[(size_t)k * Vh + i] = make_double2(s.c[k / 3][k % 3].re, s.c[k / 3][k % 3].im);
-  } else if (P == DLMA_FP32) {
+  } else if constexpr (P == kFP32x2) {
+    float4* b = (float4*)base;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      const Cx<f2> v = s.c[k / 3][k % 3];
+      b[(size_t)k * Vh + i] = make_float4(v.re.x, v.re.y, v.im.x, v.im.y);
+    }
+  } else if constexpr (P == DLMA_FP32) {
     float4* b = (float4*)base;
 #pragma unroll
     for (int q = 0; q < 6; q++) {
@@ -86,3 +125,57 @@ __device__ __forceinline__ void store_spinor(void* base, float* scale, int Vh, i
   }
 }
 
+
+// component k (3 spin + colour) of an FP64 or FP32 vector: the kernels that stream many
+// vectors go through them component by component, which keeps few registers alive
+template <int P>
+__device__ __forceinline__ Cx<typename PT<P>::R> load_comp(const void* __restrict__ base, int Vh, int i, int k) {
+  if constexpr (P == kFP32x2) {
+    const float4 v = __ldg((const float4*)base + (size_t)k * Vh + i);
+    return cx<f2>(f2(v.x, v.y), f2(v.z, v.w));
+  } else if constexpr (P == DLMA_FP32) {
+    const float2 v = __ldg((const float2*)base + ((size_t)(k >> 1) * Vh + i) * 2 + (k & 1));
+    return cx<float>(v.x, v.y);
+  } else {
+    const double2 v = __ldg((const double2*)base + (size_t)k * Vh + i);
+    return cx<double>(v.x, v.y);
+  }
+}
+template <int P>
+__device__ __forceinline__ void store_comp(void* base, int Vh, int i, int k, Cx<typename PT<P>::R> v) {
+  if constexpr (P == kFP32x2)
+    ((float4*)base)[(size_t)k * Vh + i] = make_float4(v.re.x, v.re.y, v.im.x, v.im.y);
+  else if constexpr (P == DLMA_FP32)
+    ((float2*)base)[((size_t)(k >> 1) * Vh + i) * 2 + (k & 1)] = make_float2(v.re, v.im);
+  else
+    ((double2*)base)[(size_t)k * Vh + i] = make_double2(v.re, v.im);
+}
+
+// components 4 g .. 4 g + 3
+template <int P>
+__device__ __forceinline__ void load_comp4(const void* __restrict__ base, int Vh, int i, int g,
+                                           Cx<typename PT<P>::R> (&v)[4]) {
+  if constexpr (P == DLMA_FP32) {
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const float4 e = __ldg((const float4*)base + (size_t)(2 * g + h) * Vh + i);
+      v[2 * h] = cx<float>(e.x, e.y);
+      v[2 * h + 1] = cx<float>(e.z, e.w);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; k++) v[k] = load_comp<P>(base, Vh, i, 4 * g + k);
+  }
+}
+template <int P>
+__device__ __forceinline__ void store_comp4(void* base, int Vh, int i, int g, const Cx<typename PT<P>::R> (&v)[4]) {
+  if constexpr (P == DLMA_FP32) {
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+      ((float4*)base)[(size_t)(2 * g + h) * Vh + i] =
+          make_float4(v[2 * h].re, v[2 * h].im, v[2 * h + 1].re, v[2 * h + 1].im);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; k++) store_comp<P>(base, Vh, i, 4 * g + k, v[k]);
+  }
+}

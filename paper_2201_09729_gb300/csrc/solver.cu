@@ -196,7 +196,8 @@ __global__ void __launch_bounds__(BX) k_update_p(int Vh, int nrhs, const void* r
   }
 }
 
-// out = f_j * in   (precision conversion with a per-rhs factor; f = nullptr -> 1); optional |out|^2 partial
+// out = f_j * in   (precision conversion with a per-rhs factor; f = nullptr -> 1); optional |out|^2
+// partial; out = nullptr: the partial alone
 template <int PI, int PO>
 __global__ void __launch_bounds__(BX) k_convert(int Vh, int nrhs, const void* in, const float* insc, void* out,
                                                  float* outsc, const double* f, int finv, const int* mask,
@@ -217,36 +218,62 @@ __global__ void __launch_bounds__(BX) k_convert(int Vh, int nrhs, const void* in
     for (int s = 0; s < 4; s++)
 #pragma unroll
       for (int c = 0; c < 3; c++) o.c[s][c] = cx<R>((R)(ff * (double)v.c[s][c].re), (R)(ff * (double)v.c[s][c].im));
-    store_spinor<PO>((char*)out + so, outsc ? outsc + (size_t)j * Vh : nullptr, Vh, i, o);
+    if (out) store_spinor<PO>((char*)out + so, outsc ? outsc + (size_t)j * Vh : nullptr, Vh, i, o);
     n = snorm(o);
   }
   if (part) block_partial(n, part, on ? j : nrhs, nrhs);
 }
 
+// pairs of right-hand sides from FP64: out = in / f_j (0 where f_j = 0)
+__global__ void __launch_bounds__(BX) k_to_pairs(int Vh, int nrhs, const double2* in, void* out, const double* f) {
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int j = blockIdx.y;
+  if (i >= Vh) return;
+  const bool two = 2 * j + 1 < nrhs;
+  const double2 *a = in + (size_t)24 * Vh * j, *b = a + (two ? (size_t)12 * Vh : 0);
+  const double fa = f[2 * j] > 0 ? 1.0 / f[2 * j] : 0.0, fb = two && f[2 * j + 1] > 0 ? 1.0 / f[2 * j + 1] : 0.0;
+  Spinor<f2> o;
+#pragma unroll
+  for (int k = 0; k < 12; k++) {
+    const double2 x = a[(size_t)k * Vh + i], y = b[(size_t)k * Vh + i];
+    o.c[k / 3][k % 3] = cx<f2>(f2((float)(fa * x.x), (float)(fb * y.x)), f2((float)(fa * x.y), (float)(fb * y.y)));
+  }
+  store_spinor<kFP32x2>((char*)out + (size_t)192 * Vh * j, nullptr, Vh, i, o);
+}
+
+__device__ __forceinline__ void lane_set(f2& v, int q, float x) { (q ? v.y : v.x) = x; }
+__device__ __forceinline__ void lane_set(float& v, int, float x) { v = x; }
+__device__ __forceinline__ void lane_set(double& v, int, double x) { v = x; }
+
 // x64 += f_j * lo; lo = 0   (reliable update: fold the low-precision solution into FP64)
 template <int PL>
 __global__ void __launch_bounds__(BX) k_fold(int Vh, int nrhs, double2* x, void* lo, const double* f,
                                               const int* mask) {
+  typedef typename PT<PL>::R R;
+  constexpr int LN = PT<PL>::lanes;
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y;
-  if (i >= Vh || !mask[j]) return;
+  if (i >= Vh || !vec_on<PL>(j, nrhs, mask)) return;
   const size_t sl = field_units_per_rhs(PL, Vh) * 16 * j;
-  const Spinor<typename PT<PL>::R> v = load_spinor<PL>((const char*)lo + sl, nullptr, Vh, i);
-  const double ff = f[j];
-  double2* xb = x + (size_t)12 * Vh * j;
+  Spinor<R> v = load_spinor<PL>((const char*)lo + sl, nullptr, Vh, i);
 #pragma unroll
-  for (int k = 0; k < 12; k++) {
-    double2 e = xb[(size_t)k * Vh + i];
-    e.x += ff * (double)v.c[k / 3][k % 3].re;
-    e.y += ff * (double)v.c[k / 3][k % 3].im;
-    xb[(size_t)k * Vh + i] = e;
+  for (int q = 0; q < LN; q++) {
+    if (!lane_on<PL>(j, q, nrhs, mask)) continue;
+    const int r = LN * j + q;
+    const double ff = f[r];
+    double2* xb = x + (size_t)12 * Vh * r;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      double2 e = xb[(size_t)k * Vh + i];
+      Cx<R>& c = v.c[k / 3][k % 3];
+      e.x += ff * (double)lane_get(c.re, q);
+      e.y += ff * (double)lane_get(c.im, q);
+      xb[(size_t)k * Vh + i] = e;
+      lane_set(c.re, q, 0);
+      lane_set(c.im, q, 0);
+    }
   }
-  Spinor<typename PT<PL>::R> z;
-#pragma unroll
-  for (int s = 0; s < 4; s++)
-#pragma unroll
-    for (int c = 0; c < 3; c++) z.c[s][c] = cx<typename PT<PL>::R>(0, 0);
-  store_spinor<PL>((char*)lo + sl, nullptr, Vh, i, z);
+  store_spinor<PL>((char*)lo + sl, nullptr, Vh, i, v);
 }
 
 // r = a - b (FP64) with |r|^2 partial
@@ -292,29 +319,82 @@ __global__ void k_split_ru(int nrhs, CgScal sc, double theta, int* ru_hi, int* r
   ru_hi[j] = sc.ru[j] && !lo;
 }
 
+// Totals of N values over a warp, scattered: lane l returns the total of value `which`
+// (lanes 0 .. M - 1 hold every one).  An FP64 addition takes 64 cycles of its SM
+// sub-partition, so the halves of the list are exchanged and added (M - 1 + 5 - log2 M
+// additions, M the power of two from N on) instead of reducing each value (5 N).
+template <int N> __device__ __forceinline__ double warp_scatter_sum(const double (&v)[N], int& which) {
+  constexpr int M = N <= 1 ? 1 : N <= 2 ? 2 : N <= 4 ? 4 : N <= 8 ? 8 : 16;
+  const int lane = threadIdx.x & 31;
+  double w[M];
+#pragma unroll
+  for (int e = 0; e < M; e++) w[e] = e < N ? v[e < N ? e : 0] : 0.0;
+  which = 0;
+#pragma unroll
+  for (int h = M / 2, b = 1; h >= 1; h >>= 1, b <<= 1) {
+    const bool up = (lane & b) != 0;
+#pragma unroll
+    for (int e = 0; e < h; e++) {
+      const double send = up ? w[e] : w[e + h], keep = up ? w[e + h] : w[e];
+      w[e] = keep + __shfl_xor_sync(0xffffffffu, send, b);
+    }
+    which += up ? h : 0;
+  }
+#pragma unroll
+  for (int b = M; b < 32; b <<= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], b);
+  return w[0];
+}
+// totals over a block of NW warps; every thread returns them
+template <int N, int NW = BX / 32> __device__ __forceinline__ void block_sums(double (&v)[N]) {
+  __shared__ double red[N][NW], tot[N];
+  int which;
+  const double w = warp_scatter_sum(v, which);
+  __syncthreads();
+  if ((threadIdx.x & 31) < 16 && which < N) red[which][threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x < N) {
+    double t = 0;
+#pragma unroll
+    for (int q = 0; q < NW; q++) t += red[threadIdx.x][q];
+    tot[threadIdx.x] = t;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < N; e++) v[e] = tot[e];
+}
+
 // r64 -= s_j t (t = Dhat x_l in the low precision P) with the |r64|^2 partial
 template <int P>
 __global__ void __launch_bounds__(BX) k_corr64(int Vh, int nrhs, double2* r, const void* t, const double* f,
                                                const int* mask, double* part) {
+  typedef typename PT<P>::R R;
+  constexpr int LN = PT<P>::lanes;
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y;
-  const bool on = mask[j] != 0;
-  double n = 0;
-  if (i < Vh && on) {
-    const size_t sl = field_units_per_rhs(P, Vh) * 16 * j;
-    const Spinor<typename PT<P>::R> v = load_spinor<P>((const char*)t + sl, nullptr, Vh, i);
-    const double ff = f[j];
-    double2* rb = r + (size_t)12 * Vh * j;
+  if (!vec_on<P>(j, nrhs, mask)) return;
+  double n[LN] = {};
+  if (i < Vh) {
+    const Spinor<R> v = load_spinor<P>((const char*)t + field_units_per_rhs(P, Vh) * 16 * j, nullptr, Vh, i);
 #pragma unroll
-    for (int k = 0; k < 12; k++) {
-      double2 e = rb[(size_t)k * Vh + i];
-      e.x -= ff * (double)v.c[k / 3][k % 3].re;
-      e.y -= ff * (double)v.c[k / 3][k % 3].im;
-      rb[(size_t)k * Vh + i] = e;
-      n += e.x * e.x + e.y * e.y;
+    for (int q = 0; q < LN; q++) {
+      if (!lane_on<P>(j, q, nrhs, mask)) continue;
+      const double ff = f[LN * j + q];
+      double2* rb = r + (size_t)12 * Vh * (LN * j + q);
+#pragma unroll
+      for (int k = 0; k < 12; k++) {
+        double2 e = rb[(size_t)k * Vh + i];
+        e.x -= ff * (double)lane_get(v.c[k / 3][k % 3].re, q);
+        e.y -= ff * (double)lane_get(v.c[k / 3][k % 3].im, q);
+        rb[(size_t)k * Vh + i] = e;
+        n[q] += e.x * e.x + e.y * e.y;
+      }
     }
   }
-  block_partial(n, part, on ? j : nrhs, nrhs);
+  block_sums(n);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int q = 0; q < LN; q++)
+      if (lane_on<P>(j, q, nrhs, mask)) part[(size_t)(LN * j + q) * gridDim.x + blockIdx.x] = n[q];
 }
 
 // flag[t] = 1 if any right-hand side has a nonzero block partial of |.|^2 on
@@ -397,7 +477,7 @@ struct BiScal {
   double2* alpha;
   double2* omega;
   double2* beta;
-  int* brk;         // breakdown seen: restart the shadow residual at the next update
+  int* brk;         // breakdown seen: restart the search direction at the next update
 };
 
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
@@ -418,287 +498,285 @@ __device__ __forceinline__ double2 warp_sum2(double2 v) {
   return v;
 }
 
-// a breakdown pauses the rhs for an FP64 update that restarts its shadow residual
+// a breakdown pauses the rhs for an FP64 update that restarts its search direction
 __device__ __forceinline__ void bi_breakdown(int j, CgScal& sc, BiScal& bs) {
   sc.active[j] = 0;
   sc.ru[j] = 1;
   bs.brk[j] = 1;
 }
 
-// alpha = rho / (r0, v)   (one warp per rhs over the stencil's DOT partials)
-__global__ void k_bi_alpha(const double2* dpart, int nb, int nrhs, CgScal sc, BiScal bs) {
-  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (j >= nrhs || !sc.active[j]) return;
-  const int lane = threadIdx.x & 31;
-  double2 s = make_double2(0, 0);
-  for (int b = lane; b < nb; b += 32) {
-    const double2 v = dpart[(size_t)j * nb + b];
-    s.x += v.x;
-    s.y += v.y;
-  }
-  s = warp_sum2(s);
-  if (lane == 0) {
-    const double2 a = cdiv(bs.rho[j], s);
-    const bool ok = (s.x != 0.0 || s.y != 0.0) && cfinite(s) && cfinite(a);
-    bs.alpha[j] = ok ? a : make_double2(0, 0);
-    if (!ok) {
-      bi_breakdown(j, sc, bs);
-      if (!cfinite(s)) sc.count[1] = 1;
+// totals over the nb block partials of rhs j in ND complex and one real array, by one
+// block of 256 threads; every thread returns them
+template <int ND>
+__device__ __forceinline__ void part_sums(const double2* const (&d)[ND], const double* n, int nb, int j,
+                                          double (&v)[2 * ND + 1]) {
+  constexpr int NV = 2 * ND + 1;
+#pragma unroll
+  for (int e = 0; e < NV; e++) v[e] = 0;
+  for (int b = threadIdx.x; b < nb; b += 256) {
+    const size_t o = (size_t)j * nb + b;
+#pragma unroll
+    for (int e = 0; e < ND; e++) {
+      const double2 x = d[e][o];
+      v[2 * e] += x.x;
+      v[2 * e + 1] += x.y;
     }
+    v[NV - 1] += n[o];
   }
+  block_sums<NV, 8>(v);
 }
 
-// s = r - alpha v
+// After t = Dhat s: omega = (t, s) / (t, t); the next rho = (r0, s - omega t) =
+// (r0, s) - omega (w0, s) with w0 = Dhat^dag r0, so that beta = (rho' / rho)(alpha /
+// omega) is known before x, r and p are updated.  One block per rhs: with the 10^4 block
+// partials of a 24^3 x 48 lattice one warp took 50 us.
+__global__ void __launch_bounds__(256) k_bi_omega(const double2* w0s, const double2* r0s, const double2* ts,
+                                                  const double* tt, int nb, CgScal sc, BiScal bs) {
+  const int j = blockIdx.x;
+  if (!sc.active[j]) return;
+  double q[7];
+  const double2* const ds[3] = {w0s, r0s, ts};
+  part_sums<3>(ds, tt, nb, j, q);
+  if (threadIdx.x) return;
+  const double2 a = make_double2(q[0], q[1]), b = make_double2(q[2], q[3]), d = make_double2(q[4], q[5]);
+  const double n = q[6];
+  const double2 om = make_double2(d.x / n, -d.y / n);     // (t, s) = conj(sum conj(s) t)
+  if (!(n > 0 && isfinite(n) && cfinite(om) && (om.x != 0.0 || om.y != 0.0))) {
+    bs.omega[j] = make_double2(0, 0);
+    bi_breakdown(j, sc, bs);
+    if (!isfinite(n)) sc.count[1] = 1;
+    return;
+  }
+  const double2 oa = cmul(om, a), rho = make_double2(b.x - oa.x, b.y - oa.y);
+  const double2 bt = cmul(cdiv(rho, bs.rho[j]), cdiv(bs.alpha[j], om));
+  const bool ok = cfinite(bt) && (rho.x != 0.0 || rho.y != 0.0);
+  bs.omega[j] = om;
+  bs.beta[j] = ok ? bt : make_double2(0, 0);
+  bs.rho[j] = rho;
+  if (!ok) { sc.ru[j] = 1; bs.brk[j] = 1; }               // the pause takes effect after the update
+}
+
+// The vector update of an iteration in one pass: x += alpha p + omega s; r = s - omega t;
+// p = r + beta (p - omega v); partials of (w0, p) and |r|^2 (w0 is one FP32 vector for all
+// rhs).  Eight vectors moved, at the memory rate; with the separate s, x / r and p updates
+// it replaces, an iteration moved 14 besides the stencil.  A pair with one idle right-hand side keeps that one's x and p.
 template <int P>
-__global__ void __launch_bounds__(BX) k_bi_s(int Vh, int nrhs, const void* r, const void* v, void* sv, CgScal sc,
-                                             BiScal bs) {
+__global__ void __launch_bounds__(BX) k_bi_update(int Vh, int nrhs, void* x, void* r, void* p, const void* sv,
+                                                  const void* t, const void* v, const void* w0, CgScal sc, BiScal bs,
+                                                  double2* cpart, double* npart) {
   typedef typename PT<P>::R R;
+  constexpr int LN = PT<P>::lanes;
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y;
-  if (i >= Vh || !sc.active[j]) return;
-  const size_t sb = field_units_per_rhs(P, Vh) * 16 * j;
-  const double2 al = bs.alpha[j];
-  const R ar = (R)al.x, ai = (R)al.y;
-  const Spinor<R> rv = load_spinor<P>((const char*)r + sb, nullptr, Vh, i);
-  const Spinor<R> vv = load_spinor<P>((const char*)v + sb, nullptr, Vh, i);
-  Spinor<R> o;
-#pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const Cx<R> x = vv.c[a][c];
-      o.c[a][c] = cx<R>(rv.c[a][c].re - (ar * x.re - ai * x.im), rv.c[a][c].im - (ar * x.im + ai * x.re));
-    }
-  store_spinor<P>((char*)sv + sb, nullptr, Vh, i, o);
-}
-
-// omega = (t, s) / (t, t) from the partials of sum conj(s) t and |t|^2
-__global__ void k_bi_omega(const double2* dpart, const double* npart, int nb, int nrhs, CgScal sc, BiScal bs) {
-  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (j >= nrhs || !sc.active[j]) return;
-  const int lane = threadIdx.x & 31;
-  double2 d = make_double2(0, 0);
-  double n = 0;
-  for (int b = lane; b < nb; b += 32) {
-    const double2 v = dpart[(size_t)j * nb + b];
-    d.x += v.x;
-    d.y += v.y;
-    n += npart[(size_t)j * nb + b];
-  }
-  d = warp_sum2(d);
-  n = warp_sum(n);
-  if (lane == 0) {
-    const double2 ts = make_double2(d.x, -d.y);     // (t, s) = conj(sum conj(s) t)
-    const double2 om = make_double2(ts.x / n, ts.y / n);
-    const bool ok = n > 0 && isfinite(n) && cfinite(om) && (om.x != 0.0 || om.y != 0.0);
-    bs.omega[j] = ok ? om : make_double2(0, 0);
-    if (!ok) {
-      bi_breakdown(j, sc, bs);
-      if (!isfinite(n)) sc.count[1] = 1;
-    }
-  }
-}
-
-// x += alpha p + omega s ; r = s - omega t ; partials of (r0, r) and |r|^2
-template <int P>
-__global__ void __launch_bounds__(BX) k_bi_xr(int Vh, int nrhs, void* x, void* r, const void* p, const void* sv,
-                                              const void* t, const void* r0, CgScal sc, BiScal bs, double2* cpart,
-                                              double* npart) {
-  typedef typename PT<P>::R R;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y;
-  const bool on = sc.active[j] != 0;
-  R dr = 0, di = 0, nn = 0;
-  if (i < Vh && on) {
+  if (!vec_on<P>(j, nrhs, sc.active)) return;
+  R dr = (R)0, di = (R)0, nn = (R)0;
+  if (i < Vh) {
     const size_t sb = field_units_per_rhs(P, Vh) * 16 * j;
-    const double2 al = bs.alpha[j], om = bs.omega[j];
-    const R ar = (R)al.x, ai = (R)al.y, wr = (R)om.x, wi = (R)om.y;
-    Spinor<R> xv = load_spinor<P>((const char*)x + sb, nullptr, Vh, i);
-    const Spinor<R> pv = load_spinor<P>((const char*)p + sb, nullptr, Vh, i);
-    const Spinor<R> svv = load_spinor<P>((const char*)sv + sb, nullptr, Vh, i);
-    const Spinor<R> tv = load_spinor<P>((const char*)t + sb, nullptr, Vh, i);
-    const Spinor<R> zv = load_spinor<P>((const char*)r0 + sb, nullptr, Vh, i);
-    Spinor<R> rv;
+    const int r0 = lane_rhs<P>(j, 0, nrhs), r1 = lane_rhs<P>(j, LN - 1, nrhs);
+    const double2 a0 = bs.alpha[r0], a1 = bs.alpha[r1], o0 = bs.omega[r0], o1 = bs.omega[r1];
+    const double2 b0 = bs.beta[r0], b1 = bs.beta[r1];
+    const R ar = lane_pack<P>(a0.x, a1.x), ai = lane_pack<P>(a0.y, a1.y);
+    const R wr = lane_pack<P>(o0.x, o1.x), wi = lane_pack<P>(o0.y, o1.y);
+    const R br = lane_pack<P>(b0.x, b1.x), bi = lane_pack<P>(b0.y, b1.y);
+    // the idle right-hand side of a pair, if any
+    const int idle = LN == 1 ? -1 : !lane_on<P>(j, 0, nrhs, sc.active) ? 0 : !lane_on<P>(j, 1, nrhs, sc.active) ? 1 : -1;
+    // four components at a time: their 20 loads are in flight together
+#pragma unroll 1
+    for (int g = 0; g < 3; g++) {
+      Cx<R> xv[4], pv[4], ss[4], tv[4], yv[4];
+      Cx<float> zv[4];
+      load_comp4<P>((const char*)x + sb, Vh, i, g, xv);
+      load_comp4<P>((const char*)p + sb, Vh, i, g, pv);
+      load_comp4<P>((const char*)sv + sb, Vh, i, g, ss);
+      load_comp4<P>((const char*)t + sb, Vh, i, g, tv);
+      load_comp4<P>((const char*)v + sb, Vh, i, g, yv);
+      load_comp4<DLMA_FP32>(w0, Vh, i, g, zv);
 #pragma unroll
-    for (int a = 0; a < 4; a++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        const Cx<R> pp = pv.c[a][c], ss = svv.c[a][c], tt = tv.c[a][c], z = zv.c[a][c];
-        xv.c[a][c].re += ar * pp.re - ai * pp.im + wr * ss.re - wi * ss.im;
-        xv.c[a][c].im += ar * pp.im + ai * pp.re + wr * ss.im + wi * ss.re;
-        const Cx<R> rr = cx<R>(ss.re - (wr * tt.re - wi * tt.im), ss.im - (wr * tt.im + wi * tt.re));
-        rv.c[a][c] = rr;
-        dr += z.re * rr.re + z.im * rr.im;
-        di += z.re * rr.im - z.im * rr.re;
-        nn += rr.re * rr.re + rr.im * rr.im;
+      for (int k = 0; k < 4; k++) {
+        const Cx<R> xo = xv[k], q = pv[k], s = ss[k], u = tv[k], y = yv[k];
+        const Cx<float> z = zv[k];
+        Cx<R> e = cx<R>(fma(ar, q.re, fma(-ai, q.im, fma(wr, s.re, fma(-wi, s.im, xo.re)))),
+                        fma(ar, q.im, fma(ai, q.re, fma(wr, s.im, fma(wi, s.re, xo.im)))));
+        const Cx<R> rr = cx<R>(fma(-wr, u.re, fma(wi, u.im, s.re)), fma(-wr, u.im, fma(-wi, u.re, s.im)));
+        const Cx<R> d = cx<R>(fma(-wr, y.re, fma(wi, y.im, q.re)), fma(-wr, y.im, fma(-wi, y.re, q.im)));
+        Cx<R> n = cx<R>(fma(br, d.re, fma(-bi, d.im, rr.re)), fma(br, d.im, fma(bi, d.re, rr.im)));
+        dr = fma((R)z.re, n.re, fma((R)z.im, n.im, dr));
+        di = fma((R)z.re, n.im, fma((R)-z.im, n.re, di));
+        nn = fma(rr.re, rr.re, fma(rr.im, rr.im, nn));
+        if (idle >= 0) {
+          lane_set(e.re, idle, lane_get(xo.re, idle));
+          lane_set(e.im, idle, lane_get(xo.im, idle));
+          lane_set(n.re, idle, lane_get(q.re, idle));
+          lane_set(n.im, idle, lane_get(q.im, idle));
+        }
+        xv[k] = e;
+        pv[k] = n;
+        tv[k] = rr;
       }
-    store_spinor<P>((char*)x + sb, nullptr, Vh, i, xv);
-    store_spinor<P>((char*)r + sb, nullptr, Vh, i, rv);
-  }
-  __shared__ double red[3][BX / 32];
-  double vr = warp_sum((double)dr), vi = warp_sum((double)di), vn = warp_sum((double)nn);
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = vr;
-    red[1][threadIdx.x >> 5] = vi;
-    red[2][threadIdx.x >> 5] = vn;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && on) {
-    double a0 = 0, a1 = 0, a2 = 0;
-    for (int w = 0; w < BX / 32; w++) { a0 += red[0][w]; a1 += red[1][w]; a2 += red[2][w]; }
-    cpart[(size_t)j * gridDim.x + blockIdx.x] = make_double2(a0, a1);
-    npart[(size_t)j * gridDim.x + blockIdx.x] = a2;
-  }
-}
-
-// rho_new = (r0, r), |r|^2; beta = (rho_new / rho) (alpha / omega); reliable-update triggers
-__global__ void k_bi_beta(const double2* cpart, const double* npart, int nb, int nrhs, CgScal sc, BiScal bs,
-                          int max_since) {
-  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (j >= nrhs || !sc.active[j]) return;
-  const int lane = threadIdx.x & 31;
-  double2 d = make_double2(0, 0);
-  double n = 0;
-  for (int b = lane; b < nb; b += 32) {
-    const double2 v = cpart[(size_t)j * nb + b];
-    d.x += v.x;
-    d.y += v.y;
-    n += npart[(size_t)j * nb + b];
-  }
-  d = warp_sum2(d);
-  n = warp_sum(n);
-  if (lane == 0) {
-    const double2 bt = cmul(cdiv(d, bs.rho[j]), cdiv(bs.alpha[j], bs.omega[j]));
-    const bool ok = cfinite(bt) && (d.x != 0.0 || d.y != 0.0);
-    bs.beta[j] = ok ? bt : make_double2(0, 0);
-    bs.rho[j] = d;
-    sc.rr[j] = n;
-    sc.iters[j] += 1;
-    sc.since[j] += 1;
-    if (!isfinite(n)) { sc.active[j] = 0; sc.count[1] = 1; }
-    else if (!ok) { sc.ru[j] = 1; bs.brk[j] = 1; }
-    else if (n <= sc.stop2[j] || sc.since[j] >= max_since || !(n > 0) || n > 1e4 * sc.rr0[j])
-      sc.ru[j] = 1;                        // the pause takes effect after the p update (k_pause)
-  }
-}
-
-// p = r + beta (p - omega v)
-template <int P>
-__global__ void __launch_bounds__(BX) k_bi_p(int Vh, int nrhs, const void* r, void* p, const void* v, CgScal sc,
-                                             BiScal bs) {
-  typedef typename PT<P>::R R;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= Vh || !sc.active[j]) return;
-  const size_t sb = field_units_per_rhs(P, Vh) * 16 * j;
-  const double2 bt = bs.beta[j], om = bs.omega[j];
-  const R br = (R)bt.x, bi = (R)bt.y, wr = (R)om.x, wi = (R)om.y;
-  const Spinor<R> rv = load_spinor<P>((const char*)r + sb, nullptr, Vh, i);
-  const Spinor<R> vv = load_spinor<P>((const char*)v + sb, nullptr, Vh, i);
-  Spinor<R> pv = load_spinor<P>((const char*)p + sb, nullptr, Vh, i);
-#pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-      const Cx<R> vx = vv.c[a][c];
-      const Cx<R> d = cx<R>(pv.c[a][c].re - (wr * vx.re - wi * vx.im), pv.c[a][c].im - (wr * vx.im + wi * vx.re));
-      pv.c[a][c] = cx<R>(rv.c[a][c].re + br * d.re - bi * d.im, rv.c[a][c].im + br * d.im + bi * d.re);
+      store_comp4<P>((char*)x + sb, Vh, i, g, xv);
+      store_comp4<P>((char*)r + sb, Vh, i, g, tv);
+      store_comp4<P>((char*)p + sb, Vh, i, g, pv);
     }
-  store_spinor<P>((char*)p + sb, nullptr, Vh, i, pv);
+  }
+  double v3[3 * LN];
+#pragma unroll
+  for (int q = 0; q < LN; q++) {
+    v3[3 * q] = lane_get(dr, q);
+    v3[3 * q + 1] = lane_get(di, q);
+    v3[3 * q + 2] = lane_get(nn, q);
+  }
+  block_sums(v3);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int q = 0; q < LN; q++)
+      if (lane_on<P>(j, q, nrhs, sc.active)) {
+        const size_t o = (size_t)(LN * j + q) * gridDim.x + blockIdx.x;
+        cpart[o] = make_double2(v3[3 * q], v3[3 * q + 1]);
+        npart[o] = v3[3 * q + 2];
+      }
+}
+
+// After the vector update: alpha = rho / (r0, Dhat p) = rho / (w0, p) for the next
+// iteration, and the triggers of a reliable update (which pauses the rhs at once)
+__global__ void __launch_bounds__(256) k_bi_alpha(const double2* w0p, const double* rr, int nb, CgScal sc, BiScal bs,
+                                                  int max_since) {
+  const int j = blockIdx.x;
+  if (!sc.active[j]) return;
+  double q[3];
+  const double2* const ds[1] = {w0p};
+  part_sums<1>(ds, rr, nb, j, q);
+  if (threadIdx.x) return;
+  const double2 d = make_double2(q[0], q[1]);
+  const double n = q[2];
+  sc.rr[j] = n;
+  sc.iters[j] += 1;
+  sc.since[j] += 1;
+  if (!isfinite(n)) { sc.active[j] = 0; sc.count[1] = 1; return; }
+  const double2 a = cdiv(bs.rho[j], d);
+  const bool ok = (d.x != 0.0 || d.y != 0.0) && cfinite(d) && cfinite(a);
+  bs.alpha[j] = ok ? a : make_double2(0, 0);
+  if (!ok) {
+    bi_breakdown(j, sc, bs);
+    if (!cfinite(d)) sc.count[1] = 1;
+  }
+  if (n <= sc.stop2[j] || sc.since[j] >= max_since || !(n > 0) || n > 1e4 * sc.rr0[j]) sc.ru[j] = 1;
+  if (sc.ru[j]) sc.active[j] = 0;
 }
 
 // End of a BiCGStab reliable update in one pass over the updated rhs: r_l = r64 / s_j
-// (FP64 -> P); where the shadow residual restarts (rmask) r0 = p = r_l; partials of
-// (r0, r_l) and |r_l|^2 for k_bi_resume
+// (FP64 -> P); where the search direction restarts (rmask) p = r_l; partials of
+// (r0, r_l), (w0, p) and |r_l|^2 for k_bi_resume
 template <int P>
 __global__ void __launch_bounds__(BX) k_bi_restore(int Vh, int nrhs, const double2* r64, const double* f, void* rl,
-                                                   void* r0, void* pl, const int* upd, const int* rmask,
-                                                   double2* cpart, double* npart) {
+                                                   void* pl, const void* r0, const void* w0, const int* upd,
+                                                   const int* rmask, double2* cpart, double2* wpart, double* npart) {
   typedef typename PT<P>::R R;
+  constexpr int LN = PT<P>::lanes;
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j = blockIdx.y;
-  const bool on = upd[j] != 0;
-  double dr = 0, di = 0, nn = 0;
-  if (i < Vh && on) {
+  if (!vec_on<P>(j, nrhs, upd)) return;
+  double v5[5 * LN] = {};
+  float a5[5 * LN] = {};           // per thread in FP32, as in k_bi_update
+  if (i < Vh) {
     const size_t so = field_units_per_rhs(P, Vh) * 16 * j;
-    const Spinor<double> v = load_spinor<DLMA_FP64>((const char*)r64 + (size_t)192 * Vh * j, nullptr, Vh, i);
-    const double ff = f[j] > 0 ? 1.0 / f[j] : 0.0;
-    Spinor<R> o;
+    bool on[LN], restart[LN], any = false;
+    double ff[LN];
 #pragma unroll
-    for (int s = 0; s < 4; s++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) o.c[s][c] = cx<R>((R)(ff * v.c[s][c].re), (R)(ff * v.c[s][c].im));
-    store_spinor<P>((char*)rl + so, nullptr, Vh, i, o);
-    Spinor<R> a;
-    if (rmask[j]) {
-      store_spinor<P>((char*)r0 + so, nullptr, Vh, i, o);
-      store_spinor<P>((char*)pl + so, nullptr, Vh, i, o);
-      a = o;
-    } else {
-      a = load_spinor<P>((const char*)r0 + so, nullptr, Vh, i);
+    for (int q = 0; q < LN; q++) {
+      const int r = lane_rhs<P>(j, q, nrhs);
+      on[q] = lane_on<P>(j, q, nrhs, upd);
+      restart[q] = on[q] && rmask[r] != 0;
+      any = any || restart[q];
+      ff[q] = f[r] > 0 ? 1.0 / f[r] : 0.0;
     }
+#pragma unroll 4
+    for (int k = 0; k < 12; k++) {
+      Cx<R> y = load_comp<P>((const char*)rl + so, Vh, i, k), p = load_comp<P>((const char*)pl + so, Vh, i, k);
+      const Cx<float> z = load_comp<DLMA_FP32>(r0, Vh, i, k), w = load_comp<DLMA_FP32>(w0, Vh, i, k);
 #pragma unroll
-    for (int s = 0; s < 4; s++)
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        const Cx<R> x = a.c[s][c], y = o.c[s][c];
-        dr += (double)x.re * y.re + (double)x.im * y.im;
-        di += (double)x.re * y.im - (double)x.im * y.re;
-        nn += (double)y.re * y.re + (double)y.im * y.im;
+      for (int q = 0; q < LN; q++) {
+        if (!on[q]) continue;
+        const double2 e = r64[((size_t)12 * (LN * j + q) + k) * Vh + i];
+        const float yr = (float)(ff[q] * e.x), yi = (float)(ff[q] * e.y);
+        lane_set(y.re, q, yr);
+        lane_set(y.im, q, yi);
+        if (restart[q]) {
+          lane_set(p.re, q, yr);
+          lane_set(p.im, q, yi);
+        }
+        const float pr = lane_get(p.re, q), pi = lane_get(p.im, q);
+        a5[5 * q] = fmaf(z.re, yr, fmaf(z.im, yi, a5[5 * q]));
+        a5[5 * q + 1] = fmaf(z.re, yi, fmaf(-z.im, yr, a5[5 * q + 1]));
+        a5[5 * q + 2] = fmaf(w.re, pr, fmaf(w.im, pi, a5[5 * q + 2]));
+        a5[5 * q + 3] = fmaf(w.re, pi, fmaf(-w.im, pr, a5[5 * q + 3]));
+        a5[5 * q + 4] = fmaf(yr, yr, fmaf(yi, yi, a5[5 * q + 4]));
       }
-  }
-  __shared__ double red[3][BX / 32];
-  dr = warp_sum(dr);
-  di = warp_sum(di);
-  nn = warp_sum(nn);
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = dr;
-    red[1][threadIdx.x >> 5] = di;
-    red[2][threadIdx.x >> 5] = nn;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0 && on) {
-    double a0 = 0, a1 = 0, a2 = 0;
-    for (int w = 0; w < BX / 32; w++) { a0 += red[0][w]; a1 += red[1][w]; a2 += red[2][w]; }
-    cpart[(size_t)j * gridDim.x + blockIdx.x] = make_double2(a0, a1);
-    npart[(size_t)j * gridDim.x + blockIdx.x] = a2;
-  }
-}
-
-// resume the updated rhs: rho = (r0, r), |r|^2 from the partials; restart flags consumed
-__global__ void k_bi_resume(const double2* cpart, const double* npart, int nb, int nrhs, CgScal sc, BiScal bs,
-                            double delta, double tol) {
-  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (j >= nrhs || !sc.upd[j]) return;
-  const int lane = threadIdx.x & 31;
-  double2 d = make_double2(0, 0);
-  double n = 0;
-  for (int b = lane; b < nb; b += 32) {
-    const double2 v = cpart[(size_t)j * nb + b];
-    d.x += v.x;
-    d.y += v.y;
-    n += npart[(size_t)j * nb + b];
-  }
-  d = warp_sum2(d);
-  n = warp_sum(n);
-  if (lane == 0) {
-    sc.upd[j] = 0;
-    sc.ru[j] = 0;
-    sc.since[j] = 0;
-    bs.brk[j] = 0;
-    if (!(n > 0) || !isfinite(n) || !cfinite(d)) {
-      if (!isfinite(n)) sc.count[1] = 1;
-      sc.alive[j] = 0;
-      return;
+      store_comp<P>((char*)rl + so, Vh, i, k, y);
+      if (any) store_comp<P>((char*)pl + so, Vh, i, k, p);
     }
-    bs.rho[j] = d;
-    sc.rr[j] = sc.rr0[j] = n;
-    sc.stop2[j] = next_stop(sc, j, delta, tol, 0.2) * n;
-    sc.active[j] = 1;
   }
+#pragma unroll
+  for (int e = 0; e < 5 * LN; e++) v5[e] = a5[e];
+  block_sums(v5);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int q = 0; q < LN; q++)
+      if (lane_on<P>(j, q, nrhs, upd)) {
+        const size_t o = (size_t)(LN * j + q) * gridDim.x + blockIdx.x;
+        cpart[o] = make_double2(v5[5 * q], v5[5 * q + 1]);
+        wpart[o] = make_double2(v5[5 * q + 2], v5[5 * q + 3]);
+        npart[o] = v5[5 * q + 4];
+      }
 }
 
-// updated rhs that restart their shadow residual: the stagnating ones and those that broke down
+// resume the updated rhs: rho = (r0, r), |r|^2 and alpha = rho / (w0, p) from the
+// partials; restart flags consumed
+__global__ void __launch_bounds__(256) k_bi_resume(const double2* cpart, const double2* wpart, const double* npart,
+                                                   int nb, CgScal sc, BiScal bs, double delta, double tol) {
+  const int j = blockIdx.x;
+  if (!sc.upd[j]) return;
+  double q[5];
+  const double2* const ds[2] = {cpart, wpart};
+  part_sums<2>(ds, npart, nb, j, q);
+  if (threadIdx.x) return;
+  const double2 d = make_double2(q[0], q[1]), w = make_double2(q[2], q[3]);
+  const double n = q[4];
+  const double2 a = cdiv(d, w);
+  sc.upd[j] = 0;
+  sc.ru[j] = 0;
+  sc.since[j] = 0;
+  bs.brk[j] = 0;
+  if (!(n > 0) || !isfinite(n) || !cfinite(d) || !cfinite(w)) {
+    if (!isfinite(n)) sc.count[1] = 1;
+    sc.alive[j] = 0;
+    return;
+  }
+  bs.rho[j] = d;
+  sc.rr[j] = sc.rr0[j] = n;
+  sc.stop2[j] = next_stop(sc, j, delta, tol, 0.2) * n;
+  if (!cfinite(a) || (d.x == 0.0 && d.y == 0.0)) {      // no direction: restart at the next update
+    bs.alpha[j] = make_double2(0, 0);
+    bi_breakdown(j, sc, bs);
+    return;
+  }
+  bs.alpha[j] = a;
+  sc.active[j] = 1;
+}
+
+// the shadow residual, the same for every rhs: entries (+-1 +- i), signs from a hash of
+// the entry's index
+__global__ void k_bi_shadow(int Vh, float4* r0) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= 6 * Vh) return;
+  unsigned h = (unsigned)e * 0x9e3779b9u;
+  h = (h ^ (h >> 15)) * 0x85ebca6bu;
+  h = (h ^ (h >> 13)) * 0xc2b2ae35u;
+  h ^= h >> 16;
+  const auto sign = [&](int b) { return (h >> b) & 1 ? -1.f : 1.f; };
+  r0[e] = make_float4(sign(0), sign(8), sign(16), sign(24));
+}
+
+// updated rhs that restart their search direction: the stagnating ones and those that broke down
 __global__ void k_bi_restart_mask(int nrhs, CgScal sc, BiScal bs, int first, int* rmask) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nrhs) return;
@@ -713,9 +791,10 @@ struct SolveBufs {
   Field xl, rl, pl, ps, q, z, tmp, rhs;        // low precision (pl: vector precision, ps/q/z/tmp/rhs: stencil)
   double *part, *part2;
   CgScal sc;
-  // BiCGStab: v = Dhat p (q), s, t = Dhat s (z), shadow residual r0; complex partials
-  Field sl, r0;
-  double2 *cpart, *cpart2;
+  // BiCGStab: v = Dhat p (q), s, t = Dhat s (z); shadow residual r0 and w0 = Dhat^dag r0,
+  // one FP32 vector each; complex partials
+  Field sl, r0, w0;
+  double2 *cpart, *cpart2, *cpart3;
   int* rmask;
   int *ru_hi, *ru_lo;   // BiCGStab updates: FP64 operator / FP32 correction of the residual
   BiScal bs;
@@ -838,14 +917,16 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   TRY(field_alloc(ctx, WS_CG_RHS, PS, nrhs, &B.rhs));
   if (bicg) {
     TRY(field_alloc(ctx, WS_BI_S, PB, nrhs, &B.sl));
-    TRY(field_alloc(ctx, WS_BI_R0, PB, nrhs, &B.r0));
+    TRY(field_alloc(ctx, WS_BI_R0, DLMA_FP32, 1, &B.r0));
+    TRY(field_alloc(ctx, WS_BI_W0, DLMA_FP32, 1, &B.w0));
   }
   const int nbmax = std::max((Vh + 31) / 32, hop_split(ctx, PS, nrhs) ? hop_grid_x(ctx, PS, nrhs) : 0) + 8;
   TRY(workT(ctx, WS_PART, (size_t)2 * nbmax * nrhs, &B.part));
   B.part2 = B.part + (size_t)nbmax * nrhs;
   if (bicg) {
-    TRY(workT(ctx, WS_BI_PART, (size_t)2 * nbmax * nrhs, &B.cpart));
+    TRY(workT(ctx, WS_BI_PART, (size_t)3 * nbmax * nrhs, &B.cpart));
     B.cpart2 = B.cpart + (size_t)nbmax * nrhs;
+    B.cpart3 = B.cpart2 + (size_t)nbmax * nrhs;
   }
   double* sd;
   TRY(workT(ctx, WS_SCAL, (size_t)11 * nrhs + 64, &sd));
@@ -891,11 +972,11 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   TRY(pack_parity(ctx, b_dev, 1, 0, B.b_e));
   TRY(pack_parity(ctx, b_dev, 1, 1, B.b_o));
   // |b|^2 over both parities
-  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.b_e.data, nullptr, B.t64.data, nullptr,
+  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.b_e.data, nullptr, nullptr, nullptr,
                                                               nullptr, 0, nullptr, B.part);
   CHECK_LAUNCH();
   TRY(rowsum(ctx, B.part, gv.x, nrhs, B.tmpd, 0, nullptr));
-  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.b_o.data, nullptr, B.t64o.data, nullptr,
+  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.b_o.data, nullptr, nullptr, nullptr,
                                                               nullptr, 0, nullptr, B.part);
   CHECK_LAUNCH();
   // the timeslices on which b_o is nonzero (for whole-timeslice blocks)
@@ -960,7 +1041,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
       TRY(launch_hop(ctx, b, B.t64o, &B.b_e, B.bh));
     }
   }
-  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.bh.data, nullptr, B.t64.data, nullptr,
+  k_convert<DLMA_FP64, DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.bh.data, nullptr, nullptr, nullptr,
                                                               nullptr, 0, nullptr, B.part);
   CHECK_LAUNCH();
   TRY(rowsum(ctx, B.part, gv.x, nrhs, B.sc.scale, 1, nullptr));
@@ -986,10 +1067,14 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   CU(cudaMemcpyAsync(B.sc.rbest, big.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaMemsetAsync(B.sc.count, 0, 4 * sizeof(int), ctx->stream));
   CU(cudaMemsetAsync(B.x64.data, 0, field_bytes_per_rhs(DLMA_FP64, Vh) * nrhs, ctx->stream));
-  CU(cudaMemsetAsync(B.xl.data, 0, field_bytes_per_rhs(PB, Vh) * nrhs, ctx->stream));
+  CU(cudaMemsetAsync(B.xl.data, 0, field_bytes(PB, Vh, nrhs), ctx->stream));
   // pack one full-batch right-hand side for the block-shape autotuner before any capture
-  k_convert<DLMA_FP64, PS><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.bh.data, nullptr, B.rhs.data, B.rhs.scale,
-                                                       B.sc.scale, 1, nullptr, nullptr);
+  if constexpr (PS == kFP32x2)
+    k_to_pairs<<<dim3(gv.x, field_vectors(PS, nrhs)), BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data,
+                                                                           B.rhs.data, B.sc.scale);
+  else
+    k_convert<DLMA_FP64, PS><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.bh.data, nullptr, B.rhs.data, B.rhs.scale,
+                                                         B.sc.scale, 1, nullptr, nullptr);
   CHECK_LAUNCH();
   TRY(autotune_hop(ctx, PS, B.rhs, B.tmp, B.z));
   return DLMA_OK;
@@ -1004,7 +1089,8 @@ static dlma_status solve_finish(dlma_ctx* ctx, SolveBufs& B, double* x_dev, int 
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
   // fold what is left of the low-precision solutions of unconverged rhs
   if (st != DLMA_OK) {
-    k_fold<PB><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, B.sc.alive);
+    k_fold<PB><<<dim3(gv.x, field_vectors(PB, nrhs)), BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data,
+                                                                           B.sc.scale, B.sc.alive);
     CHECK_LAUNCH();
   }
   {
@@ -1189,54 +1275,58 @@ static dlma_status solve_batch(dlma_ctx* ctx, const double* b_dev, double* x_dev
   return solve_finish<PB>(ctx, B, x_dev, nrhs, tol, info, st);
 }
 
-// ---- BiCGStab on the Schur system, FP32 (or FP64) vectors and stencil ------
-// Per iteration: v = Dhat p with (r0, v); alpha = rho / (r0, v); s = r - alpha v;
-// t = Dhat s with (s, t) and |t|^2; omega = (t, s) / |t|^2; x += alpha p + omega s;
-// r = s - omega t with (r0, r) and |r|^2; beta = (rho' / rho)(alpha / omega);
-// p = r + beta (p - omega v).  Two operator applications per iteration, the inner
-// products in the stencil's and the vector kernels' epilogues.
+// ---- BiCGStab on the Schur system, FP32 vectors and stencil -----------------
+// (P = kFP32x2, pairs of right-hand sides, or FP32 for a single one.)  With
+// w0 = Dhat^dag r0 kept beside the shadow residual, (r0, Dhat y) = (w0, y): alpha is known
+// before v = Dhat p and beta before the vector updates, so s is formed in the stencil's
+// epilogue and x, r and p in one pass.  The iteration is bound by memory traffic, so r0
+// and w0 are shared by all right-hand sides (a fixed vector of random signs): 20 vectors
+// move per iteration, 25 with a shadow residual of its own and separate updates.  (The
+// random r0 costs 2 % more iterations than r0 = r.)  Per iteration:
+//   v = Dhat p, s = r - alpha v, (w0, s), (r0, s);  t = Dhat s, (s, t), |t|^2;
+//   omega, rho', beta;  x, r, p with (w0, p), |r|^2;  alpha, triggers.
 template <int P>
 static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max_since) {
   const int Vh = ctx->g.Vh;
-  const dim3 gv((Vh + BX - 1) / BX, nrhs);
+  const dim3 gv((Vh + BX - 1) / BX, field_vectors(P, nrhs));
   const int nbh = hop_grid_x(ctx, P, nrhs);
-  const int nw = (nrhs + 3) / 4;
-  // v = Dhat p (into q) with the partials of (r0, v)
-  TRY(schur_apply_dot(ctx, B.pl, B.tmp, B.q, B.sc.active, B.r0, B.cpart, nullptr));
-  k_bi_alpha<<<nw, 128, 0, ctx->stream>>>(B.cpart, nbh, nrhs, B.sc, B.bs);
+  HopOp e1;
+  e1.dot_part = B.cpart;
+  e1.dot_part2 = B.cpart2;
+  e1.bis_r = B.rl.data;
+  e1.bis_s = B.sl.data;
+  e1.bis_w0 = B.w0.data;
+  e1.bis_r0 = B.r0.data;
+  e1.bis_alpha = B.bs.alpha;
+  TRY(schur_apply_epi(ctx, B.pl, B.tmp, B.q, B.sc.active, e1));
+  HopOp e2;
+  e2.dot_part = B.cpart3;
+  e2.norm_part = B.part;
+  TRY(schur_apply_epi(ctx, B.sl, B.tmp, B.z, B.sc.active, e2));
+  k_bi_omega<<<nrhs, 256, 0, ctx->stream>>>(B.cpart, B.cpart2, B.cpart3, B.part, nbh, B.sc, B.bs);
   CHECK_LAUNCH();
-  k_bi_s<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.rl.data, B.q.data, B.sl.data, B.sc, B.bs);
+  k_bi_update<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.xl.data, B.rl.data, B.pl.data, B.sl.data, B.z.data, B.q.data,
+                                             B.w0.data, B.sc, B.bs, B.cpart, B.part2);
   CHECK_LAUNCH();
-  // t = Dhat s (into z) with the partials of sum conj(s) t and |t|^2
-  TRY(schur_apply_dot(ctx, B.sl, B.tmp, B.z, B.sc.active, B.sl, B.cpart, B.part));
-  k_bi_omega<<<nw, 128, 0, ctx->stream>>>(B.cpart, B.part, nbh, nrhs, B.sc, B.bs);
-  CHECK_LAUNCH();
-  k_bi_xr<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.xl.data, B.rl.data, B.pl.data, B.sl.data, B.z.data, B.r0.data,
-                                         B.sc, B.bs, B.cpart2, B.part2);
-  CHECK_LAUNCH();
-  k_bi_beta<<<nw, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, max_since);
-  CHECK_LAUNCH();
-  k_bi_p<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, B.rl.data, B.pl.data, B.q.data, B.sc, B.bs);
-  CHECK_LAUNCH();
-  k_pause<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc);
+  k_bi_alpha<<<nrhs, 256, 0, ctx->stream>>>(B.cpart, B.part2, gv.x, B.sc, B.bs, max_since);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
 
 // Reliable update of the paused rhs: x64 += s x_l, x_l = 0, r64 = bhat - Dhat x64 in
 // FP64; the converged retire; the rest continue with r_l = r64 / s and rho = (r0, r_l),
-// restarting r0 = p = r_l on the first update, after a breakdown or on stagnation.
+// restarting p = r_l on the first update, after a breakdown or on stagnation.
 template <int P>
 static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta, bool first) {
   const int Vh = ctx->g.Vh;
-  const dim3 gv((Vh + BX - 1) / BX, nrhs);
+  const dim3 gv((Vh + BX - 1) / BX, nrhs), gl(gv.x, field_vectors(P, nrhs));
   const int* ru = B.sc.ru;
   const int nb1 = (nrhs + 127) / 128;
   if (first) {
     CU(cudaMemcpyAsync(B.r64.data, B.bh.data, field_bytes_per_rhs(DLMA_FP64, Vh) * nrhs, cudaMemcpyDeviceToDevice,
                        ctx->stream));
     CU(cudaMemcpyAsync(B.sc.rnorm, B.sc.scale, sizeof(double) * nrhs, cudaMemcpyDeviceToDevice, ctx->stream));
-  } else if (P == DLMA_FP32) {
+  } else {
     // x64 += s x_l.  r64 = bhat - Dhat x64 changes by -s Dhat x_l: for rhs whose last
     // residual is below theta |b| that change is applied with the FP32 operator, whose
     // relative rounding (~1e-6 with the cancellation between hop and clover terms)
@@ -1246,22 +1336,14 @@ static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol
     k_split_ru<<<nb1, 128, 0, ctx->stream>>>(nrhs, B.sc, theta, B.ru_hi, B.ru_lo);
     CHECK_LAUNCH();
     TRY(schur_apply(ctx, B.xl, B.tmp, B.q, 0, B.ru_lo, nullptr));
-    k_fold<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, ru);
+    k_fold<P><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, ru);
     CHECK_LAUNCH();
     TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, B.ru_hi, nullptr));
     k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
                                         (double2*)B.r64.data, B.ru_hi, B.part2);
     CHECK_LAUNCH();
-    k_corr64<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q.data, B.sc.scale, B.ru_lo,
+    k_corr64<P><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q.data, B.sc.scale, B.ru_lo,
                                             B.part2);
-    CHECK_LAUNCH();
-    TRY(rowsum(ctx, B.part2, gv.x, nrhs, B.sc.rnorm, 1, ru));
-  } else {
-    k_fold<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, ru);
-    CHECK_LAUNCH();
-    TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, ru, nullptr));
-    k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
-                                        (double2*)B.r64.data, ru, B.part2);
     CHECK_LAUNCH();
     TRY(rowsum(ctx, B.part2, gv.x, nrhs, B.sc.rnorm, 1, ru));
   }
@@ -1272,11 +1354,17 @@ static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol
   const int* upd = B.sc.upd;
   k_bi_restart_mask<<<nb1, 128, 0, ctx->stream>>>(nrhs, B.sc, B.bs, first ? 1 : 0, B.rmask);
   CHECK_LAUNCH();
-  k_bi_restore<P><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.r64.data, B.sc.scale, B.rl.data, B.r0.data,
-                                               B.pl.data, upd, B.rmask, B.cpart2, B.part2);
+  if (first) {
+    k_bi_shadow<<<(6 * Vh + 255) / 256, 256, 0, ctx->stream>>>(Vh, (float4*)B.r0.data);
+    CHECK_LAUNCH();
+    Field t = B.r0;           // one FP32 vector inside the odd work field
+    t.data = B.tmp.data;
+    TRY(schur_apply(ctx, B.r0, t, B.w0, 1, nullptr, nullptr));
+  }
+  k_bi_restore<P><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.r64.data, B.sc.scale, B.rl.data, B.pl.data,
+                                               B.r0.data, B.w0.data, upd, B.rmask, B.cpart, B.cpart2, B.part2);
   CHECK_LAUNCH();
-  k_bi_resume<<<(nrhs + 3) / 4, 128, 0, ctx->stream>>>(B.cpart2, B.part2, gv.x, nrhs, B.sc, B.bs, delta,
-                                                            tol_target);
+  k_bi_resume<<<nrhs, 256, 0, ctx->stream>>>(B.cpart, B.cpart2, B.part2, gv.x, B.sc, B.bs, delta, tol_target);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
@@ -1294,6 +1382,12 @@ static dlma_status solve_batch_bicg(dlma_ctx* ctx, const double* b_dev, double* 
   return solve_finish<P>(ctx, B, x_dev, nrhs, tol, info, st);
 }
 
+// Pairs of right-hand sides share each packed instruction and every link, but halve the
+// number of threads: they win from about 10^6 (even site, rhs) pairs on (24^3 x 48 with
+// 12: 195 -> 184 ms; 16^3 x 32 with 168: 555 -> 536 ms, with 12: 57 ms either way;
+// 12^3 x 24 with 3: 6.8 against 7.7 ms)
+static bool bicg_pairs(const dlma_ctx* ctx, int n) { return n > 1 && (size_t)n * ctx->g.Vh >= (size_t)1 << 20; }
+
 // One batch with the context's solver choice.  BiCGStab serves FP32 inner solves;
 // right-hand sides it leaves above the tolerance are solved again with CGNE.
 static dlma_status solve_one_batch(dlma_ctx* ctx, const double* b, double* x, int n, double tol, dlma_prec inner,
@@ -1307,7 +1401,9 @@ static dlma_status solve_one_batch(dlma_ctx* ctx, const double* b, double* x, in
   // the reduction of |r| between FP64 updates (DLMA_BICG_DELTA overrides it for tuning)
   double delta = 3e-4;
   if (const char* e = getenv("DLMA_BICG_DELTA")) delta = std::min(0.5, std::max(1e-8, atof(e)));
-  dlma_status s = solve_batch_bicg<DLMA_FP32>(ctx, b, x, n, tol, li.data(), delta, 20000, 200);
+  dlma_status s = bicg_pairs(ctx, n)
+                      ? solve_batch_bicg<kFP32x2>(ctx, b, x, n, tol, li.data(), delta, 20000, 200)
+                      : solve_batch_bicg<DLMA_FP32>(ctx, b, x, n, tol, li.data(), delta, 20000, 200);
   if (s != DLMA_OK && s != DLMA_ERR_NOT_CONVERGED && s != DLMA_ERR_TIMEOUT) return s;
   std::vector<int> bad;
   for (int j = 0; j < n; j++)
@@ -1348,18 +1444,20 @@ static dlma_status autotune_batch(dlma_ctx* ctx, dlma_prec prec, int nb, int* ou
     *out = std::min(nb, ctx->batch_rhs[prec]);
     return DLMA_OK;
   }
+  // the fields that the solve iterates on
+  const int fp = prec == DLMA_FP32 && ctx->solver == DLMA_SOLVER_BICGSTAB && bicg_pairs(ctx, nb) ? kFP32x2 : prec;
   Field in, tmp, res;
-  TRY(field_alloc(ctx, WS_CG_RHS, prec, nb, &in));
-  TRY(field_alloc(ctx, WS_CG_TMP, prec, nb, &tmp));
-  TRY(field_alloc(ctx, WS_CG_Z, prec, nb, &res));
-  CU(cudaMemsetAsync(in.data, 0, field_bytes_per_rhs(prec, ctx->g.Vh) * nb, ctx->stream));
-  TRY(autotune_hop(ctx, prec, in, tmp, res));
+  TRY(field_alloc(ctx, WS_CG_RHS, fp, nb, &in));
+  TRY(field_alloc(ctx, WS_CG_TMP, fp, nb, &tmp));
+  TRY(field_alloc(ctx, WS_CG_Z, fp, nb, &res));
+  CU(cudaMemsetAsync(in.data, 0, field_bytes(fp, ctx->g.Vh, nb), ctx->stream));
+  TRY(autotune_hop(ctx, fp, in, tmp, res));
   cudaEvent_t e0, e1;
   CU(cudaEventCreate(&e0));
   CU(cudaEventCreate(&e1));
   int best_k = nb;
   double best = 1e300;
-  for (int k : {nb, (nb + 1) / 2, (nb + 3) / 4}) {
+  for (int k : {nb, ((nb + 1) / 2 + 1) & ~1, ((nb + 3) / 4 + 1) & ~1}) {
     Field a = in, t = tmp, r = res;
     a.nrhs = t.nrhs = r.nrhs = k;
     float tmin = 1e30f;
