@@ -11,7 +11,7 @@
 // meeting in shared memory: about 100 FP64 instructions deep, 41 warp instructions per
 // pair against k_hop's 37, so k_hop stays ahead once every sub-partition has a warp of
 // its own (kHopSplitPairs).  Measured, one Schur application on 4^3 x 8: 87 -> 20 us with
-// one vector, 87 -> 31 us with 12 (12 us at the FP64 rate; the rest is the latency of two
+// one vector, 87 -> 29 us with 12 (12 us at the FP64 rate; the rest is the latency of two
 // dependent loads and two barriers per launch).  Signs, factors +-i and the conjugations are integer
 // operations on the operands, not FP64 ones.
 //
@@ -86,20 +86,25 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
   if (i >= g.Vh) i -= g.Vh;
   __shared__ double2 W[kSplitSites][16][3];
   __shared__ double2 Rs[kSplitSites][12];
-  const int sp = q / 3, c = q - 3 * sp, ch = sp >> 1, row = (sp & 1) * 3 + c;   // step 2's spin-colour row
-  const bool work = on && q < 12;
+  // step 2: 12 threads per site, in three full warps
+  const int s2 = threadIdx.x / 12, q2 = threadIdx.x - 12 * s2;
+  const int sp = q2 / 3, c = q2 - 3 * sp, ch = sp >> 1, row = (sp & 1) * 3 + c;
+  const int il2 = tile * kSplitSites + s2;
+  const bool work = s2 < kSplitSites && il2 < a.nsites;
+  int i2 = a.site0 + il2;
+  if (i2 >= g.Vh) i2 -= g.Vh;
   Cx<double> ko[6], ow[6];
   if (work && a.own_op) {
-    const double2* o = a.own.p + (size_t)j * a.own.rhs + split_site(g, a.own.lay, a.p_out, i);
+    const double2* o = a.own.p + (size_t)j * a.own.rhs + split_site(g, a.own.lay, a.p_out, i2);
     const size_t cs = a.own.lay == kLayInternal ? (size_t)g.Vh : 1;
 #pragma unroll
     for (int r = 0; r < 6; r++) {
       const double2 e = o[(size_t)(6 * ch + r) * cs];
       ow[r] = cx<double>(e.x, e.y);
     }
-    if (a.own_op == 2) load_row(a.Kown, g.Vh, i, ch, row, ko);
+    if (a.own_op == 2) load_row(a.Kown, g.Vh, i2, ch, row, ko);
   }
-  if (work && a.kout) load_row(a.Kout, g.Vh, i, ch, row, ko);
+  if (work && a.kout) load_row(a.Kout, g.Vh, i2, ch, row, ko);
   if (a.hop && on) {
     // 1. one direction and one projected spin: w = U (psi_s + coef psi_k), or U^dag
     const int d = q >> 1, h = q & 1, mu = d >> 1, bwd = d & 1;
@@ -144,7 +149,7 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
       const int h = up ? sp : ((mu == 0 || mu == 3) ? sp - 2 : 3 - sp);
       const int imag = !up && (mu == 1 || mu == 3);
       const int neg = !up && (mu == 0 ? bwd : mu == 1 ? 1 - bwd : (bwd ^ (sp == 2)));
-      const double2 w = W[sl][2 * d + h][c];
+      const double2 w = W[s2][2 * d + h][c];
       res = res + unit_mul(cx<double>(w.x, w.y), imag, neg);
     }
     const double f = flip_if(-0.5 * a.s, a.g5_hop && sp >= 2);
@@ -161,19 +166,19 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
     res = res + t;
   }
   if (a.kout) {
-    if (work) Rs[sl][q] = make_double2(res.re, res.im);
+    if (work) Rs[s2][q2] = make_double2(res.re, res.im);
     __syncthreads();
     if (work) {
       Cx<double> v[6];
 #pragma unroll
-      for (int r = 0; r < 6; r++) v[r] = cx<double>(Rs[sl][6 * ch + r].x, Rs[sl][6 * ch + r].y);
+      for (int r = 0; r < 6; r++) v[r] = cx<double>(Rs[s2][6 * ch + r].x, Rs[s2][6 * ch + r].y);
       res = row_mul(ko, v);
     }
   }
   double nrm = 0;
   if (work) {
     if (a.cg_x) {                            // the CG update of k_hop's epilogue
-      const size_t o = ((size_t)12 * j + q) * g.Vh + i;
+      const size_t o = ((size_t)12 * j + q2) * g.Vh + i2;
       const double al = a.cg_alpha[j];
       double2 x = a.cg_x[o], r = a.cg_r[o];
       const double2 p = a.cg_p[o];
@@ -183,8 +188,8 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
       a.cg_r[o] = r;
       nrm = r.x * r.x + r.y * r.y;
     } else {
-      double2* o = a.out.p + (size_t)j * a.out.rhs + split_site(g, a.out.lay, a.p_out, i);
-      o[(size_t)q * (a.out.lay == kLayInternal ? (size_t)g.Vh : 1)] = make_double2(res.re, res.im);
+      double2* o = a.out.p + (size_t)j * a.out.rhs + split_site(g, a.out.lay, a.p_out, i2);
+      o[(size_t)q2 * (a.out.lay == kLayInternal ? (size_t)g.Vh : 1)] = make_double2(res.re, res.im);
       nrm = norm2(res);
     }
   }
