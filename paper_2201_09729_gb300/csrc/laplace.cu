@@ -73,126 +73,222 @@ __device__ __forceinline__ void ld_cols(const Cx<float>* __restrict__ p, Cx<floa
   }
 }
 template <int NC>
-__device__ __forceinline__ void ld_cols(const Cx<double>* __restrict__ p, Cx<double> (&v)[NC]) {
-#pragma unroll
-  for (int c = 0; c < NC; c++) v[c] = p[c];
-}
-template <int NC>
 __device__ __forceinline__ void st_cols(Cx<float>* p, const Cx<float> (&v)[NC]) {
 #pragma unroll
   for (int c = 0; c < NC; c += 2) *(float4*)(p + c) = make_float4(v[c].re, v[c].im, v[c + 1].re, v[c + 1].im);
 }
-template <int NC>
-__device__ __forceinline__ void st_cols(Cx<double>* p, const Cx<double> (&v)[NC]) {
-#pragma unroll
-  for (int c = 0; c < NC; c++) p[c] = v[c];
-}
-
 // storage (R) <-> arithmetic (A) precision: A = R, or A = df for FP64 storage (the
 // double-float arithmetic of the FP64 phase, see dfloat.cuh)
 template <class A, class R> __device__ __forceinline__ Cx<A> to_a(Cx<R> v) { return cx<A>((A)v.re, (A)v.im); }
 template <class R, class A> __device__ __forceinline__ Cx<R> to_s(Cx<A> v) { return cx<R>((R)v.re, (R)v.im); }
 
-// out = alpha_t (A in) + beta_t in + gamma_t prev + alpha_t s[t][j] rin,  A = 6 - hopping = -lap
-// (in == nullptr: the stencil and beta terms vanish; prev / rin may be nullptr).
-// One thread per (site, NC adjacent columns): the six links of the site are loaded
-// (and, in FP32, rebuilt from 12 reals) once for NC columns.  The FP32 form is
-// compiled for three blocks per SM (80 registers, a few spilled words: matvec of
-// 16^3 x 32, N = 32, 61 -> 56 ms against two blocks), FP64 for two.  The block is
-// [t][site][colour][m] with m even, so a pair of FP32 columns is 16-byte aligned.
-template <class R, class A, int NC>
-__global__ void __launch_bounds__(256, sizeof(A) == 4 ? 3 : 2) k_lap(Geom g, int t0, int Tn, int m, const typename LinkT<R>::T* __restrict__ U,
-                                             const Cx<R>* __restrict__ in, const Cx<R>* __restrict__ prev,
-                                             const Cx<float>* __restrict__ rin, const double* __restrict__ scol,
-                                             Cx<R>* __restrict__ out, const double* __restrict__ coef) {
+// out = A in, A = 6 - hopping = -lap, in FP64: one thread per (site, column); the block is
+// [t][site][colour][m].  Bound by FP64 arithmetic (about 250 instructions per entry).
+__global__ void __launch_bounds__(256, 2) k_lap(Geom g, int t0, int Tn, int m, const double2* __restrict__ U,
+                                                const Cx<double>* __restrict__ in, Cx<double>* __restrict__ out) {
   // 32-bit index arithmetic (the host keeps Tn Vs m below 2^31): 64-bit divisions
   // would cost more than the stencil's arithmetic
   const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned mg = (unsigned)m / NC;
-  const unsigned total = (unsigned)Tn * (unsigned)g.Vs * mg;
-  if (e >= total) return;
-  const unsigned sl = e / mg;
-  const int j0 = (int)(e - sl * mg) * NC;
+  if (e >= (unsigned)Tn * (unsigned)g.Vs * (unsigned)m) return;
+  const unsigned sl = e / (unsigned)m;
+  const int j0 = (int)(e - sl * (unsigned)m);
   const int tl = (int)(sl / (unsigned)g.Vs);
   const int ms = (int)(sl - (unsigned)tl * (unsigned)g.Vs);
-  const A alpha = (A)coef[3 * tl], beta = (A)coef[3 * tl + 1], gamma = (A)coef[3 * tl + 2];
   const size_t rowbase = (size_t)tl * g.Vs;
-  Cx<A> res[3][NC];
+  const int yz = ms / g.L, x = ms - yz * g.L, z = yz / g.L, y = yz - z * g.L;
+  const size_t s = (size_t)(t0 + tl) * g.Vs + ms;
+  Cx<double> acc[3];
 #pragma unroll
-  for (int a = 0; a < 3; a++)
+  for (int a = 0; a < 3; a++) acc[a] = 6.0 * in[((rowbase + ms) * 3 + a) * m + j0];
 #pragma unroll
-    for (int c = 0; c < NC; c++) res[a][c] = cx<A>(0, 0);
-  if (in) {
-    const int yz = ms / g.L, x = ms - yz * g.L, z = yz / g.L, y = yz - z * g.L;
-    const size_t s = (size_t)(t0 + tl) * g.Vs + ms;
-    Cx<A> acc[3][NC];
+  for (int k = 0; k < 3; k++) {
+    int xf = x, yf = y, zf = z, xb = x, yb = y, zb = z;
+    if (k == 0) { xf = x + 1 == g.L ? 0 : x + 1; xb = x == 0 ? g.L - 1 : x - 1; }
+    else if (k == 1) { yf = y + 1 == g.L ? 0 : y + 1; yb = y == 0 ? g.L - 1 : y - 1; }
+    else { zf = z + 1 == g.L ? 0 : z + 1; zb = z == 0 ? g.L - 1 : z - 1; }
+    const int mf = xf + g.L * (yf + g.L * zf), mb = xb + g.L * (yb + g.L * zb);
+    Cx<double> uf[3][3], ub[3][3], vf[3], vb[3];
+    load_link3(U, k, s, (size_t)g.V, uf);
+    load_link3(U, k, (size_t)(t0 + tl) * g.Vs + mb, (size_t)g.V, ub);
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      Cx<R> v[NC];
-      ld_cols<NC>(in + ((rowbase + ms) * 3 + a) * m + j0, v);   // own term, kept for beta
-#pragma unroll
-      for (int c = 0; c < NC; c++) {
-        res[a][c] = to_a<A>(v[c]);
-        acc[a][c] = (A)6 * res[a][c];
-      }
+      vf[a] = in[((rowbase + mf) * 3 + a) * m + j0];
+      vb[a] = in[((rowbase + mb) * 3 + a) * m + j0];
     }
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-      int xf = x, yf = y, zf = z, xb = x, yb = y, zb = z;
-      if (k == 0) { xf = x + 1 == g.L ? 0 : x + 1; xb = x == 0 ? g.L - 1 : x - 1; }
-      else if (k == 1) { yf = y + 1 == g.L ? 0 : y + 1; yb = y == 0 ? g.L - 1 : y - 1; }
-      else { zf = z + 1 == g.L ? 0 : z + 1; zb = z == 0 ? g.L - 1 : z - 1; }
-      const int mf = xf + g.L * (yf + g.L * zf), mb = xb + g.L * (yb + g.L * zb);
-      Cx<A> uf[3][3], ub[3][3];
-      load_link3(U, k, s, (size_t)g.V, uf);
-      load_link3(U, k, (size_t)(t0 + tl) * g.Vs + mb, (size_t)g.V, ub);
-      Cx<R> vf[3][NC], vb[3][NC];
+    for (int a = 0; a < 3; a++) {
+      Cx<double> h = cx<double>(0, 0);
 #pragma unroll
-      for (int a = 0; a < 3; a++) {
-        ld_cols<NC>(in + ((rowbase + mf) * 3 + a) * m + j0, vf[a]);
-        ld_cols<NC>(in + ((rowbase + mb) * 3 + a) * m + j0, vb[a]);
+      for (int b = 0; b < 3; b++) {
+        fma_acc(h, uf[a][b], vf[b]);
+        fma_conj_acc(h, ub[b][a], vb[b]);
       }
-#pragma unroll
-      for (int c = 0; c < NC; c++)
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-          Cx<A> h = cx<A>(0, 0);
-#pragma unroll
-          for (int b = 0; b < 3; b++) {
-            fma_acc(h, uf[a][b], to_a<A>(vf[b][c]));
-            fma_conj_acc(h, ub[b][a], to_a<A>(vb[b][c]));
-          }
-          acc[a][c] = acc[a][c] - h;
-        }
+      acc[a] = acc[a] - h;
     }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; a++) out[((rowbase + ms) * 3 + a) * m + j0] = acc[a];
+}
+
+// FP32: out = alpha_t (A in) + beta_t in + gamma_t prev + alpha_t s[t][j] rin (prev and rin
+// may be nullptr).
+// Two columns per thread (m is even, so a pair is 16-byte aligned), marching along z: a
+// thread keeps its column's sites z, z + 1 and the backward product U_z(z)^dag v(z) in
+// registers, so every value is loaded once along z and each z link once; a block covers a
+// patch of px x py sites of a plane, whose x and y neighbours meet in L1.  The plain form
+// (k_lap: a row of sites per block) moved 6.5 vectors per application from L2 to the SMs
+// (0.215 ms for a block of 16^3 x 32 with 64 columns, 2.12 for 24^3 x 48 with 128); this
+// one moves about 3.5 and takes 0.196 and 1.87 ms, bound by instruction issue (some 800
+// per site and column pair, a sixth of them rebuilding link rows; DRAM floor 0.09, 0.92).
+// Block: pw column pairs x (px py) sites; grid: (patches of a plane x z segments x column
+// groups, timeslices).
+struct LapTiling {
+  int pw, px, py, groups, nx, ny, nz, zlen;
+};
+__global__ void __launch_bounds__(256, 2) k_lap_z(Geom g, int t0, int m, LapTiling L, const float4* __restrict__ U,
+                                                  const Cx<float>* __restrict__ in, const Cx<float>* __restrict__ prev,
+                                                  const Cx<float>* __restrict__ rin, const double* __restrict__ scol,
+                                                  Cx<float>* __restrict__ out, const double* __restrict__ coef) {
+  const int tl = blockIdx.y;
+  int b = blockIdx.x;
+  const int grp = b % L.groups;
+  b /= L.groups;
+  const int bx = b % L.nx;
+  b /= L.nx;
+  const int by = b % L.ny, bz = b / L.ny;
+  const int site = threadIdx.x / L.pw, pair = grp * L.pw + (threadIdx.x - site * L.pw);
+  const int x = bx * L.px + site % L.px, y = by * L.py + site / L.px;
+  if (site >= L.px * L.py || x >= g.L || y >= g.L || 2 * pair >= m) return;
+  const int z0 = bz * L.zlen, z1 = min(g.L, z0 + L.zlen);
+  const int j0 = 2 * pair, plane = g.L * g.L;
+  const float alpha = (float)coef[3 * tl], beta = (float)coef[3 * tl + 1], gamma = (float)coef[3 * tl + 2];
+  const size_t row0 = (size_t)tl * g.Vs;                   // first site of the block's timeslice
+  const size_t s0 = (size_t)(t0 + tl) * g.Vs;              // ... and of the links'
+  const int xf = x + 1 == g.L ? 0 : x + 1, xb = x == 0 ? g.L - 1 : x - 1;
+  const int yf = y + 1 == g.L ? 0 : y + 1, yb = y == 0 ? g.L - 1 : y - 1;
+  const int o = x + g.L * y, oxb = xb + g.L * y, oyb = x + g.L * yb;
+  const int nbr[4] = {xf + g.L * y, oxb, x + g.L * yf, oyb};
+  float fr0 = 0, fr1 = 0;
+  if (rin) {
+    fr0 = alpha * (float)scol[(size_t)tl * m + j0];
+    fr1 = alpha * (float)scol[(size_t)tl * m + j0 + 1];
+  }
+  const auto load = [&](const Cx<float>* p, int ms, Cx<float>(&v)[3][2]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) ld_cols<2>(p + ((row0 + ms) * 3 + a) * m + j0, v[a]);
+  };
+  // w = U^dag v
+  const auto dag_mul = [&](const Cx<float>(&u)[3][3], const Cx<float>(&v)[3][2], Cx<float>(&w)[3][2]) {
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
-      for (int c = 0; c < NC; c++) res[a][c] = alpha * acc[a][c] + beta * res[a][c];
+      for (int c = 0; c < 2; c++) {
+        w[a][c] = cx<float>(0, 0);
+#pragma unroll
+        for (int q = 0; q < 3; q++) fma_conj_acc(w[a][c], u[q][a], v[q][c]);
+      }
+  };
+  Cx<float> cur[3][2], wz[3][2];
+  {
+    const int zb = z0 == 0 ? g.L - 1 : z0 - 1;
+    Cx<float> u[3][3], v[3][2];
+    load_link3(U, 2, s0 + o + (size_t)plane * zb, (size_t)g.V, u);
+    load(in, o + plane * zb, v);
+    dag_mul(u, v, wz);
+    load(in, o + plane * z0, cur);
   }
+  for (int z = z0; z < z1; z++) {
+    const int zo = plane * z, zf = plane * (z + 1 == g.L ? 0 : z + 1);
+    Cx<float> nxt[3][2], acc[3][2];
+    load(in, o + zf, nxt);
+    {
+      Cx<float> u[3][3], w[3][2];
+      load_link3(U, 2, s0 + o + zo, (size_t)g.V, u);
 #pragma unroll
-  for (int a = 0; a < 3; a++) {
-    const size_t idx = ((rowbase + ms) * 3 + a) * m + j0;
-    if (prev) {
-      Cx<R> pv[NC];
-      ld_cols<NC>(prev + idx, pv);
+      for (int a = 0; a < 3; a++)
 #pragma unroll
-      for (int c = 0; c < NC; c++) res[a][c] = res[a][c] + gamma * to_a<A>(pv[c]);
+        for (int c = 0; c < 2; c++) {
+          Cx<float> h = wz[a][c];
+#pragma unroll
+          for (int q = 0; q < 3; q++) fma_acc(h, u[a][q], nxt[q][c]);
+          acc[a][c] = 6.f * cur[a][c] - h;
+        }
+      dag_mul(u, cur, w);
+#pragma unroll
+      for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int c = 0; c < 2; c++) wz[a][c] = w[a][c];
     }
-    if (rin) {
-      Cx<float> rv[NC];
-      ld_cols<NC>(rin + idx, rv);
 #pragma unroll
-      for (int c = 0; c < NC; c++) {
-        const A f = alpha * (A)scol[(size_t)tl * m + j0 + c];
-        res[a][c] = res[a][c] + f * cx<A>((A)rv[c].re, (A)rv[c].im);
+    for (int k = 0; k < 2; k++) {
+      Cx<float> u[3][3], v[3][2], w[3][2];
+      load_link3(U, k, s0 + o + zo, (size_t)g.V, u);
+      load(in, nbr[2 * k] + zo, v);
+#pragma unroll
+      for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          Cx<float> h = cx<float>(0, 0);
+#pragma unroll
+          for (int q = 0; q < 3; q++) fma_acc(h, u[a][q], v[q][c]);
+          acc[a][c] = acc[a][c] - h;
+        }
+      load_link3(U, k, s0 + (k == 0 ? oxb : oyb) + zo, (size_t)g.V, u);
+      load(in, nbr[2 * k + 1] + zo, v);
+      dag_mul(u, v, w);
+#pragma unroll
+      for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int c = 0; c < 2; c++) acc[a][c] = acc[a][c] - w[a][c];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      const size_t idx = ((row0 + o + zo) * 3 + a) * m + j0;
+      Cx<float> r[2];
+#pragma unroll
+      for (int c = 0; c < 2; c++) r[c] = alpha * acc[a][c] + beta * cur[a][c];
+      if (prev) {
+        Cx<float> pv[2];
+        ld_cols<2>(prev + idx, pv);
+#pragma unroll
+        for (int c = 0; c < 2; c++) r[c] = r[c] + gamma * pv[c];
+      }
+      if (rin) {
+        Cx<float> rv[2];
+        ld_cols<2>(rin + idx, rv);
+        r[0] = r[0] + fr0 * rv[0];
+        r[1] = r[1] + fr1 * rv[1];
+      }
+      st_cols<2>(out + idx, r);
+#pragma unroll
+      for (int c = 0; c < 2; c++) cur[a][c] = nxt[a][c];
+    }
+  }
+}
+
+// tiling of k_lap_z: at most 32 column pairs per block; the patch that loads the fewest
+// halo sites and idle threads; z segments so that the grid fills the GPU a few times
+static LapTiling lap_tiling(int L, int m, int Tn) {
+  LapTiling best{};
+  const int mg = m / 2, groups = (mg + 31) / 32, pw = (mg + groups - 1) / groups;
+  double cost = 1e300;
+  for (int px = 1; px <= 8; px++)
+    for (int py = 1; py <= px; py++) {
+      if (px * py * pw > 256) continue;
+      const int nx = (L + px - 1) / px, ny = (L + py - 1) / py;
+      const double loads = (double)(px * py + 2 * px + 2 * py) * nx * ny, threads = 256.0 / pw * nx * ny;
+      const double c = loads + threads;
+      if (c < cost) {
+        cost = c;
+        best = LapTiling{pw, px, py, groups, nx, ny, 1, L};
       }
     }
-    Cx<R> o[NC];
-#pragma unroll
-    for (int c = 0; c < NC; c++) o[c] = to_s<R>(res[a][c]);
-    st_cols<NC>(out + idx, o);
-  }
+  const long blocks = (long)best.nx * best.ny * groups * Tn;
+  // each segment reloads two planes' worth at its ends: at least 4 planes
+  best.nz = (int)std::max<long>(1, std::min<long>(L / 4, (4 * 304 + blocks - 1) / blocks));
+  best.zlen = (L + best.nz - 1) / best.nz;
+  best.nz = (L + best.zlen - 1) / best.zlen;
+  return best;
 }
 
 // Gram partials: part[t][split][i][j] = sum_{k in chunk} conj(X_t[k][i]) Y_t[k][j]
@@ -330,18 +426,25 @@ __global__ void __launch_bounds__(256) k_rotate(const Cx<R>* __restrict__ X, con
     }
 }
 
-// residual norms res[t][j] = ||W_j - theta_j X_j||; optionally R = W - X Theta stored in FP32
+// residual norms res[t][j] = ||W_j - theta_j X_j||; optionally R = W - X Theta stored in
+// FP32.  Bound by memory: the rows of a timeslice are shared out over blockIdx.z (one
+// block per 32 columns and timeslice kept 64 of 152 SMs busy: 0.51 ms for an FP32 block
+// of 16^3 x 32, 64 columns, now
+// 0.07), with the partial sums in part[t][z][j].
+constexpr int kResidSplit = 24;
 template <class R>
 __global__ void __launch_bounds__(256) k_resid(const Cx<R>* __restrict__ X, const Cx<R>* __restrict__ W,
-                                               const double* __restrict__ theta, int n, int m, double* res,
+                                               const double* __restrict__ theta, int n, int m, double* part,
                                                Cx<float>* Rout) {
   const int t = blockIdx.y;
   const int j = blockIdx.x * 32 + (threadIdx.x & 31), lane = threadIdx.x >> 5;
+  const int chunk = (n + gridDim.z - 1) / gridDim.z, k0 = blockIdx.z * chunk, k1 = min(n, k0 + chunk);
   R s = 0;   // in the block's precision (FP64 arithmetic is scarce next to an FP32 block)
   if (j < m) {
     const R th = (R)theta[(size_t)t * m + j];
     const size_t base = (size_t)t * n * m;
-    for (int k = lane; k < n; k += 8) {
+#pragma unroll 4
+    for (int k = k0 + lane; k < k1; k += 8) {
       const size_t idx = base + (size_t)k * m + j;
       const Cx<R> w = W[idx], x = X[idx];
       const R dx = w.re - th * x.re, dy = w.im - th * x.im;
@@ -355,8 +458,16 @@ __global__ void __launch_bounds__(256) k_resid(const Cx<R>* __restrict__ X, cons
   if (lane == 0 && j < m) {
     double tot = 0;
     for (int q = 0; q < 8; q++) tot += red[q][threadIdx.x];
-    res[(size_t)t * m + j] = sqrt(tot);
+    part[((size_t)t * gridDim.z + blockIdx.z) * m + j] = tot;
   }
+}
+__global__ void k_resid_sum(const double* __restrict__ part, int splits, int m, int total, double* res) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const int t = e / m, j = e - t * m;
+  double s = 0;
+  for (int z = 0; z < splits; z++) s += part[((size_t)t * splits + z) * m + j];
+  res[e] = sqrt(s);
 }
 
 // Y64 = X64 + E32 / s[t][j]  (phase B filter output, column j divided by s_d(theta_j)).
@@ -377,6 +488,16 @@ __global__ void k_combine(const Cx<double>* __restrict__ X, const Cx<float>* __r
   // a vanishing s_d (possible only when the cut is pushed below 12 on a block that
   // spans nearly the whole timeslice) keeps the unscaled column
   Y[e] = fabs(sj) > 1e-280 ? X[e] + (1.0 / sj) * ed : sj * X[e] + ed;
+}
+
+// first step of phase B's filter: out = alpha_t s[t][j] rin
+__global__ void k_filter_start(const Cx<float>* __restrict__ rin, const double* __restrict__ scol,
+                               const double* __restrict__ coef, size_t nm, int m, size_t total, Cx<float>* out) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const unsigned e32 = (unsigned)e;
+  const unsigned t = e32 / (unsigned)nm;
+  out[e] = ((float)coef[3 * t] * (float)scol[t * m + e32 % (unsigned)m]) * rin[e];
 }
 
 template <class A, class B> __global__ void k_convert_block(const Cx<A>* in, Cx<B>* out, size_t total) {
@@ -500,16 +621,15 @@ static dlma_status lap(Eig& E, const Cx<R>* in, const Cx<R>* prev, const Cx<floa
   if (total >= (1ull << 31)) return set_err(ctx, DLMA_ERR_INVALID_ARG, "eigensolver block above 2^31 entries");
   phase(E, kPhMatvec);
   // m is even; FP32: two columns per thread (one 128-bit access per pair, links
-  // rebuilt once per pair); FP64 is bound by its arithmetic and keeps one
-  // (measured alternatives: four FP32 columns per thread, 145 registers, and a
-  // double-float FP64 matvec, 170 registers and a split of every loaded value,
-  // were both slower)
+  // rebuilt once per pair); FP64 is bound by its arithmetic and keeps one (a
+  // double-float FP64 matvec, 170 registers and a split of every loaded value, was
+  // slower)
   if constexpr (sizeof(R) == 4) {
-    k_lap<R, R, 2><<<(unsigned)((total / 2 + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->g, E.t0, E.Tn, E.m, links<R>(ctx), in, prev, rin, scol, out, coef);
+    const LapTiling t = lap_tiling(ctx->g.L, E.m, E.Tn);
+    k_lap_z<<<dim3((unsigned)(t.nx * t.ny * t.nz * t.groups), E.Tn), 256, 0, ctx->stream>>>(
+        ctx->g, E.t0, E.m, t, links<R>(ctx), in, prev, rin, scol, out, coef);
   } else {
-    k_lap<R, R, 1><<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(ctx->g, E.t0, E.Tn, E.m, links<R>(ctx), in,
-                                                                             prev, rin, scol, out, coef);
+    k_lap<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(ctx->g, E.t0, E.Tn, E.m, links<R>(ctx), in, out);
   }
   CHECK_LAUNCH();
   return DLMA_OK;
@@ -573,6 +693,19 @@ template <class T> static dlma_status small_rr(Eig& E) {
   return DLMA_OK;
 }
 
+template <class R> static dlma_status resid(Eig& E, const Cx<R>* X, const Cx<R>* W, Cx<float>* Rout) {
+  dlma_ctx* ctx = E.ctx;
+  phase(E, kPhOrtho);
+  // partial sums in the Gram partials' work area, which holds 2 m^2 doubles per timeslice
+  const int splits = std::max(1, std::min(std::min(kResidSplit, E.n / 64), 2 * E.m));
+  k_resid<R><<<dim3((E.m + 31) / 32, E.Tn, splits), 256, 0, ctx->stream>>>(X, W, E.theta, E.n, E.m, (double*)E.part,
+                                                                          Rout);
+  CHECK_LAUNCH();
+  k_resid_sum<<<(E.m * E.Tn + 127) / 128, 128, 0, ctx->stream>>>((const double*)E.part, splits, E.m, E.m * E.Tn, E.res);
+  CHECK_LAUNCH();
+  return DLMA_OK;
+}
+
 // Rayleigh-Ritz of the block Y: W = A Y, then X <- Y C, AX <- W C, residuals (and R = AX - X Theta in FP32)
 template <class R>
 static dlma_status rayleigh_ritz(Eig& E, Cx<R>* Y, Cx<R>* W, Cx<R>* Xout, Cx<R>* AXout, Cx<float>* Rout,
@@ -583,11 +716,7 @@ static dlma_status rayleigh_ritz(Eig& E, Cx<R>* Y, Cx<R>* W, Cx<R>* Xout, Cx<R>*
   TRY(small_rr<R>(E));
   TRY(rotate<R>(E, Y, Xout));
   TRY(rotate<R>(E, W, AXout));
-  dlma_ctx* ctx = E.ctx;
-  phase(E, kPhOrtho);
-  k_resid<R><<<dim3((E.m + 31) / 32, E.Tn), 256, 0, ctx->stream>>>(Xout, AXout, E.theta, E.n, E.m, E.res, Rout);
-  CHECK_LAUNCH();
-  return DLMA_OK;
+  return resid<R>(E, Xout, AXout, Rout);
 }
 
 // fetch theta / residuals; returns the worst relative residual over the wanted pairs.
@@ -693,6 +822,12 @@ static void cheb_coefficients(Eig& E, int d, std::vector<double>& hc, std::vecto
   }
 }
 
+// complex multiply-adds (n m^2 Tn) from which a phase-B product takes the tensor cores
+// instead of double-float (eigensolve, double-float against tensor cores: 18.6 and 17.4 ms
+// on 10^3 x 18 with 40 columns, 9e7; 110 and 96 ms on 16^3 x 32 with 64, 2e9; 1277 and
+// 957 ms on 24^3 x 48 with 128; equal at 2.5e7, 8^3 x 16 with 32)
+constexpr double kTcWork = 5.0e7;
+
 static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, double* lam_out,
                              Cx<double>** Xres, int* m_out, int* iters_out, PhaseTimer* pt) {
   Eig E;
@@ -794,12 +929,9 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   // The FP64 blocks' Gram matrices and rotations run in double-float on the FP32
   // units when the tolerance leaves room for its ~2^-46 rounding.
   E.df = ctx->df_eigs && tol >= 1e-11;
-  // products of many multiply-adds (n m^2 per timeslice) take the tensor cores
-  // (16^3 x 32: orthogonalisation 250 -> 200 ms at N = 64, 617 -> 533 ms at N = 128;
-  // 32^3 x 64, N = 96: 5.4 -> 4.4 s); small ones stay in double-float, where the
-  // tensor-core launches do not fill the GPU (16^3 x 32, N = 32: 65 against 70 ms).
-  // DLMA_EIGS_TC=1 / 0 forces either.
-  E.tc = E.df && (double)E.n * E.m * E.m * E.Tn >= 4.0e9;
+  // (and from kTcWork multiply-adds per product on the tensor cores; DLMA_EIGS_TC=1 / 0
+  // forces either)
+  E.tc = E.df && (double)E.n * E.m * E.m * E.Tn >= kTcWork;
   if (const char* e = getenv("DLMA_EIGS_TC")) E.tc = E.df && atoi(e) == 1;
   Cx<double> *X64 = E.D0, *W64 = E.D1, *Y64 = E.D2;
   // phase A's last Ritz pairs were not fetched, or hold refilled (random) columns
@@ -824,9 +956,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
     TRY(rayleigh_ritz<double>(E, Y64, W64, X64, Y64, R32, plain));
   } else {
     TRY(lap<double>(E, X64, nullptr, nullptr, nullptr, Y64, plain));
-    phase(E, kPhOrtho);
-    k_resid<double><<<dim3((m + 31) / 32, Tn), 256, 0, ctx->stream>>>(X64, Y64, E.theta, E.n, m, E.res, R32);
-    CHECK_LAUNCH();
+    TRY(resid<double>(E, X64, Y64, R32));
   }
   bool conv = false;
   int itB = 0;
@@ -841,7 +971,10 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
     CU(cudaMemcpyAsync(E.scol, hs.data(), sizeof(double) * nscol, cudaMemcpyHostToDevice, ctx->stream));
     // E_1 = a_1 R s_0 ; E_{k+1} = a_k A E_k + b_k E_k + c_k E_{k-1} + a_k R s_k
     Cx<float>*em = nullptr, *ec = Ebuf[0], *en = Ebuf[1], *spare = Ebuf[2];
-    TRY(lap<float>(E, nullptr, nullptr, R32, E.scol, ec, E.coef));
+    phase(E, kPhMatvec);
+    k_filter_start<<<(unsigned)((E.blk + 255) / 256), 256, 0, ctx->stream>>>(R32, E.scol, E.coef, (size_t)E.n * m, m,
+                                                                             E.blk, ec);
+    CHECK_LAUNCH();
     for (int k = 2; k <= dB; k++) {
       TRY(lap<float>(E, ec, em, R32, E.scol + (size_t)(k - 1) * Tn * m, en, E.coef + (size_t)(k - 1) * 3 * Tn));
       Cx<float>* t = em ? em : spare;
@@ -861,9 +994,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
     TRY(small_rr<double>(E));
     TRY(rotate<double>(E, Y64, X64));
     TRY(lap<double>(E, X64, nullptr, nullptr, nullptr, Y64, plain));   // A X, fresh (cheaper than W C)
-    phase(E, kPhOrtho);
-    k_resid<double><<<dim3((m + 31) / 32, Tn), 256, 0, ctx->stream>>>(X64, Y64, E.theta, E.n, m, E.res, R32);
-    CHECK_LAUNCH();
+    TRY(resid<double>(E, X64, Y64, R32));
   }
   if (!conv) {
     TRY(fetch<double>(E, &worst, X64));
