@@ -355,13 +355,94 @@ __global__ void __launch_bounds__(256) k_gram(const Cx<R>* __restrict__ X, const
     }
 }
 
-__global__ void k_gram_reduce(const double2* part, int nsplit, int m, int Tn, int herm, double2* G) {
+// FP32 blocks: 64 x 64 output tiles, 4 x 4 entries per thread, so that 64 multiply-adds
+// share four 128-bit shared loads (32 x 32 tiles with 2 x 2 entries were bound by shared
+// memory: 6.8 ms for 24^3 x 48 with 128 columns, now 3.9; FP32 floor 2.6).  The next
+// slab of 16 rows is loaded into registers while the current one is used.
+constexpr int FT = 64, FK = 16;
+__device__ __forceinline__ void ld4(const Cx<float>* __restrict__ p, bool on, int room, Cx<float> (&v)[4]) {
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const float4 e = on && 2 * h < room ? __ldg((const float4*)(p + 2 * h)) : make_float4(0, 0, 0, 0);
+    v[2 * h] = cx<float>(e.x, e.y);
+    v[2 * h + 1] = cx<float>(e.z, e.w);
+  }
+}
+__device__ __forceinline__ void sh4(const Cx<float>* p, Cx<float> (&v)[4]) {
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const float4 e = *(const float4*)(p + 2 * h);
+    v[2 * h] = cx<float>(e.x, e.y);
+    v[2 * h + 1] = cx<float>(e.z, e.w);
+  }
+}
+__device__ __forceinline__ void st4(Cx<float>* p, const Cx<float> (&v)[4]) {
+#pragma unroll
+  for (int h = 0; h < 2; h++)
+    *(float4*)(p + 2 * h) = make_float4(v[2 * h].re, v[2 * h].im, v[2 * h + 1].re, v[2 * h + 1].im);
+}
+__global__ void __launch_bounds__(256) k_gram_f(const Cx<float>* __restrict__ X, const Cx<float>* __restrict__ Y, int n,
+                                                int m, int nsplit, int herm, double2* part) {
+  __shared__ __align__(16) Cx<float> xs[2][FK][FT], ys[2][FK][FT];
+  const int tiles_j = (m + FT - 1) / FT;
+  int ti = blockIdx.x / tiles_j, tj = blockIdx.x % tiles_j;
+  if (herm) {                 // blockIdx.x enumerates the pairs ti <= tj row by row
+    int b = blockIdx.x;
+    ti = 0;
+    while (b >= tiles_j - ti) { b -= tiles_j - ti; ti++; }
+    tj = ti + b;
+  }
+  const int i0 = ti * FT, j0 = tj * FT;
+  const int split = blockIdx.y, t = blockIdx.z;
+  const int chunk = (n + nsplit - 1) / nsplit;
+  const int k0 = split * chunk, k1 = min(n, k0 + chunk);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const Cx<float>* Xt = X + (size_t)t * n * m + i0 + 4 * tx;
+  const Cx<float>* Yt = Y + (size_t)t * n * m + j0 + 4 * tx;
+  const int rx = m - i0 - 4 * tx, ry = m - j0 - 4 * tx;     // columns left (m is even)
+  Cx<float> acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) acc[a][b] = cx<float>(0, 0);
+  Cx<float> vx[4], vy[4];
+  ld4(Xt + (size_t)(k0 + ty) * m, k0 + ty < k1, rx, vx);
+  ld4(Yt + (size_t)(k0 + ty) * m, k0 + ty < k1, ry, vy);
+  for (int kb = k0, st = 0; kb < k1; kb += FK, st ^= 1) {
+    st4(&xs[st][ty][4 * tx], vx);
+    st4(&ys[st][ty][4 * tx], vy);
+    __syncthreads();
+    const int kn = kb + FK + ty;
+    ld4(Xt + (size_t)kn * m, kn < k1, rx, vx);
+    ld4(Yt + (size_t)kn * m, kn < k1, ry, vy);
+#pragma unroll
+    for (int r = 0; r < FK; r++) {
+      Cx<float> xv[4], yv[4];
+      sh4(&xs[st][r][4 * ty], xv);
+      sh4(&ys[st][r][4 * tx], yv);
+#pragma unroll
+      for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) fma_conj_acc(acc[a][b], xv[a], yv[b]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      const int i = i0 + 4 * ty + a, j = j0 + 4 * tx + b;
+      if (i < m && j < m)
+        part[(((size_t)t * nsplit + split) * m + i) * m + j] = make_double2((double)acc[a][b].re, (double)acc[a][b].im);
+    }
+}
+
+__global__ void k_gram_reduce(const double2* part, int nsplit, int m, int Tn, int herm, int tile, double2* G) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t per = (size_t)m * m;
   if (e >= per * Tn) return;
   const size_t t = e / per;
   const int i = (int)((e % per) / m), j = (int)(e % m);
-  const bool mirror = herm && (i / GT) > (j / GT);    // tile below the diagonal: conj of (j, i)
+  const bool mirror = herm && (i / tile) > (j / tile);    // tile below the diagonal: conj of (j, i)
   const size_t ij = mirror ? (size_t)j * m + i : (size_t)i * m + j;
   double2 s = make_double2(0, 0);
   for (int q = 0; q < nsplit; q++) {
@@ -424,6 +505,63 @@ __global__ void __launch_bounds__(256) k_rotate(const Cx<R>* __restrict__ X, con
       const int k = k0 + tr + 16 * a, j = j0 + tc + 16 * b;
       if (k < n && j < m) Zt[(size_t)k * m + j] = to_s<R>(acc[a][b]);
     }
+}
+
+// FP32 blocks: the same 64 x 64 tiles as k_gram_f (5.95 ms for 24^3 x 48 with 128 columns
+// with scalar shared loads, now 5.8; FP32 floor 3.5)
+__global__ void __launch_bounds__(256) k_rotate_f(const Cx<float>* __restrict__ X, const double2* __restrict__ Cm, int n,
+                                                  int m, Cx<float>* __restrict__ Z) {
+  __shared__ __align__(16) Cx<float> xs[2][FK][FT + 2], cs[2][FK][FT];     // xs transposed: [l][k]
+  const int t = blockIdx.z, k0 = blockIdx.x * FT, j0 = blockIdx.y * FT;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int xr = threadIdx.x >> 2, xl = (threadIdx.x & 3) * 4;             // this thread's row and columns of X
+  const Cx<float>* Xt = X + ((size_t)t * n + k0 + xr) * m + xl;
+  const double2* C = Cm + (size_t)t * m * m + j0 + 4 * tx;
+  const bool xon = k0 + xr < n;
+  Cx<float> acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) acc[a][b] = cx<float>(0, 0);
+  Cx<float> vx[4], vc[4];
+  const auto fetch = [&](int l0) {
+    ld4(Xt + l0, xon, m - l0 - xl, vx);
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      const bool on = l0 + ty < m && j0 + 4 * tx + b < m;
+      const double2 e = on ? C[(size_t)(l0 + ty) * m + b] : make_double2(0, 0);
+      vc[b] = cx<float>((float)e.x, (float)e.y);
+    }
+  };
+  fetch(0);
+  for (int l0 = 0, st = 0; l0 < m; l0 += FK, st ^= 1) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) xs[st][xl + q][xr] = vx[q];
+    st4(&cs[st][ty][4 * tx], vc);
+    __syncthreads();
+    fetch(l0 + FK);
+#pragma unroll
+    for (int l = 0; l < FK; l++) {
+      Cx<float> xv[4], cv[4];
+      sh4(&xs[st][l][4 * ty], xv);
+      sh4(&cs[st][l][4 * tx], cv);
+#pragma unroll
+      for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) fma_acc(acc[a][b], xv[a], cv[b]);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const int k = k0 + 4 * ty + a;
+    if (k >= n) continue;
+    Cx<float>* z = Z + ((size_t)t * n + k) * m + j0 + 4 * tx;
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+      if (j0 + 4 * tx + 2 * h < m)
+        *(float4*)(z + 2 * h) = make_float4(acc[a][2 * h].re, acc[a][2 * h].im, acc[a][2 * h + 1].re,
+                                            acc[a][2 * h + 1].im);
+  }
 }
 
 // residual norms res[t][j] = ||W_j - theta_j X_j||; optionally R = W - X Theta stored in
@@ -585,7 +723,7 @@ __global__ void k_lap_canonical(Geom g, const double2* __restrict__ U3, const do
 // ---------------------------------------------------------------------------
 struct Eig {
   dlma_ctx* ctx;
-  int t0, Tn, N, m, n, nsplit, degree;
+  int t0, Tn, N, m, n, nsplit, nsplit_f, degree;   // row splits of the Gram products, FP64 and FP32 blocks
   int df = 0;   // phase B: Gram matrices and rotations in double-float (tol >= 1e-11)
   int tc = 0;   // phase B: Gram matrices and rotations on the tensor cores (tcproj.cu)
   size_t blk;                    // m * Tn * n complex entries per block
@@ -649,11 +787,15 @@ template <class R> static dlma_status gram(Eig& E, const Cx<R>* X, const Cx<R>* 
     if (E.df) k_gram<R, df><<<grid, 256, 0, ctx->stream>>>(X, Y, E.n, E.m, E.nsplit, herm, E.part);
     else k_gram<R, R><<<grid, 256, 0, ctx->stream>>>(X, Y, E.n, E.m, E.nsplit, herm, E.part);
   } else {
-    k_gram<R, R><<<grid, 256, 0, ctx->stream>>>(X, Y, E.n, E.m, E.nsplit, herm, E.part);
+    const int tf = (E.m + FT - 1) / FT;
+    k_gram_f<<<dim3(herm ? tf * (tf + 1) / 2 : tf * tf, E.nsplit_f, E.Tn), 256, 0, ctx->stream>>>(
+        X, Y, E.n, E.m, E.nsplit_f, herm, E.part);
   }
   CHECK_LAUNCH();
   const size_t tot = (size_t)E.m * E.m * E.Tn;
-  k_gram_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(E.part, E.nsplit, E.m, E.Tn, herm, out);
+  const bool f32 = sizeof(R) == 4;
+  k_gram_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(E.part, f32 ? E.nsplit_f : E.nsplit, E.m, E.Tn,
+                                                                       herm, f32 ? FT : GT, out);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
@@ -669,7 +811,7 @@ template <class R> static dlma_status rotate(Eig& E, const Cx<R>* X, Cx<R>* Z) {
     if (E.df) k_rotate<R, df><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
     else k_rotate<R, R><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
   } else {
-    k_rotate<R, R><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
+    k_rotate_f<<<dim3((E.n + FT - 1) / FT, (E.m + FT - 1) / FT, E.Tn), 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
   }
   CHECK_LAUNCH();
   return DLMA_OK;
@@ -850,6 +992,11 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   if (E.blk >= (1ull << 31)) return set_err(ctx, DLMA_ERR_INVALID_ARG, "eigensolver block above 2^31 entries");
   E.nsplit = std::max(1, std::min(64, (4 * 152) / std::max(1, Tn * ((m + GT - 1) / GT) * ((m + GT - 1) / GT))));
   E.nsplit = std::min(E.nsplit, std::max(1, E.n / 256));
+  {
+    const int tf = (m + FT - 1) / FT;
+    E.nsplit_f = std::max(1, std::min(64, (4 * 152) / std::max(1, Tn * tf * (tf + 1) / 2)));
+    E.nsplit_f = std::min(E.nsplit_f, std::max(1, E.n / 256));
+  }
   TRY(workT(ctx, WS_EIG_X, E.blk * 2, &E.F0));
   E.F1 = E.F0 + E.blk;
   TRY(workT(ctx, WS_EIG_Y, E.blk * 2, &E.F2));
@@ -861,7 +1008,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   TRY(workT(ctx, WS_EIG_G, 3 * mm * Tn, &E.G));
   E.H = E.G + mm * Tn;
   E.C = E.H + mm * Tn;
-  TRY(workT(ctx, WS_EIG_PART, (size_t)E.nsplit * mm * Tn, &E.part));
+  TRY(workT(ctx, WS_EIG_PART, (size_t)std::max(E.nsplit, E.nsplit_f) * mm * Tn, &E.part));
   TRY(workT(ctx, WS_EIG_S, 3 * (size_t)m * (m + 1) * Tn, &E.gwork));
   const int d = E.degree;
   double* aux;
