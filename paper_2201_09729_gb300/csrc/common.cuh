@@ -27,6 +27,13 @@ template <class R> __host__ __device__ __forceinline__ Cx<R> operator*(R s, Cx<R
 template <class R> __host__ __device__ __forceinline__ Cx<R> conj(Cx<R> a) { return cx<R>(a.re, -a.im); }
 // i * a
 template <class R> __host__ __device__ __forceinline__ Cx<R> mul_i(Cx<R> a) { return cx<R>(-a.im, a.re); }
+// a + s b and a + s i b for a real s
+template <class S, class R> __device__ __forceinline__ Cx<R> add_s(Cx<R> a, S s, Cx<R> b) {
+  return cx<R>(fma((R)s, b.re, a.re), fma((R)s, b.im, a.im));
+}
+template <class S, class R> __device__ __forceinline__ Cx<R> add_si(Cx<R> a, S s, Cx<R> b) {
+  return cx<R>(fma((R)-s, b.im, a.re), fma((R)s, b.re, a.im));
+}
 // a + i b, a - i b
 template <class R> __host__ __device__ __forceinline__ Cx<R> add_i(Cx<R> a, Cx<R> b) { return cx<R>(a.re - b.im, a.im + b.re); }
 template <class R> __host__ __device__ __forceinline__ Cx<R> sub_i(Cx<R> a, Cx<R> b) { return cx<R>(a.re + b.im, a.im - b.re); }
@@ -160,7 +167,7 @@ struct dlma_ctx {
   uint4* U16a = nullptr;    // [2][4][Vh]     halves 0..7 of rows 0, 1
   uint2* U16b = nullptr;    // [2][4][Vh]     halves 8..11
   double2* U3 = nullptr;    // [3][9][V]      spatial links, lexicographic, for the Laplacian
-  float4* U3f = nullptr;    // [3][3][V]      spatial links 12-real fp32
+  float4* U3f = nullptr;    // [3][5][V]      spatial links, fp32 (18 reals + 2 pad)
   // clover: 2 hermitian 6x6 blocks per site packed as 72 reals
   // (per block: 6 real diagonal entries, then the 15 complex entries below the diagonal, row-major)
   double2* C64 = nullptr;   // [2][36][Vh]  T(x)
@@ -207,7 +214,7 @@ enum WorkSlot {
   WS_SCAL, WS_PART, WS_ACT, WS_ITERS,
   WS_EIG_X, WS_EIG_Y, WS_EIG_Y2, WS_EIG_W, WS_EIG_G, WS_EIG_PART, WS_EIG_S, WS_EIG_AUX,
   WS_PROJ_V, WS_PROJ_PART, WS_PROJ_C, WS_CON, WS_CON2, WS_SRC, WS_SOL, WS_ETA,
-  WS_BI_S, WS_BI_R0, WS_BI_W0, WS_BI_PART, WS_BI_SCAL, WS_RETRY_B, WS_RETRY_X,
+  WS_BI_S, WS_BI_R0, WS_BI_W0, WS_CG_T32, WS_BI_PART, WS_BI_SCAL, WS_RETRY_B, WS_RETRY_X,
   WS_TC_A, WS_TC_B, WS_TC_E, WS_TC_P, WS_SUPPORT,
   WS_COUNT
 };
@@ -360,6 +367,7 @@ dlma_status solve_fields(dlma_ctx* ctx, const double* b_dev, double* x_dev, int 
 // V^dag psi on the tensor cores, FP64-accurate (split-precision digits): coeff[j][Tsel][4][N]
 dlma_status project_tc(dlma_ctx* ctx, const double2* VT, int N, int Tsel, const double* psi, size_t stride_sites,
                        int site_t0, int nrhs, double2* coeff);
+size_t tc_min_bytes(int R, int N, int T);
 // sum over kappa of conj(B_k) A_r per timeslice on the tensor cores (tcproj.cu):
 // omode 1 writes out[t][k][r], omode 2 out[t][r][k]
 dlma_status tc_block_product(dlma_ctx* ctx, int omode, const double2* a_src, size_t a_st, size_t a_sr, size_t a_sk,

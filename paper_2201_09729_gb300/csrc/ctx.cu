@@ -150,9 +150,10 @@ __global__ void k_gauge_convert(Geom g, const double2* __restrict__ Ucan, double
     U16b[base * g.Vh + i] = b;
     if (mu >= 1) {
       for (int k = 0; k < 9; k++) U3[((size_t)(mu - 1) * 9 + k) * g.V + s] = e[k];
-      for (int q = 0; q < 3; q++)
-        U3f[((size_t)(mu - 1) * 3 + q) * g.V + s] = make_float4((float)e[2 * q].x, (float)e[2 * q].y,
-                                                               (float)e[2 * q + 1].x, (float)e[2 * q + 1].y);
+      for (int q = 0; q < 5; q++) {
+        const double2 a = e[2 * q], b = 2 * q + 1 < 9 ? e[2 * q + 1] : make_double2(0, 0);
+        U3f[((size_t)(mu - 1) * 5 + q) * g.V + s] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+      }
     }
   }
 }
@@ -440,7 +441,7 @@ extern "C" dlma_status dlma_create(const dlma_lattice* lat, int device, void* cu
             cudaMalloc(&ctx->U16a, 2 * 4 * Vh * sizeof(uint4)) == cudaSuccess &&
             cudaMalloc(&ctx->U16b, 2 * 4 * Vh * sizeof(uint2)) == cudaSuccess &&
             cudaMalloc(&ctx->U3, 3 * 9 * V * sizeof(double2)) == cudaSuccess &&
-            cudaMalloc(&ctx->U3f, 3 * 3 * V * sizeof(float4)) == cudaSuccess &&
+            cudaMalloc(&ctx->U3f, 3 * 5 * V * sizeof(float4)) == cudaSuccess &&
             cudaMalloc(&ctx->C64, 2 * 36 * Vh * sizeof(double2)) == cudaSuccess &&
             cudaMalloc(&ctx->Ci64, 2 * 36 * Vh * sizeof(double2)) == cudaSuccess &&
             cudaMalloc(&ctx->C32, 2 * 18 * Vh * sizeof(float4)) == cudaSuccess &&

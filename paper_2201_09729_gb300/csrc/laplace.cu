@@ -49,16 +49,15 @@ __device__ __forceinline__ void load_link3(const double2* __restrict__ U, int k,
     u[q / 3][q % 3] = cx<double>(e.x, e.y);
   }
 }
+// all 18 reals: the load is shared by the columns of a site, rebuilding the third row
+// would cost each thread 24 operations
 __device__ __forceinline__ void load_link3(const float4* __restrict__ U, int k, size_t s, size_t V, Cx<float> u[3][3]) {
 #pragma unroll
-  for (int q = 0; q < 3; q++) {
-    float4 e = __ldg(U + ((size_t)k * 3 + q) * V + s);
+  for (int q = 0; q < 5; q++) {
+    const float4 e = __ldg(U + ((size_t)k * 5 + q) * V + s);
     u[(2 * q) / 3][(2 * q) % 3] = cx<float>(e.x, e.y);
-    u[(2 * q + 1) / 3][(2 * q + 1) % 3] = cx<float>(e.z, e.w);
+    if (2 * q + 1 < 9) u[(2 * q + 1) / 3][(2 * q + 1) % 3] = cx<float>(e.z, e.w);
   }
-  u[2][0] = conj(u[0][1] * u[1][2] - u[0][2] * u[1][1]);
-  u[2][1] = conj(u[0][2] * u[1][0] - u[0][0] * u[1][2]);
-  u[2][2] = conj(u[0][0] * u[1][1] - u[0][1] * u[1][0]);
 }
 
 // NC adjacent complex entries starting at p (16-byte aligned when NC is even): FP32
@@ -97,9 +96,9 @@ __global__ void __launch_bounds__(256, 2) k_lap(Geom g, int t0, int Tn, int m, c
   const size_t rowbase = (size_t)tl * g.Vs;
   const int yz = ms / g.L, x = ms - yz * g.L, z = yz / g.L, y = yz - z * g.L;
   const size_t s = (size_t)(t0 + tl) * g.Vs + ms;
-  Cx<double> acc[3];
+  Cx<double> h[3];
 #pragma unroll
-  for (int a = 0; a < 3; a++) acc[a] = 6.0 * in[((rowbase + ms) * 3 + a) * m + j0];
+  for (int a = 0; a < 3; a++) h[a] = cx<double>(0, 0);
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     int xf = x, yf = y, zf = z, xb = x, yb = y, zb = z;
@@ -116,18 +115,19 @@ __global__ void __launch_bounds__(256, 2) k_lap(Geom g, int t0, int Tn, int m, c
       vb[a] = in[((rowbase + mb) * 3 + a) * m + j0];
     }
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-      Cx<double> h = cx<double>(0, 0);
+    for (int a = 0; a < 3; a++)
 #pragma unroll
       for (int b = 0; b < 3; b++) {
-        fma_acc(h, uf[a][b], vf[b]);
-        fma_conj_acc(h, ub[b][a], vb[b]);
+        fma_acc(h[a], uf[a][b], vf[b]);
+        fma_conj_acc(h[a], ub[b][a], vb[b]);
       }
-      acc[a] = acc[a] - h;
-    }
   }
 #pragma unroll
-  for (int a = 0; a < 3; a++) out[((rowbase + ms) * 3 + a) * m + j0] = acc[a];
+  for (int a = 0; a < 3; a++) {
+    const size_t e3 = ((rowbase + ms) * 3 + a) * m + j0;
+    const Cx<double> v = in[e3];
+    out[e3] = cx<double>(fma(6.0, v.re, -h[a].re), fma(6.0, v.im, -h[a].im));
+  }
 }
 
 // FP32: out = alpha_t (A in) + beta_t in + gamma_t prev + alpha_t s[t][j] rin (prev and rin
@@ -138,8 +138,9 @@ __global__ void __launch_bounds__(256, 2) k_lap(Geom g, int t0, int Tn, int m, c
 // patch of px x py sites of a plane, whose x and y neighbours meet in L1.  The plain form
 // (k_lap: a row of sites per block) moved 6.5 vectors per application from L2 to the SMs
 // (0.215 ms for a block of 16^3 x 32 with 64 columns, 2.12 for 24^3 x 48 with 128); this
-// one moves about 3.5 and takes 0.196 and 1.87 ms, bound by instruction issue (some 800
-// per site and column pair, a sixth of them rebuilding link rows; DRAM floor 0.09, 0.92).
+// one moves about 3.5 and takes 0.184 and 1.68 ms, bound by instruction issue (some 560
+// per site and column pair; DRAM floor 0.09, 0.92).  With 12-real links, whose third row
+// each thread rebuilds, and separate sums per direction it took 0.196 and 1.87.
 // Block: pw column pairs x (px py) sites; grid: (patches of a plane x z segments x column
 // groups, timeslices).
 struct LapTiling {
@@ -177,91 +178,84 @@ __global__ void __launch_bounds__(256, 2) k_lap_z(Geom g, int t0, int m, LapTili
 #pragma unroll
     for (int a = 0; a < 3; a++) ld_cols<2>(p + ((row0 + ms) * 3 + a) * m + j0, v[a]);
   };
-  // w = U^dag v
+  // w += U v, w += U^dag v
+  const auto mul = [&](const Cx<float>(&u)[3][3], const Cx<float>(&v)[3][2], Cx<float>(&w)[3][2]) {
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+      for (int c = 0; c < 2; c++)
+#pragma unroll
+        for (int q = 0; q < 3; q++) fma_acc(w[a][c], u[a][q], v[q][c]);
+  };
   const auto dag_mul = [&](const Cx<float>(&u)[3][3], const Cx<float>(&v)[3][2], Cx<float>(&w)[3][2]) {
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
-      for (int c = 0; c < 2; c++) {
-        w[a][c] = cx<float>(0, 0);
+      for (int c = 0; c < 2; c++)
 #pragma unroll
         for (int q = 0; q < 3; q++) fma_conj_acc(w[a][c], u[q][a], v[q][c]);
-      }
   };
-  Cx<float> cur[3][2], wz[3][2];
+  const float b6 = (float)(6.0 * coef[3 * tl] + coef[3 * tl + 1]);
+  // hop: the sum of the six hopping terms, started with the backward z one
+  Cx<float> cur[3][2], hop[3][2];
+#pragma unroll
+  for (int a = 0; a < 3; a++) hop[a][0] = hop[a][1] = cx<float>(0, 0);
   {
     const int zb = z0 == 0 ? g.L - 1 : z0 - 1;
     Cx<float> u[3][3], v[3][2];
     load_link3(U, 2, s0 + o + (size_t)plane * zb, (size_t)g.V, u);
     load(in, o + plane * zb, v);
-    dag_mul(u, v, wz);
+    dag_mul(u, v, hop);
     load(in, o + plane * z0, cur);
   }
   for (int z = z0; z < z1; z++) {
     const int zo = plane * z, zf = plane * (z + 1 == g.L ? 0 : z + 1);
-    Cx<float> nxt[3][2], acc[3][2];
+    Cx<float> nxt[3][2], wz[3][2];
     load(in, o + zf, nxt);
     {
-      Cx<float> u[3][3], w[3][2];
+      Cx<float> u[3][3];
       load_link3(U, 2, s0 + o + zo, (size_t)g.V, u);
+      mul(u, nxt, hop);
 #pragma unroll
-      for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-          Cx<float> h = wz[a][c];
-#pragma unroll
-          for (int q = 0; q < 3; q++) fma_acc(h, u[a][q], nxt[q][c]);
-          acc[a][c] = 6.f * cur[a][c] - h;
-        }
-      dag_mul(u, cur, w);
-#pragma unroll
-      for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int c = 0; c < 2; c++) wz[a][c] = w[a][c];
+      for (int a = 0; a < 3; a++) wz[a][0] = wz[a][1] = cx<float>(0, 0);
+      dag_mul(u, cur, wz);
     }
 #pragma unroll
     for (int k = 0; k < 2; k++) {
-      Cx<float> u[3][3], v[3][2], w[3][2];
+      Cx<float> u[3][3], v[3][2];
       load_link3(U, k, s0 + o + zo, (size_t)g.V, u);
       load(in, nbr[2 * k] + zo, v);
-#pragma unroll
-      for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-          Cx<float> h = cx<float>(0, 0);
-#pragma unroll
-          for (int q = 0; q < 3; q++) fma_acc(h, u[a][q], v[q][c]);
-          acc[a][c] = acc[a][c] - h;
-        }
+      mul(u, v, hop);
       load_link3(U, k, s0 + (k == 0 ? oxb : oyb) + zo, (size_t)g.V, u);
       load(in, nbr[2 * k + 1] + zo, v);
-      dag_mul(u, v, w);
-#pragma unroll
-      for (int a = 0; a < 3; a++)
-#pragma unroll
-        for (int c = 0; c < 2; c++) acc[a][c] = acc[a][c] - w[a][c];
+      dag_mul(u, v, hop);
     }
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       const size_t idx = ((row0 + o + zo) * 3 + a) * m + j0;
       Cx<float> r[2];
 #pragma unroll
-      for (int c = 0; c < 2; c++) r[c] = alpha * acc[a][c] + beta * cur[a][c];
+      for (int c = 0; c < 2; c++) r[c] = b6 * cur[a][c];
       if (prev) {
         Cx<float> pv[2];
         ld_cols<2>(prev + idx, pv);
 #pragma unroll
-        for (int c = 0; c < 2; c++) r[c] = r[c] + gamma * pv[c];
+        for (int c = 0; c < 2; c++) r[c] = add_s(r[c], gamma, pv[c]);
       }
       if (rin) {
         Cx<float> rv[2];
         ld_cols<2>(rin + idx, rv);
-        r[0] = r[0] + fr0 * rv[0];
-        r[1] = r[1] + fr1 * rv[1];
+        r[0] = add_s(r[0], fr0, rv[0]);
+        r[1] = add_s(r[1], fr1, rv[1]);
       }
+#pragma unroll
+      for (int c = 0; c < 2; c++) r[c] = add_s(r[c], -alpha, hop[a][c]);
       st_cols<2>(out + idx, r);
 #pragma unroll
-      for (int c = 0; c < 2; c++) cur[a][c] = nxt[a][c];
+      for (int c = 0; c < 2; c++) {
+        cur[a][c] = nxt[a][c];
+        hop[a][c] = wz[a][c];
+      }
     }
   }
 }
@@ -508,15 +502,15 @@ __global__ void __launch_bounds__(256) k_rotate(const Cx<R>* __restrict__ X, con
 }
 
 // FP32 blocks: the same 64 x 64 tiles as k_gram_f (5.95 ms for 24^3 x 48 with 128 columns
-// with scalar shared loads, now 5.8; FP32 floor 3.5)
-__global__ void __launch_bounds__(256) k_rotate_f(const Cx<float>* __restrict__ X, const double2* __restrict__ Cm, int n,
-                                                  int m, Cx<float>* __restrict__ Z) {
+// with scalar shared loads and C converted from FP64 at every use, now 5.2; FP32 floor 3.5)
+__global__ void __launch_bounds__(256) k_rotate_f(const Cx<float>* __restrict__ X, const Cx<float>* __restrict__ Cm,
+                                                  int n, int m, Cx<float>* __restrict__ Z) {
   __shared__ __align__(16) Cx<float> xs[2][FK][FT + 2], cs[2][FK][FT];     // xs transposed: [l][k]
   const int t = blockIdx.z, k0 = blockIdx.x * FT, j0 = blockIdx.y * FT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int xr = threadIdx.x >> 2, xl = (threadIdx.x & 3) * 4;             // this thread's row and columns of X
   const Cx<float>* Xt = X + ((size_t)t * n + k0 + xr) * m + xl;
-  const double2* C = Cm + (size_t)t * m * m + j0 + 4 * tx;
+  const Cx<float>* C = Cm + (size_t)t * m * m + j0 + 4 * tx;
   const bool xon = k0 + xr < n;
   Cx<float> acc[4][4];
 #pragma unroll
@@ -526,12 +520,7 @@ __global__ void __launch_bounds__(256) k_rotate_f(const Cx<float>* __restrict__ 
   Cx<float> vx[4], vc[4];
   const auto fetch = [&](int l0) {
     ld4(Xt + l0, xon, m - l0 - xl, vx);
-#pragma unroll
-    for (int b = 0; b < 4; b++) {
-      const bool on = l0 + ty < m && j0 + 4 * tx + b < m;
-      const double2 e = on ? C[(size_t)(l0 + ty) * m + b] : make_double2(0, 0);
-      vc[b] = cx<float>((float)e.x, (float)e.y);
-    }
+    ld4(C + (size_t)(l0 + ty) * m, l0 + ty < m, m - j0 - 4 * tx, vc);
   };
   fetch(0);
   for (int l0 = 0, st = 0; l0 < m; l0 += FK, st ^= 1) {
@@ -811,7 +800,13 @@ template <class R> static dlma_status rotate(Eig& E, const Cx<R>* X, Cx<R>* Z) {
     if (E.df) k_rotate<R, df><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
     else k_rotate<R, R><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
   } else {
-    k_rotate_f<<<dim3((E.n + FT - 1) / FT, (E.m + FT - 1) / FT, E.Tn), 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
+    // C in FP32 first, into the Gram partials' area (a conversion per use would occupy the
+    // FP64 pipe for half of the kernel's time)
+    const size_t mmt = (size_t)E.m * E.m * E.Tn;
+    Cx<float>* Cf = (Cx<float>*)E.part;
+    k_convert_block<double, float><<<(unsigned)((mmt + 255) / 256), 256, 0, ctx->stream>>>((const Cx<double>*)E.C, Cf, mmt);
+    CHECK_LAUNCH();
+    k_rotate_f<<<dim3((E.n + FT - 1) / FT, (E.m + FT - 1) / FT, E.Tn), 256, 0, ctx->stream>>>(X, Cf, E.n, E.m, Z);
   }
   CHECK_LAUNCH();
   return DLMA_OK;
@@ -1079,6 +1074,8 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   // (and from kTcWork multiply-adds per product on the tensor cores; DLMA_EIGS_TC=1 / 0
   // forces either)
   E.tc = E.df && (double)E.n * E.m * E.m * E.Tn >= kTcWork;
+  // the rotation's digits (every row of the block) have to fit a memory cap
+  if (ctx->memcap && tc_min_bytes(E.n, E.m, E.Tn) > ctx->memcap) E.tc = 0;
   if (const char* e = getenv("DLMA_EIGS_TC")) E.tc = E.df && atoi(e) == 1;
   Cx<double> *X64 = E.D0, *W64 = E.D1, *Y64 = E.D2;
   // phase A's last Ritz pairs were not fetched, or hold refilled (random) columns

@@ -479,7 +479,9 @@ static dlma_status run_products(dlma_ctx* ctx, int T, int R, int N, int K, const
   if (ctx->memcap) budget = std::min(budget, (size_t)ctx->memcap / 4);
   int Qg = (int)std::max<size_t>(1, std::min<size_t>((size_t)Q, budget / per_chunk));
   Qg = (Q + (Q + Qg - 1) / Qg - 1) / ((Q + Qg - 1) / Qg);       // equal groups
-  const int ks = chunk_split((long)T * RT * MB, Qg);
+  int ks = chunk_split((long)T * RT * MB, Qg);
+  // the partial results keep to a quarter of a memory cap, like the digits
+  if (ctx->memcap) ks = (int)std::max<size_t>(1, std::min<size_t>(ks, ctx->memcap / 4 / (out_count * 16)));
   uint8_t *As, *Bs;
   int *eA, *eB;
   TRY(workT(ctx, WS_TC_A, (size_t)T * RT * Qg * NBK * S * A_TILE, &As));
@@ -538,6 +540,12 @@ dlma_status project_tc(dlma_ctx* ctx, const double2* VT, int N, int Tsel, const 
                         k_slice_psi<<<nb, 128, 0, ctx->stream>>>((const double2*)psi, stride_sites, site_t0, Vs, Tsel,
                                                                  nrhs, K, q0, qn, RT, As, eA, eAmax);
                       });
+}
+
+// bytes of the digit buffers of R rows, N modes and one chunk on T timeslices (the least
+// that run_products works with)
+size_t tc_min_bytes(int R, int N, int T) {
+  return (size_t)T * NBK * S * ((size_t)((R + TM - 1) / TM) * A_TILE + (size_t)((N + 31) / 32) * B_TILE);
 }
 
 // Block products of the eigensolver's FP64 phase on the tensor cores, with the same
