@@ -199,12 +199,12 @@ __device__ __forceinline__ void load_chiral(const void* __restrict__ base, const
   }
 }
 
-// out = A in for one 6 x 6 hermitian chirality block (36 packed reals: diagonal, then
-// the strictly lower triangle row by row)
-template <class S, class R>
-__device__ __forceinline__ void clover_block_mul(const S a[36], const Cx<R> in[6], Cx<R> out[6]) {
+// out = A in (ADD: out += A in) for one 6 x 6 hermitian chirality block (36 packed reals:
+// diagonal, then the strictly lower triangle row by row)
+template <bool ADD, class S, class R>
+__device__ __forceinline__ void clover_block(const S a[36], const Cx<R> in[6], Cx<R> out[6]) {
 #pragma unroll
-  for (int r = 0; r < 6; r++) out[r] = a[r] * in[r];
+  for (int r = 0; r < 6; r++) out[r] = ADD ? add_s(out[r], a[r], in[r]) : a[r] * in[r];
   int k = 6;
 #pragma unroll
   for (int r = 1; r < 6; r++)
@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
 #pragma unroll
         for (int c = 0; c < 3; c++) res[q].c[s][c] = cx<R>((R)0, (R)0);
     if (HOP) {
+      const S f = (S)(-0.5 * a.s);
       const int4 q0 = __ldg(a.nbr + ((size_t)a.p_out * 2 + 0) * g.Vh + i);
       const int4 q1 = __ldg(a.nbr + ((size_t)a.p_out * 2 + 1) * g.Vh + i);
       const int nb8[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
@@ -319,7 +320,14 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
           Cx<S> U[3][3];
           // forward: U_mu(x) at this site; backward: U_mu(x - mu) at the neighbour
           load_link<P>(a.Ua, a.Ub, dir == 0 ? a.p_out : 1 - a.p_out, mu, dir == 0 ? i : n, g.Vh, U, L18);
-          const S ph = raw < 0 ? (S)-1 : (S)1;    // antiperiodic time phase (bit 31, mu = 0 only)
+          // FP64 (bound by its arithmetic): the factor -s / 2 of the hopping term, with the
+          // antiperiodic time phase (bit 31, mu = 0 only) and the sign of gamma_5 on the
+          // lower spins, rides on the accumulation's multiply-adds (Dw of 8 vectors on
+          // 16^3 x 32: 2.34 -> 2.25 ms).  FP32: the factors' registers cost more than the
+          // scaling at the end.
+          constexpr bool kScaled = P == DLMA_FP64;
+          const S ph = mu == 0 && raw < 0 ? (S)-1 : (S)1;
+          const S fu = ph * f, fl = G5HOP ? -fu : fu;
 #pragma unroll
           for (int q = 0; q < NR; q++) {
             Spinor<R> ps = load_spinor<P>((const char*)a.in + (size_t)jl[q] * a.in_stride,
@@ -349,6 +357,17 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
             Spinor<R>& rq = res[q];
 #pragma unroll
             for (int c = 0; c < 3; c++) {
+              if constexpr (kScaled) {
+                const Cx<R> x0 = w0[c], x1 = w1[c];
+                rq.c[0][c] = add_s(rq.c[0][c], fu, x0);
+                rq.c[1][c] = add_s(rq.c[1][c], fu, x1);
+                const S g = dir == 0 ? fl : -fl;
+                if (mu == 0) { rq.c[2][c] = add_s(rq.c[2][c], g, x0); rq.c[3][c] = add_s(rq.c[3][c], g, x1); }
+                else if (mu == 1) { rq.c[2][c] = add_si(rq.c[2][c], -g, x1); rq.c[3][c] = add_si(rq.c[3][c], -g, x0); }
+                else if (mu == 2) { rq.c[2][c] = add_s(rq.c[2][c], -g, x1); rq.c[3][c] = add_s(rq.c[3][c], g, x0); }
+                else { rq.c[2][c] = add_si(rq.c[2][c], -g, x0); rq.c[3][c] = add_si(rq.c[3][c], g, x1); }
+                continue;
+              }
               const Cx<R> x0 = mu == 0 ? ph * w0[c] : w0[c], x1 = mu == 0 ? ph * w1[c] : w1[c];
               rq.c[0][c] = rq.c[0][c] + x0;
               rq.c[1][c] = rq.c[1][c] + x1;
@@ -367,16 +386,17 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
           }
         }
       }
-      const S f = (S)(-0.5 * a.s);
+      if constexpr (P != DLMA_FP64) {
 #pragma unroll
-      for (int q = 0; q < NR; q++)
+        for (int q = 0; q < NR; q++)
 #pragma unroll
-        for (int s = 0; s < 4; s++)
+          for (int s = 0; s < 4; s++)
 #pragma unroll
-          for (int c = 0; c < 3; c++) {
-            const S ff = (G5HOP && s >= 2) ? -f : f;
-            res[q].c[s][c] = ff * res[q].c[s][c];
-          }
+            for (int c = 0; c < 3; c++) {
+              const S ff = (G5HOP && s >= 2) ? -f : f;
+              res[q].c[s][c] = ff * res[q].c[s][c];
+            }
+      }
     }
     // own-site term and outer clover factor, chirality block by block: each block
     // of the clover field is loaded once for the NR right-hand sides
@@ -391,11 +411,14 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
             Cx<R> o[6], t[6];
             load_chiral<P>((const char*)a.own + (size_t)jl[q] * a.own_stride,
                            a.own_scale ? a.own_scale + (size_t)jl[q] * g.Vh : nullptr, g.Vh, i, ch, o);
-            if (OWN == 2) clover_block_mul(k, o, t);
+            // FP64 sums into the result (24 additions less), FP32 apart (fewer registers
+            // with packed operands: 1.57 against 1.61 ms per Schur application)
+            constexpr bool kAdd = OWN == 2 && P == DLMA_FP64;
+            if (OWN == 2) clover_block<kAdd>(k, o, kAdd ? &res[q].c[2 * ch][0] : t);
 #pragma unroll
             for (int r = 0; r < 6; r++) {
               Cx<R>& e = res[q].c[2 * ch + r / 3][r % 3];
-              e = e + (OWN == 2 ? t[r] : o[r]);
+              if (!kAdd) e = e + (OWN == 2 ? t[r] : o[r]);
               if (DOT) {           // the result is complete here (no outer factor)
                 dre[q] = fma(o[r].re, e.re, fma(o[r].im, e.im, dre[q]));
                 dim[q] = fma(o[r].re, e.im, fma(-o[r].im, e.re, dim[q]));
@@ -411,7 +434,7 @@ __global__ void __launch_bounds__(256, hop_minb(P, NR)) k_hop(HopArgs a) {
             Cx<R> o[6], t[6];
 #pragma unroll
             for (int r = 0; r < 6; r++) o[r] = res[q].c[2 * ch + r / 3][r % 3];
-            clover_block_mul(k, o, t);
+            clover_block<false>(k, o, t);
 #pragma unroll
             for (int r = 0; r < 6; r++) res[q].c[2 * ch + r / 3][r % 3] = t[r];
           }
@@ -947,8 +970,13 @@ static dlma_status check_ready(dlma_ctx* ctx) {
   return DLMA_OK;
 }
 
-// the internal form of a batch: FP32 in pairs from two right-hand sides on
-static int field_prec(int prec, int nrhs) { return prec == DLMA_FP32 && nrhs > 1 ? kFP32x2 : prec; }
+// The internal form of a batch of one operator call: FP32 in pairs of right-hand sides once
+// their half as many threads still fill the GPU (Schur application, pairs against single
+// vectors: 10^3 x 18, 7 right-hand sides (63000 pairs of site and vector), 23 and 21 us,
+// 24 (216000), 46 and 48; 16^3 x 32, 168, 1.57 and 1.77 ms).
+static int field_prec(const dlma_ctx* ctx, int prec, int nrhs) {
+  return prec == DLMA_FP32 && nrhs > 1 && (size_t)nrhs * ctx->g.Vh >= 100000 ? kFP32x2 : prec;
+}
 // a caller's canonical FP64 array as a field of the split stencil
 static Field canonical(dlma_ctx* ctx, const double* p, int nrhs, int lay) {
   Field f;
@@ -983,7 +1011,7 @@ extern "C" dlma_status dlma_apply_Dw(dlma_ctx* ctx, const double* in, double* ou
     CU(cudaStreamSynchronize(ctx->stream));
     return DLMA_OK;
   }
-  const int fp = field_prec(prec, nrhs), nv = field_vectors(fp, nrhs);
+  const int fp = field_prec(ctx, prec, nrhs), nv = field_vectors(fp, nrhs);
   Field fe, fo, re, ro;
   TRY(field_alloc(ctx, WS_T0, fp, nrhs, &fe));
   TRY(field_alloc(ctx, WS_T1, fp, nrhs, &fo));
@@ -1027,7 +1055,7 @@ extern "C" dlma_status dlma_apply_schur(dlma_ctx* ctx, const double* in, double*
   // few pairs: the split stencil reads and writes the canonical arrays themselves
   const bool direct = hop_split(ctx, prec, nrhs) && disjoint(din, dout, bytes);
   Field fe, tmp, res;
-  const int fp = field_prec(prec, nrhs);
+  const int fp = field_prec(ctx, prec, nrhs);
   TRY(field_alloc(ctx, WS_T1, fp, nrhs, &tmp));
   if (direct) {
     fe = canonical(ctx, din, nrhs, kLayHalf);

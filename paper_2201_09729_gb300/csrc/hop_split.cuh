@@ -68,10 +68,15 @@ __device__ __forceinline__ void load_row(const double2* __restrict__ K, int Vh, 
     m[c] = r == c ? cx<double>((r & 1) ? l.y : l.x, 0.0) : cx<double>(l.x, flip_if(l.y, r < c));
   }
 }
-__device__ __forceinline__ Cx<double> row_mul(const Cx<double> m[6], const Cx<double> v[6]) {
-  Cx<double> s = m[0] * v[0];
+// (r's own, real entry multiplies no imaginary parts: 0 x Inf would be NaN)
+__device__ __forceinline__ Cx<double> row_mul(const Cx<double> m[6], const Cx<double> v[6], int r) {
+  Cx<double> s = cx<double>(0, 0);
 #pragma unroll
-  for (int c = 1; c < 6; c++) fma_acc(s, m[c], v[c]);
+  for (int c = 0; c < 6; c++) {
+    const double xr = c == r ? 0.0 : v[c].re, xi = c == r ? 0.0 : v[c].im;
+    s.re = fma(-m[c].im, xi, fma(m[c].re, v[c].re, s.re));
+    s.im = fma(m[c].im, xr, fma(m[c].re, v[c].im, s.im));
+  }
   return s;
 }
 
@@ -157,7 +162,7 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
   }
   if (work && a.own_op) {
     Cx<double> t = cx<double>(0, 0);
-    if (a.own_op == 2) t = row_mul(ko, ow);
+    if (a.own_op == 2) t = row_mul(ko, ow, row);
     else {
 #pragma unroll
       for (int r = 0; r < 6; r++)
@@ -172,7 +177,7 @@ __global__ void __launch_bounds__(16 * kSplitSites) k_hop_split(SplitArgs a) {
       Cx<double> v[6];
 #pragma unroll
       for (int r = 0; r < 6; r++) v[r] = cx<double>(Rs[s2][6 * ch + r].x, Rs[s2][6 * ch + r].y);
-      res = row_mul(ko, v);
+      res = row_mul(ko, v, row);
     }
   }
   double nrm = 0;

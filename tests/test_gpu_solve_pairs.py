@@ -1,5 +1,6 @@
-"""BiCGStab on pairs of right-hand sides (large batches) against the single-vector form
-(small ones): an odd batch just above the switch, with a zero source and a repeated one."""
+"""FP32 on pairs of right-hand sides (large batches): odd batches just above the switches,
+the operator against FP64, BiCGStab with a zero source and a repeated one against the
+single-vector form."""
 import numpy as np
 import pytest
 
@@ -36,4 +37,21 @@ def test_pairs_and_single(dl):
     one, _ = ctx.dlma_solve(b[:1].contiguous(), tol, dl.FP32)
     for y in (x[0], x[nrhs - 1]):
         assert float(torch.linalg.vector_norm(y - one[0]) / torch.linalg.vector_norm(one[0])) < 1e-8
+    ctx.close()
+
+
+def test_operator_pairs(dl):
+    torch = pytest.importorskip("torch")
+    L, T, nrhs = 8, 16, 27                         # 27 x 4096 even sites: above 10^5
+    ctx = dl.Context(L, T, 1, 0)
+    ctx.dlma_set_gauge(synth.gauge_field(L, T, 0.25, 633))
+    ctx.dlma_set_params(0.1, 1.2)
+    V = L ** 3 * T
+    psi = torch.from_numpy(synth.gaussian_spinors(nrhs, V, 634)).cuda()
+    he = psi[:, :V // 2].contiguous()
+    for got, want in [(ctx.dlma_apply_Dw(psi, dl.FP32), ctx.dlma_apply_Dw(psi, dl.FP64)),
+                      (ctx.dlma_apply_schur(he, 0, dl.FP32), ctx.dlma_apply_schur(he, 0, dl.FP64)),
+                      (ctx.dlma_apply_schur(he, 1, dl.FP32), ctx.dlma_apply_schur(he, 1, dl.FP64))]:
+        d = torch.linalg.vector_norm((got - want).flatten(1), dim=1)
+        assert bool((d < 1e-6 * torch.linalg.vector_norm(want.flatten(1), dim=1)).all())
     ctx.close()
