@@ -161,9 +161,10 @@ dlma_status dlma_apply_schur_noalloc(dlma_ctx* ctx, const double* in, double* ou
  * dlma_set_solver); `inner` = DLMA_FP64 runs it in double precision, DLMA_FP32 /
  * DLMA_FP16S run the Krylov iteration in that precision (FP16: storage, FP32
  * arithmetic) with FP64 reliable updates: when a right-hand side's iterated
- * residual has dropped by a fixed factor since its last update, its solution
- * is folded into FP64 and its residual recomputed in FP64 (for BiCGStab's
- * last update see dlma_set_solver).  Each right-hand side stops when its
+ * residual has dropped by a fixed factor since its last update (or by what is
+ * still missing, with a margin, if that is less), its solution is folded into
+ * FP64 and its residual recomputed in FP64 (for the last updates of FP32 and
+ * FP16S solves see dlma_set_solver).  Each right-hand side stops when its
  * FP64 true residual ||b - D x|| / ||b|| <= tol and is retired from the batch.  `info` (may be
  * NULL) receives nrhs records.  A zero source gives x = 0.
  * Errors: STATE, INVALID_ARG (tol <= 0, nrhs < 1), NOT_CONVERGED, NONFINITE,
@@ -181,7 +182,9 @@ dlma_status dlma_solve(dlma_ctx* ctx, const double* b, double* x, int nrhs, doub
  * right-hand side's FP64 residual is below 1e-3 (tol / 2) / 1.2e-7 times |b|,
  * its next update subtracts the FP32 operator's image of the FP32 solution
  * increment from that residual instead of applying the FP64 operator: the
- * FP32 rounding of the small product stays below 1e-3 (tol / 2) |b|.  Two operator
+ * FP32 rounding of the small product stays below 1e-3 (tol / 2) |b| (CGNE with
+ * FP32 vectors does the same).  The shadow residual is a fixed vector of random
+ * signs.  Two operator
  * applications per iteration and about half as many as CGNE needs on these
  * systems.  Right-hand sides it leaves above the tolerance are solved again
  * with CGNE in the same call; their info sums both iteration counts.

@@ -860,7 +860,7 @@ static int pipeline_batch(dlma_ctx* ctx, int J, int granule) {
   // own previous call still holds
   size_t held = 0;
   for (int s : {WS_SRC, WS_SOL, WS_SOLVE_B, WS_SOLVE_X64, WS_SOLVE_R64, WS_SOLVE_BH, WS_SOLVE_TMP64, WS_CG_X, WS_CG_R,
-                WS_CG_P, WS_CG_PLO, WS_CG_Q, WS_CG_Z, WS_CG_TMP, WS_CG_RHS, WS_BI_S, WS_BI_R0, WS_RETRY_B, WS_RETRY_X})
+                WS_CG_P, WS_CG_PLO, WS_CG_Q, WS_CG_Z, WS_CG_TMP, WS_CG_RHS, WS_BI_S, WS_BI_R0, WS_CG_T32, WS_RETRY_B, WS_RETRY_X})
     held += ctx->wb[s].bytes;
   const size_t budget = ctx->memcap ? ctx->memcap : (size_t)(0.8 * (double)(freeb + held));
   int nb = (int)std::max<size_t>((size_t)granule, std::min<size_t>((size_t)J, budget / per_rhs));

@@ -796,7 +796,8 @@ struct SolveBufs {
   Field sl, r0, w0;
   double2 *cpart, *cpart2, *cpart3;
   int* rmask;
-  int *ru_hi, *ru_lo;   // BiCGStab updates: FP64 operator / FP32 correction of the residual
+  int *ru_hi, *ru_lo;   // updates: FP64 operator / FP32 correction of the residual
+  Field t32, q32;       // work fields of that correction (vector precision)
   BiScal bs;
   // host copies of the set-up
   std::vector<double> bn;
@@ -831,6 +832,37 @@ static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int ma
   return DLMA_OK;
 }
 
+// x64 += s x_l, x_l = 0 and the new r64 = bhat - Dhat x64 of the paused rhs, with the
+// |r64|^2 partials in part2 (one block of BX sites each).  r64 changes by -s Dhat x_l: for
+// FP32 solutions of rhs whose last residual is below theta |b| that change is applied with
+// the FP32 operator, whose relative rounding (~1e-6 with the cancellation between hop and
+// clover terms) leaves an error below 1e-3 of the target tolerance; the others evaluate
+// the residual with the FP64 operator.
+template <int PL>
+static dlma_status fold_residual(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target) {
+  const int Vh = ctx->g.Vh;
+  const dim3 gv((Vh + BX - 1) / BX, nrhs), gl(gv.x, field_vectors(PL, nrhs));
+  const int* hi = B.sc.ru;
+  if constexpr (PL != DLMA_FP64) {
+    const double theta = 1e-3 * tol_target / 1.2e-7;
+    k_split_ru<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc, theta, B.ru_hi, B.ru_lo);
+    CHECK_LAUNCH();
+    TRY(schur_apply(ctx, B.xl, B.t32, B.q32, 0, B.ru_lo, nullptr));
+    hi = B.ru_hi;
+  }
+  k_fold<PL><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, B.sc.ru);
+  CHECK_LAUNCH();
+  TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, hi, nullptr));
+  k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
+                                      (double2*)B.r64.data, hi, B.part2);
+  CHECK_LAUNCH();
+  if constexpr (PL != DLMA_FP64) {
+    k_corr64<PL><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q32.data, B.sc.scale, B.ru_lo, B.part2);
+    CHECK_LAUNCH();
+  }
+  return DLMA_OK;
+}
+
 // Reliable update of the rhs in mask ru: x64 += s x_l, x_l = 0; r64 = bhat - Dhat x64 (FP64);
 // retire the converged ones; for the others r_l = Dhat^dag (r64 / s) and resume.
 // first: the initial update (nothing to fold); restart: also reset p = r (a plain
@@ -849,12 +881,7 @@ static dlma_status reliable_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double
                        ctx->stream));
     CU(cudaMemcpyAsync(B.sc.rnorm, B.sc.scale, sizeof(double) * nrhs, cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
-    k_fold<PB><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, ru);
-    CHECK_LAUNCH();
-    TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, ru, nullptr));
-    k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
-                                        (double2*)B.r64.data, ru, B.part2);
-    CHECK_LAUNCH();
+    TRY(fold_residual<PB>(ctx, B, nrhs, tol_target));
     TRY(rowsum(ctx, B.part2, gv.x, nrhs, B.sc.rnorm, 1, ru));
   }
   k_mark_exact<<<nb1, 128, 0, ctx->stream>>>(nrhs, B.sc);
@@ -915,6 +942,12 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   TRY(field_alloc(ctx, WS_CG_Z, PS, nrhs, &B.z));
   TRY(field_alloc(ctx, WS_CG_TMP, PS, nrhs, &B.tmp));
   TRY(field_alloc(ctx, WS_CG_RHS, PS, nrhs, &B.rhs));
+  B.t32 = B.tmp;
+  B.q32 = B.q;
+  if (PS != PB) {
+    TRY(field_alloc(ctx, WS_CG_T32, PB, nrhs, &B.t32));
+    TRY(field_alloc(ctx, WS_BI_S, PB, nrhs, &B.q32));
+  }
   if (bicg) {
     TRY(field_alloc(ctx, WS_BI_S, PB, nrhs, &B.sl));
     TRY(field_alloc(ctx, WS_BI_R0, DLMA_FP32, 1, &B.r0));
@@ -1327,24 +1360,7 @@ static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol
                        ctx->stream));
     CU(cudaMemcpyAsync(B.sc.rnorm, B.sc.scale, sizeof(double) * nrhs, cudaMemcpyDeviceToDevice, ctx->stream));
   } else {
-    // x64 += s x_l.  r64 = bhat - Dhat x64 changes by -s Dhat x_l: for rhs whose last
-    // residual is below theta |b| that change is applied with the FP32 operator, whose
-    // relative rounding (~1e-6 with the cancellation between hop and clover terms)
-    // leaves an error below 1e-3 of the target tolerance; the others evaluate the
-    // residual with the FP64 operator
-    const double theta = 1e-3 * tol_target / 1.2e-7;
-    k_split_ru<<<nb1, 128, 0, ctx->stream>>>(nrhs, B.sc, theta, B.ru_hi, B.ru_lo);
-    CHECK_LAUNCH();
-    TRY(schur_apply(ctx, B.xl, B.tmp, B.q, 0, B.ru_lo, nullptr));
-    k_fold<P><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, ru);
-    CHECK_LAUNCH();
-    TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, B.ru_hi, nullptr));
-    k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
-                                        (double2*)B.r64.data, B.ru_hi, B.part2);
-    CHECK_LAUNCH();
-    k_corr64<P><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q.data, B.sc.scale, B.ru_lo,
-                                            B.part2);
-    CHECK_LAUNCH();
+    TRY(fold_residual<P>(ctx, B, nrhs, tol_target));
     TRY(rowsum(ctx, B.part2, gv.x, nrhs, B.sc.rnorm, 1, ru));
   }
   k_mark_exact<<<nb1, 128, 0, ctx->stream>>>(nrhs, B.sc);
@@ -1488,7 +1504,7 @@ dlma_status solve_fields(dlma_ctx* ctx, const double* b_dev, double* x_dev, int 
   const size_t Vh = ctx->g.Vh;
   size_t per_rhs = field_bytes_per_rhs(DLMA_FP64, Vh) * 7;
   const int pb = inner == DLMA_FP64 ? DLMA_FP64 : DLMA_FP32;
-  per_rhs += field_bytes_per_rhs(pb, Vh) * 5 + field_bytes_per_rhs(inner, Vh) * 5;
+  per_rhs += field_bytes_per_rhs(pb, Vh) * (inner == DLMA_FP16S ? 7 : 5) + field_bytes_per_rhs(inner, Vh) * 5;
   size_t freeb = 0, totb = 0;
   cudaMemGetInfo(&freeb, &totb);
   size_t budget = (size_t)(0.85 * (double)(freeb + ctx->work_bytes));
