@@ -373,11 +373,6 @@ size_t tc_min_bytes(int R, int N, int T);
 dlma_status tc_block_product(dlma_ctx* ctx, int omode, const double2* a_src, size_t a_st, size_t a_sr, size_t a_sk,
                              int R, const double2* b_src, int b_conj, int N, int K, int T, double2* out);
 
-// per-context event timer helper
-struct EvTimer {
-  cudaEvent_t a = nullptr, b = nullptr;
-};
-
 // Phase timer: events recorded on the context's stream at phase boundaries; the
 // time between consecutive marks is charged to the phase opened by the earlier
 // mark.  collect() (after a stream synchronisation) adds the elapsed times to

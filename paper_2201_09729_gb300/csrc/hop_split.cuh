@@ -11,7 +11,7 @@
 // meeting in shared memory: about 100 FP64 instructions deep, 41 warp instructions per
 // pair against k_hop's 37, so k_hop stays ahead once every sub-partition has a warp of
 // its own (kHopSplitPairs).  Measured, one Schur application on 4^3 x 8: 87 -> 20 us with
-// one vector, 87 -> 29 us with 12 (12 us at the FP64 rate; the rest is the latency of two
+// one vector, 87 -> 28 us with 12 (12 us at the FP64 rate; the rest is the latency of two
 // dependent loads and two barriers per launch).  Signs, factors +-i and the conjugations are integer
 // operations on the operands, not FP64 ones.
 //

@@ -261,7 +261,7 @@ __global__ void k_fill_int(int* p, size_t n, int v) {
 // Tile (row block rt, mode block mb, timeslice tl) over a share of the group's chunks.
 // Bound by the MMAs (8192 FLOP per clock and SM) and, not overlapped with them, the
 // epilogue's reading of the six classes after every chunk (two class sets do not fit
-// in TMEM).  40 right-hand sides, 32 modes, 16^3 x 32: 3.2 ms with 36 products of 6-bit
+// in TMEM).  40 right-hand sides, 32 modes, 16^3 x 32: 2.76 ms with 36 products of 6-bit
 // digits in N = 64 instructions on 64 blocks; 1.49 ms with 21 products of 8-bit digits;
 // 0.53 ms with the digits of B side by side and 7 blocks per tile (chunk_split).
 // Warp 0: bulk copies; warp 1: TMEM and MMAs; warps 2..9: epilogue (warp w reads
