@@ -76,10 +76,12 @@ typedef struct {
 typedef struct {
   int iters_inner;     /* inner (low-precision) Krylov iterations summed over restarts */
   int iters_outer;     /* FP64 reliable updates (residual replacements) */
-  double true_resid;   /* ||b - D x||_2 / ||b||_2 in FP64: the even-odd Schur residual
-                          |bhat - Dhat x_e| of the final FP64 update (the odd rows of
-                          b - D x vanish by construction of x_o), or, for a solve stopped
-                          before converging, b - D x evaluated on the full lattice */
+  double true_resid;   /* ||b - D x||_2 / ||b||_2: the even-odd Schur residual
+                          |bhat - Dhat x_e| of the final reliable update (the odd rows of
+                          b - D x vanish by construction of x_o), evaluated in FP64 or
+                          within 0.05 (tol / 2) of that (see dlma_set_solver), or, for a
+                          solve stopped before converging, b - D x evaluated in FP64 on
+                          the full lattice */
   int converged;       /* 1 if true_resid <= tol */
 } dlma_solve_info;
 
@@ -178,13 +180,13 @@ dlma_status dlma_solve(dlma_ctx* ctx, const double* b, double* x, int nrhs, doub
  * FP32 vectors and the same FP64 reliable updates (residual replacement when
  * |r| has dropped by 3e-4 since the last update, DLMA_BICG_DELTA in the
  * environment overriding the factor; restart of the search direction after a
- * breakdown or a stagnating update).  The iteration aims at tol / 2; once a
- * right-hand side's FP64 residual is below 1e-3 (tol / 2) / 1.2e-7 times |b|,
- * its next update subtracts the FP32 operator's image of the FP32 solution
- * increment from that residual instead of applying the FP64 operator: the
- * FP32 rounding of the small product stays below 1e-3 (tol / 2) |b| (CGNE with
- * FP32 vectors does the same).  The shadow residual is a fixed vector of random
- * signs.  Two operator
+ * breakdown or a stagnating update).  The iteration aims at tol / 2.  Where that
+ * changes the reported residual by less than 0.05 (tol / 2), an update subtracts the
+ * FP32 operator's image of the FP32 solution increment from the last residual instead
+ * of applying the FP64 operator to x: the errors of doing so, bounded by
+ * |Dhat| (2 eps32 |increment| + eps64 / 2 |x|) and added up since the last FP64
+ * evaluation, have to stay within 0.05 (tol / 2) |b| (CGNE with FP32 vectors does the
+ * same).  The shadow residual is a fixed vector of random signs.  Two operator
  * applications per iteration and about half as many as CGNE needs on these
  * systems.  Right-hand sides it leaves above the tolerance are solved again
  * with CGNE in the same call; their info sums both iteration counts.

@@ -154,6 +154,7 @@ struct dlma_ctx {
 
   bool have_gauge = false, have_params = false;
   double m0 = 0, csw = 0;
+  double schur_norm = 0;               // bound of |Dhat| (set_params)
   int solver = DLMA_SOLVER_BICGSTAB;   // Krylov method of the FP32 inner solves
   // generations of the gauge field and of the cached modes: a checkpoint taken
   // under one generation is stale under the next

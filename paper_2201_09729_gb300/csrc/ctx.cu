@@ -236,9 +236,22 @@ __device__ __forceinline__ void pack_block(Cx<double> A[6][6], double* out) {
     }
 }
 
+// *norm = max(*norm, largest row sum of |A_ij|), a bound of the hermitian block's norm
+// (non-negative doubles order like their bits)
+__device__ void max_row_sum(const Cx<double> A[6][6], unsigned long long* norm) {
+  double m = 0;
+  for (int i = 0; i < 6; i++) {
+    double s = 0;
+    for (int j = 0; j < 6; j++) s += sqrt(norm2(A[i][j]));
+    m = fmax(m, s);
+  }
+  const unsigned long long b = (unsigned long long)__double_as_longlong(m);
+  if (b > *(volatile unsigned long long*)norm) atomicMax(norm, b);      // few sites exceed the maximum so far
+}
+
 __global__ void k_clover(Geom g, const double2* __restrict__ Ucan, SigmaBlocks sb, double m0, double csw,
                          double2* C64, double2* Ci64, float4* C32, float4* Ci32, uint4* C16, uint4* Ci16,
-                         int* flag) {
+                         int* flag, unsigned long long* norms) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   int x = s % g.L, y = (s / g.L) % g.L, z = (s / (g.L * g.L)) % g.L, t = s / (g.L * g.L * g.L);
@@ -270,8 +283,10 @@ __global__ void k_clover(Geom g, const double2* __restrict__ Ucan, SigmaBlocks s
             for (int b = 0; b < 3; b++) A[s1 * 3 + a][s2 * 3 + b] = A[s1 * 3 + a][s2 * 3 + b] + f * F[pl][a][b];
         }
     pack_block(A, packed + 36 * ch);
+    max_row_sum(A, norms);
     ok = ok && inv6(A, B);
     pack_block(B, packedi + 36 * ch);
+    if (ok) max_row_sum(B, norms + 1);
   }
   if (!ok) atomicOr(flag, 2);
   for (int k = 0; k < 36; k++) {
@@ -557,10 +572,12 @@ extern "C" dlma_status dlma_set_params(dlma_ctx* ctx, double m0, double c_sw) {
   CU(cudaMemsetAsync(ctx->flag, 0, 16 * sizeof(int), ctx->stream));
   int nb = (ctx->g.V + 127) / 128;
   k_clover<<<nb, 128, 0, ctx->stream>>>(ctx->g, Ucan, sb, m0, c_sw, ctx->C64, ctx->Ci64, ctx->C32, ctx->Ci32,
-                                        ctx->C16, ctx->Ci16, ctx->flag);
+                                        ctx->C16, ctx->Ci16, ctx->flag, (unsigned long long*)(ctx->flag + 4));
   CHECK_LAUNCH();
   int h = 0;
+  double norms[2];
   CU(cudaMemcpyAsync(&h, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CU(cudaMemcpyAsync(norms, ctx->flag + 4, sizeof(norms), cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   if (h & 2) {
     ctx->have_params = false;
@@ -568,6 +585,9 @@ extern "C" dlma_status dlma_set_params(dlma_ctx* ctx, double m0, double c_sw) {
   }
   ctx->m0 = m0;
   ctx->csw = c_sw;
+  // Dhat = T - D_eo T^-1 D_oe with |D_eo|, |D_oe| <= 4: half the hop is the sum over mu of
+  // S_mu-translations (S + S^dag - g_mu (S - S^dag)) / 2, each of norm 1
+  ctx->schur_norm = norms[0] + 16.0 * norms[1];
   ctx->have_params = true;
   ctx->dirac_N = 0;     // the Dirac low modes belong to the previous operator
   return DLMA_OK;

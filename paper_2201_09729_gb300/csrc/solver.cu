@@ -8,8 +8,9 @@
 // scaled by s_j = |bhat_j|.  When a right-hand side's iterated residual has
 // dropped by a factor delta since its last update, it pauses; at the end of the
 // chunk its low-precision solution is folded into the FP64 solution, the true
-// Schur residual r = bhat - Dhat x is recomputed in FP64 and, unless it is below
-// the tolerance, the iterated normal-equation residual is replaced by
+// Schur residual r = bhat - Dhat x is recomputed in FP64 (or, where a bound on the
+// error allows it, corrected with the FP32 operator, see fold_residual) and, unless it
+// is below the tolerance, the iterated normal-equation residual is replaced by
 // Dhat^dag r / s_j and the iteration resumes with the same search direction.
 // Every right-hand side carries its own CG scalars on the device and is retired
 // (masked out of every kernel) once converged.  A chunk of iterations is
@@ -31,7 +32,8 @@ struct CgScal {
   double* beta;
   double* stop2;   // |r|^2 that triggers the next reliable update
   double* rr0;     // |r|^2 right after the last update
-  double* rnorm;   // FP64 Schur residual norm per rhs (at the last update)
+  double* rnorm;   // |r64| per rhs at the last update
+  double* rerr;    // bound of |r64 - (bhat - Dhat x64)|, 0 after an FP64 evaluation
   double* bnorm;   // |b| per rhs (full lattice)
   double* scale;   // s_j = |bhat_j|: the low-precision system solves for x / s_j
   double* rrnew;   // recomputed |r|^2 after an update
@@ -46,7 +48,7 @@ struct CgScal {
   int* stall;      // consecutive updates without halving rbest
   int* rst;        // restart the search direction at this update (p = r)
   int* cf;         // mask of the final full-lattice residual evaluation
-  int* exact;      // rnorm comes from an FP64 evaluation of bhat - Dhat x64
+  int* exact;      // rnorm is that of bhat - Dhat x64, to rerr (not of an iterated residual)
   int* count;      // [0] iterating, [1] nonfinite flag, [2] paused for update
 };
 
@@ -245,80 +247,6 @@ __device__ __forceinline__ void lane_set(f2& v, int q, float x) { (q ? v.y : v.x
 __device__ __forceinline__ void lane_set(float& v, int, float x) { v = x; }
 __device__ __forceinline__ void lane_set(double& v, int, double x) { v = x; }
 
-// x64 += f_j * lo; lo = 0   (reliable update: fold the low-precision solution into FP64)
-template <int PL>
-__global__ void __launch_bounds__(BX) k_fold(int Vh, int nrhs, double2* x, void* lo, const double* f,
-                                              const int* mask) {
-  typedef typename PT<PL>::R R;
-  constexpr int LN = PT<PL>::lanes;
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y;
-  if (i >= Vh || !vec_on<PL>(j, nrhs, mask)) return;
-  const size_t sl = field_units_per_rhs(PL, Vh) * 16 * j;
-  Spinor<R> v = load_spinor<PL>((const char*)lo + sl, nullptr, Vh, i);
-#pragma unroll
-  for (int q = 0; q < LN; q++) {
-    if (!lane_on<PL>(j, q, nrhs, mask)) continue;
-    const int r = LN * j + q;
-    const double ff = f[r];
-    double2* xb = x + (size_t)12 * Vh * r;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-      double2 e = xb[(size_t)k * Vh + i];
-      Cx<R>& c = v.c[k / 3][k % 3];
-      e.x += ff * (double)lane_get(c.re, q);
-      e.y += ff * (double)lane_get(c.im, q);
-      xb[(size_t)k * Vh + i] = e;
-      lane_set(c.re, q, 0);
-      lane_set(c.im, q, 0);
-    }
-  }
-  store_spinor<PL>((char*)lo + sl, nullptr, Vh, i, v);
-}
-
-// r = a - b (FP64) with |r|^2 partial
-__global__ void __launch_bounds__(BX) k_sub64(int Vh, int nrhs, const double2* a, const double2* b, double2* r,
-                                               const int* mask, double* part) {
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y;
-  const bool on = mask ? mask[j] != 0 : true;
-  double n = 0;
-  if (i < Vh && on) {
-    const size_t o = (size_t)12 * Vh * j;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-      const double2 x = a[o + (size_t)k * Vh + i], y = b[o + (size_t)k * Vh + i];
-      const double2 d = make_double2(x.x - y.x, x.y - y.y);
-      r[o + (size_t)k * Vh + i] = d;
-      n += d.x * d.x + d.y * d.y;
-    }
-  }
-  block_partial(n, part, on ? j : nrhs, nrhs);
-}
-
-// per-rhs totals of a partial buffer: out[j] = sum_b part[j][b] (rows with mask[j] == 0 untouched)
-__global__ void k_rowsum(const double* part, int nb, int nrhs, double* out, int do_sqrt, const int* mask) {
-  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (j >= nrhs || (mask && !mask[j])) return;
-  const int lane = threadIdx.x & 31;
-  double s = 0;
-  for (int b = lane; b < nb; b += 32) s += part[(size_t)j * nb + b];
-  s = warp_sum(s);
-  if (lane == 0) out[j] = do_sqrt ? sqrt(s) : s;
-}
-
-// the paused rhs get their residual from an FP64 evaluation at this update
-// Split the rhs paused for a reliable update: those whose FP64 residual at the last
-// update is already below theta |b| (lo) correct it with an FP32 operator applied to
-// the FP32 increment; the rest (hi) recompute it with the FP64 operator.
-__global__ void k_split_ru(int nrhs, CgScal sc, double theta, int* ru_hi, int* ru_lo) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= nrhs) return;
-  const bool lo = sc.ru[j] && sc.rnorm[j] <= theta * sc.bnorm[j];
-  ru_lo[j] = lo;
-  ru_hi[j] = sc.ru[j] && !lo;
-}
-
 // Totals of N values over a warp, scattered: lane l returns the total of value `which`
 // (lanes 0 .. M - 1 hold every one).  An FP64 addition takes 64 cycles of its SM
 // sub-partition, so the halves of the list are exchanged and added (M - 1 + 5 - log2 M
@@ -363,9 +291,139 @@ template <int N, int NW = BX / 32> __device__ __forceinline__ void block_sums(do
   for (int e = 0; e < N; e++) v[e] = tot[e];
 }
 
-// r64 -= s_j t (t = Dhat x_l in the low precision P) with the |r64|^2 partial
+// site i of right-hand side r of a field in precision P = 0
+template <int P> __device__ __forceinline__ void zero_rhs(void* v, int Vh, int i, int r) {
+#pragma unroll
+  for (int k = 0; k < (P == DLMA_FP32 ? 6 : 12); k++) {
+    if constexpr (P == kFP32x2) {             // {re, re', im, im'} of the pair
+      float* e = (float*)((float4*)v + ((size_t)12 * (r >> 1) + k) * Vh + i) + (r & 1);
+      e[0] = e[2] = 0.f;
+    } else {
+      ((float4*)v)[(field_units_per_rhs(P, Vh) * r) + (size_t)k * Vh + i] = make_float4(0, 0, 0, 0);
+    }
+  }
+}
+
+// x64 += f_j * lo (reliable update: fold the low-precision solution into FP64).  NORMS:
+// partials of |lo|^2 and of the new |x64|^2, and lo stays for the FP32 image of it
+// (fold_residual); otherwise lo = 0.
+template <int PL, bool NORMS>
+__global__ void __launch_bounds__(BX) k_fold(int Vh, int nrhs, double2* x, void* lo, const double* f, const int* mask,
+                                             double* lpart, double* xpart) {
+  typedef typename PT<PL>::R R;
+  constexpr int LN = PT<PL>::lanes;
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int j = blockIdx.y;
+  if (!vec_on<PL>(j, nrhs, mask)) return;
+  double n[2 * LN] = {};
+  if (i < Vh) {
+    const size_t sl = field_units_per_rhs(PL, Vh) * 16 * j;
+    Spinor<R> v = load_spinor<PL>((const char*)lo + sl, nullptr, Vh, i);
+#pragma unroll
+    for (int q = 0; q < LN; q++) {
+      if (!lane_on<PL>(j, q, nrhs, mask)) continue;
+      const int r = LN * j + q;
+      const double ff = f[r];
+      double2* xb = x + (size_t)12 * Vh * r;
+      decltype(lane_get(R(), 0)) l2 = 0;       // a bound's norm: FP32 is enough for an FP32 vector
+#pragma unroll
+      for (int k = 0; k < 12; k++) {
+        double2 e = xb[(size_t)k * Vh + i];
+        Cx<R>& c = v.c[k / 3][k % 3];
+        const auto re = lane_get(c.re, q), im = lane_get(c.im, q);
+        e.x += ff * (double)re;
+        e.y += ff * (double)im;
+        xb[(size_t)k * Vh + i] = e;
+        if (NORMS) {
+          l2 = fma(re, re, fma(im, im, l2));
+          n[2 * q + 1] = fma(e.x, e.x, fma(e.y, e.y, n[2 * q + 1]));
+        } else {
+          lane_set(c.re, q, 0);
+          lane_set(c.im, q, 0);
+        }
+      }
+      if (NORMS) n[2 * q] = l2;
+    }
+    if (!NORMS) store_spinor<PL>((char*)lo + sl, nullptr, Vh, i, v);
+  }
+  if constexpr (NORMS) {
+    block_sums(n);
+    if (threadIdx.x == 0)
+#pragma unroll
+      for (int q = 0; q < LN; q++)
+        if (lane_on<PL>(j, q, nrhs, mask)) {
+          const size_t o = (size_t)(LN * j + q) * gridDim.x + blockIdx.x;
+          lpart[o] = n[2 * q];
+          xpart[o] = n[2 * q + 1];
+        }
+  }
+}
+
+// r = a - b (FP64) with |r|^2 partial; lo (a vector in precision PL, or null) = 0
+template <int PL>
+__global__ void __launch_bounds__(BX) k_sub64(int Vh, int nrhs, const double2* a, const double2* b, double2* r,
+                                               void* lo, const int* mask, double* part) {
+  const int i = blockIdx.x * BX + threadIdx.x;
+  const int j = blockIdx.y;
+  const bool on = mask ? mask[j] != 0 : true;
+  double n = 0;
+  if (i < Vh && on) {
+    const size_t o = (size_t)12 * Vh * j;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      const double2 x = a[o + (size_t)k * Vh + i], y = b[o + (size_t)k * Vh + i];
+      const double2 d = make_double2(x.x - y.x, x.y - y.y);
+      r[o + (size_t)k * Vh + i] = d;
+      n += d.x * d.x + d.y * d.y;
+    }
+    if (lo) zero_rhs<PL>(lo, Vh, i, j);
+  }
+  block_partial(n, part, on ? j : nrhs, nrhs);
+}
+
+// per-rhs totals of a partial buffer: out[j] = sum_b part[j][b] (rows with mask[j] == 0 untouched)
+__global__ void k_rowsum(const double* part, int nb, int nrhs, double* out, int do_sqrt, const int* mask) {
+  const int j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  if (j >= nrhs || (mask && !mask[j])) return;
+  const int lane = threadIdx.x & 31;
+  double s = 0;
+  for (int b = lane; b < nb; b += 32) s += part[(size_t)j * nb + b];
+  s = warp_sum(s);
+  if (lane == 0) out[j] = do_sqrt ? sqrt(s) : s;
+}
+
+// Split the rhs paused for a reliable update: lo corrects r64 with the FP32 operator's
+// image of x_l, hi recomputes it with the FP64 operator.  The correction leaves two errors
+// in r64: the image's rounding and that of x64 when x_l was folded into it.  The first is
+// below 2 eps32 norm s |x_l|, norm the bound of |Dhat| that set_params took (measured:
+// 0.16 ... 0.53 eps32 norm |x_l| over random fields, smooth ones and solutions, clover
+// coefficients 1 ... 2, masses -0.5 ... 2, norms 8 ... 19, 12- and 18-real links), the
+// second eps64 / 2 norm |x64|.  lo takes those whose errors, added up since their last
+// FP64 evaluation, stay within `limit` times |b|.
+__global__ void __launch_bounds__(256) k_split_ru(const double* lpart, const double* xpart, int nb, CgScal sc,
+                                                  double norm, double limit, int* ru_hi, int* ru_lo) {
+  const int j = blockIdx.x;
+  const bool on = sc.ru[j] != 0;
+  double n[2] = {0, 0};
+  if (on) {                                   // the whole block
+    for (int b = threadIdx.x; b < nb; b += 256) {
+      n[0] += lpart[(size_t)j * nb + b];
+      n[1] += xpart[(size_t)j * nb + b];
+    }
+    block_sums<2, 8>(n);
+  }
+  if (threadIdx.x) return;
+  const double err =
+      sc.rerr[j] + norm * (2.0 * 1.1920929e-7 * sc.scale[j] * sqrt(n[0]) + 1.1102231e-16 * sqrt(n[1]));
+  const bool lo = on && err <= limit * sc.bnorm[j];
+  if (on) sc.rerr[j] = lo ? err : 0.0;
+  ru_lo[j] = lo;
+  ru_hi[j] = on && !lo;
+}
+
+// r64 -= s_j t (t = Dhat x_l in the low precision P) with the |r64|^2 partial; x_l = 0
 template <int P>
-__global__ void __launch_bounds__(BX) k_corr64(int Vh, int nrhs, double2* r, const void* t, const double* f,
+__global__ void __launch_bounds__(BX) k_corr64(int Vh, int nrhs, double2* r, const void* t, void* lo, const double* f,
                                                const int* mask, double* part) {
   typedef typename PT<P>::R R;
   constexpr int LN = PT<P>::lanes;
@@ -388,6 +446,7 @@ __global__ void __launch_bounds__(BX) k_corr64(int Vh, int nrhs, double2* r, con
         rb[(size_t)k * Vh + i] = e;
         n[q] += e.x * e.x + e.y * e.y;
       }
+      zero_rhs<P>(lo, Vh, i, LN * j + q);
     }
   }
   block_sums(n);
@@ -833,31 +892,35 @@ static dlma_status inner_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int ma
 }
 
 // x64 += s x_l, x_l = 0 and the new r64 = bhat - Dhat x64 of the paused rhs, with the
-// |r64|^2 partials in part2 (one block of BX sites each).  r64 changes by -s Dhat x_l: for
-// FP32 solutions of rhs whose last residual is below theta |b| that change is applied with
-// the FP32 operator, whose relative rounding (~1e-6 with the cancellation between hop and
-// clover terms) leaves an error below 1e-3 of the target tolerance; the others evaluate
-// the residual with the FP64 operator.
+// |r64|^2 partials in part2 (one block of BX sites each).  r64 changes by -s Dhat x_l:
+// where the FP32 operator's rounding of that product (which goes as |x_l|, up to the
+// condition number times the residual) and the FP64 rounding of x64 together stay within
+// 5 % of the target, that change is applied with the FP32 operator; elsewhere, near the
+// critical mass or at tolerances near FP64's rounding, r64 is evaluated in FP64.
+constexpr double kCorrLimit = 0.05;
 template <int PL>
 static dlma_status fold_residual(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target) {
   const int Vh = ctx->g.Vh;
   const dim3 gv((Vh + BX - 1) / BX, nrhs), gl(gv.x, field_vectors(PL, nrhs));
   const int* hi = B.sc.ru;
-  if constexpr (PL != DLMA_FP64) {
-    const double theta = 1e-3 * tol_target / 1.2e-7;
-    k_split_ru<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc, theta, B.ru_hi, B.ru_lo);
+  constexpr bool kCorr = PL != DLMA_FP64;
+  k_fold<PL, kCorr><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, B.sc.ru, B.part,
+                                                B.part2);
+  CHECK_LAUNCH();
+  if constexpr (kCorr) {
+    k_split_ru<<<nrhs, 256, 0, ctx->stream>>>(B.part, B.part2, gv.x, B.sc, ctx->schur_norm, kCorrLimit * tol_target,
+                                              B.ru_hi, B.ru_lo);
     CHECK_LAUNCH();
     TRY(schur_apply(ctx, B.xl, B.t32, B.q32, 0, B.ru_lo, nullptr));
     hi = B.ru_hi;
   }
-  k_fold<PL><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, B.sc.ru);
-  CHECK_LAUNCH();
   TRY(schur_apply(ctx, B.x64, B.t64o, B.t64, 0, hi, nullptr));
-  k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
-                                      (double2*)B.r64.data, hi, B.part2);
+  k_sub64<PL><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.bh.data, (const double2*)B.t64.data,
+                                          (double2*)B.r64.data, kCorr ? B.xl.data : nullptr, hi, B.part2);
   CHECK_LAUNCH();
-  if constexpr (PL != DLMA_FP64) {
-    k_corr64<PL><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q32.data, B.sc.scale, B.ru_lo, B.part2);
+  if constexpr (kCorr) {
+    k_corr64<PL><<<gl, BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.r64.data, B.q32.data, B.xl.data, B.sc.scale,
+                                             B.ru_lo, B.part2);
     CHECK_LAUNCH();
   }
   return DLMA_OK;
@@ -962,7 +1025,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
     B.cpart3 = B.cpart2 + (size_t)nbmax * nrhs;
   }
   double* sd;
-  TRY(workT(ctx, WS_SCAL, (size_t)11 * nrhs + 64, &sd));
+  TRY(workT(ctx, WS_SCAL, (size_t)12 * nrhs + 64, &sd));
   B.sc.rr = sd;
   B.sc.alpha = sd + nrhs;
   B.sc.beta = sd + 2 * nrhs;
@@ -973,6 +1036,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
   B.sc.rrnew = sd + 7 * nrhs;
   B.tmpd = sd + 8 * nrhs;     // 2 nrhs scratch
   B.sc.rr0 = sd + 10 * nrhs;
+  B.sc.rerr = sd + 11 * nrhs;
   TRY(workT(ctx, WS_T0, (size_t)nrhs + 16, &B.sc.rbest));
   int* si;
   TRY(workT(ctx, WS_ACT, (size_t)16 * nrhs + 32, &si));
@@ -1098,6 +1162,7 @@ static dlma_status solve_setup(dlma_ctx* ctx, SolveBufs& B, const double* b_dev,
     CU(cudaMemcpyAsync(z, zeros.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, ctx->stream));
   std::vector<double> big(nrhs, 1e300);
   CU(cudaMemcpyAsync(B.sc.rbest, big.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, ctx->stream));
+  CU(cudaMemsetAsync(B.sc.rerr, 0, sizeof(double) * nrhs, ctx->stream));
   CU(cudaMemsetAsync(B.sc.count, 0, 4 * sizeof(int), ctx->stream));
   CU(cudaMemsetAsync(B.x64.data, 0, field_bytes_per_rhs(DLMA_FP64, Vh) * nrhs, ctx->stream));
   CU(cudaMemsetAsync(B.xl.data, 0, field_bytes(PB, Vh, nrhs), ctx->stream));
@@ -1122,8 +1187,8 @@ static dlma_status solve_finish(dlma_ctx* ctx, SolveBufs& B, double* x_dev, int 
   const dim3 gv((Vh + BX - 1) / BX, nrhs);
   // fold what is left of the low-precision solutions of unconverged rhs
   if (st != DLMA_OK) {
-    k_fold<PB><<<dim3(gv.x, field_vectors(PB, nrhs)), BX, 0, ctx->stream>>>(Vh, nrhs, (double2*)B.x64.data, B.xl.data,
-                                                                           B.sc.scale, B.sc.alive);
+    k_fold<PB, false><<<dim3(gv.x, field_vectors(PB, nrhs)), BX, 0, ctx->stream>>>(
+        Vh, nrhs, (double2*)B.x64.data, B.xl.data, B.sc.scale, B.sc.alive, nullptr, nullptr);
     CHECK_LAUNCH();
   }
   {
@@ -1146,14 +1211,14 @@ static dlma_status solve_finish(dlma_ctx* ctx, SolveBufs& B, double* x_dev, int 
   HopOp d;
   d.own = 2; d.kout = 0; d.p_out = 0; d.active = fm;
   TRY(launch_hop(ctx, d, B.t64o, &xe, B.t64));            // (Dx)_e
-  k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.b_e.data, (const double2*)B.t64.data,
-                                      (double2*)B.bh.data, fm, B.part);
+  k_sub64<DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.b_e.data, (const double2*)B.t64.data,
+                                                 (double2*)B.bh.data, nullptr, fm, B.part);
   CHECK_LAUNCH();
   TRY(rowsum(ctx, B.part, gv.x, nrhs, B.tmpd, 0, fm));
   d.p_out = 1;
   TRY(launch_hop(ctx, d, xe, &B.t64o, B.t64));            // (Dx)_o
-  k_sub64<<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.b_o.data, (const double2*)B.t64.data,
-                                      (double2*)B.bh.data, fm, B.part);
+  k_sub64<DLMA_FP64><<<gv, BX, 0, ctx->stream>>>(Vh, nrhs, (const double2*)B.b_o.data, (const double2*)B.t64.data,
+                                                 (double2*)B.bh.data, nullptr, fm, B.part);
   CHECK_LAUNCH();
   TRY(rowsum(ctx, B.part, gv.x, nrhs, B.tmpd + nrhs, 0, fm));
   std::vector<double> h(2 * nrhs), hr(nrhs);
