@@ -822,17 +822,24 @@ __global__ void __launch_bounds__(256) k_bi_resume(const double2* cpart, const d
   sc.active[j] = 1;
 }
 
-// the shadow residual, the same for every rhs: entries (+-1 +- i), signs from a hash of
-// the entry's index
+// the shadow residual, the same for every rhs: real and imaginary parts spread over
+// (-1, 1) by a hash of the entry's index (the finaliser of MurmurHash3).  A restart keeps
+// it, so it must not be orthogonal to a source: entries (+-1 +- i) were, exactly, for one
+// in four differences of two unit sources, which BiCGStab then gave up to CGNE.
 __global__ void k_bi_shadow(int Vh, float4* r0) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= 6 * Vh) return;
-  unsigned h = (unsigned)e * 0x9e3779b9u;
-  h = (h ^ (h >> 15)) * 0x85ebca6bu;
-  h = (h ^ (h >> 13)) * 0xc2b2ae35u;
-  h ^= h >> 16;
-  const auto sign = [&](int b) { return (h >> b) & 1 ? -1.f : 1.f; };
-  r0[e] = make_float4(sign(0), sign(8), sign(16), sign(24));
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    unsigned h = (2u * (unsigned)e + q + 1u) * 0x9e3779b9u;
+    h = (h ^ (h >> 16)) * 0x85ebca6bu;
+    h = (h ^ (h >> 13)) * 0xc2b2ae35u;
+    h ^= h >> 16;
+    v[2 * q] = ((float)(h & 0xffffu) + 0.5f) * (1.f / 32768.f) - 1.f;
+    v[2 * q + 1] = ((float)(h >> 16) + 0.5f) * (1.f / 32768.f) - 1.f;
+  }
+  r0[e] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
 // updated rhs that restart their search direction: the stagnating ones and those that broke down
@@ -1378,7 +1385,7 @@ static dlma_status solve_batch(dlma_ctx* ctx, const double* b_dev, double* x_dev
 // w0 = Dhat^dag r0 kept beside the shadow residual, (r0, Dhat y) = (w0, y): alpha is known
 // before v = Dhat p and beta before the vector updates, so s is formed in the stencil's
 // epilogue and x, r and p in one pass.  The iteration is bound by memory traffic, so r0
-// and w0 are shared by all right-hand sides (a fixed vector of random signs): 20 vectors
+// and w0 are shared by all right-hand sides (r0: a fixed random vector): 20 vectors
 // move per iteration, 25 with a shadow residual of its own and separate updates.  (The
 // random r0 costs 2 % more iterations than r0 = r.)  Per iteration:
 //   v = Dhat p, s = r - alpha v, (w0, s), (r0, s);  t = Dhat s, (s, t), |t|^2;
