@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(BX) k_bi_restore(int Vh, int nrhs, const doubl
   const int j = blockIdx.y;
   if (!vec_on<P>(j, nrhs, upd)) return;
   double v5[5 * LN] = {};
-  float a5[5 * LN] = {};           // per thread in FP32, as in k_bi_update
+  float wr[LN] = {}, wi[LN] = {};  // (w0, p) per thread in FP32, as in k_bi_update
   if (i < Vh) {
     const size_t so = field_units_per_rhs(P, Vh) * 16 * j;
     bool on[LN], restart[LN], any = false;
@@ -764,18 +764,23 @@ __global__ void __launch_bounds__(BX) k_bi_restore(int Vh, int nrhs, const doubl
           lane_set(p.im, q, yi);
         }
         const float pr = lane_get(p.re, q), pi = lane_get(p.im, q);
-        a5[5 * q] = fmaf(z.re, yr, fmaf(z.im, yi, a5[5 * q]));
-        a5[5 * q + 1] = fmaf(z.re, yi, fmaf(-z.im, yr, a5[5 * q + 1]));
-        a5[5 * q + 2] = fmaf(w.re, pr, fmaf(w.im, pi, a5[5 * q + 2]));
-        a5[5 * q + 3] = fmaf(w.re, pi, fmaf(-w.im, pr, a5[5 * q + 3]));
-        a5[5 * q + 4] = fmaf(yr, yr, fmaf(yi, yi, a5[5 * q + 4]));
+        // (r0, r_l) and |r_l|^2, on which the recursion restarts, in FP64
+        const double zr = z.re, zi = z.im, a = yr, b = yi;
+        v5[5 * q] = fma(zr, a, fma(zi, b, v5[5 * q]));
+        v5[5 * q + 1] = fma(zr, b, fma(-zi, a, v5[5 * q + 1]));
+        v5[5 * q + 4] = fma(a, a, fma(b, b, v5[5 * q + 4]));
+        wr[q] = fmaf(w.re, pr, fmaf(w.im, pi, wr[q]));
+        wi[q] = fmaf(w.re, pi, fmaf(-w.im, pr, wi[q]));
       }
       store_comp<P>((char*)rl + so, Vh, i, k, y);
       if (any) store_comp<P>((char*)pl + so, Vh, i, k, p);
     }
   }
 #pragma unroll
-  for (int e = 0; e < 5 * LN; e++) v5[e] = a5[e];
+  for (int q = 0; q < LN; q++) {
+    v5[5 * q + 2] = wr[q];
+    v5[5 * q + 3] = wi[q];
+  }
   block_sums(v5);
   if (threadIdx.x == 0)
 #pragma unroll
