@@ -970,12 +970,15 @@ static dlma_status check_ready(dlma_ctx* ctx) {
   return DLMA_OK;
 }
 
-// The internal form of a batch of one operator call: FP32 in pairs of right-hand sides once
-// their half as many threads still fill the GPU (Schur application, pairs against single
+// The internal form of a batch of one operator call, whose largest work buffer holds `per`
+// vectors per right-hand side: FP32 in pairs of right-hand sides once their half as many
+// threads still fill the GPU (Schur application, pairs against single
 // vectors: 10^3 x 18, 7 right-hand sides (63000 pairs of site and vector), 23 and 21 us,
-// 24 (216000), 46 and 48; 16^3 x 32, 168, 1.57 and 1.77 ms).
-static int field_prec(const dlma_ctx* ctx, int prec, int nrhs) {
-  return prec == DLMA_FP32 && nrhs > 1 && (size_t)nrhs * ctx->g.Vh >= 100000 ? kFP32x2 : prec;
+// 24 (216000), 46 and 48; 16^3 x 32, 168, 1.57 and 1.77 ms), unless the empty partner of
+// an odd batch takes it above a memory cap.
+static int field_prec(const dlma_ctx* ctx, int prec, int nrhs, int per) {
+  if (prec != DLMA_FP32 || nrhs < 2 || (size_t)nrhs * ctx->g.Vh < 100000) return prec;
+  return ctx->memcap && per * field_bytes(kFP32x2, ctx->g.Vh, nrhs) + 256 > ctx->memcap ? prec : kFP32x2;
 }
 // a caller's canonical FP64 array as a field of the split stencil
 static Field canonical(dlma_ctx* ctx, const double* p, int nrhs, int lay) {
@@ -1011,7 +1014,7 @@ extern "C" dlma_status dlma_apply_Dw(dlma_ctx* ctx, const double* in, double* ou
     CU(cudaStreamSynchronize(ctx->stream));
     return DLMA_OK;
   }
-  const int fp = field_prec(ctx, prec, nrhs), nv = field_vectors(fp, nrhs);
+  const int fp = field_prec(ctx, prec, nrhs, 2), nv = field_vectors(fp, nrhs);
   Field fe, fo, re, ro;
   TRY(field_alloc(ctx, WS_T0, fp, nrhs, &fe));
   TRY(field_alloc(ctx, WS_T1, fp, nrhs, &fo));
@@ -1055,7 +1058,7 @@ extern "C" dlma_status dlma_apply_schur(dlma_ctx* ctx, const double* in, double*
   // few pairs: the split stencil reads and writes the canonical arrays themselves
   const bool direct = hop_split(ctx, prec, nrhs) && disjoint(din, dout, bytes);
   Field fe, tmp, res;
-  const int fp = field_prec(ctx, prec, nrhs);
+  const int fp = field_prec(ctx, prec, nrhs, 1);
   TRY(field_alloc(ctx, WS_T1, fp, nrhs, &tmp));
   if (direct) {
     fe = canonical(ctx, din, nrhs, kLayHalf);
