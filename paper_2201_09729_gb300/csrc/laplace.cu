@@ -969,11 +969,19 @@ static void cheb_coefficients(Eig& E, int d, std::vector<double>& hc, std::vecto
   }
 }
 
-// complex multiply-adds (n m^2 Tn) from which a phase-B product takes the tensor cores
-// instead of double-float (eigensolve, double-float against tensor cores: 18.6 and 17.4 ms
-// on 10^3 x 18 with 40 columns, 9e7; 110 and 96 ms on 16^3 x 32 with 64, 2e9; 1277 and
-// 957 ms on 24^3 x 48 with 128; equal at 2.5e7, 8^3 x 16 with 32)
-constexpr double kTcWork = 5.0e7;
+// Whether phase B's products take the tensor cores instead of double-float: from 5e7
+// complex multiply-adds (n m^2 Tn) on, where they are faster (eigensolve, double-float
+// against tensor cores: 110 and 96 ms on 16^3 x 32 with 64 columns, 2e9; 1277 and 957 ms
+// on 24^3 x 48 with 128; equal at 2.5e7, 8^3 x 16 with 32), as far as the modes come out
+// no less orthonormal.  The digits' error is that of a chunk's largest entry whatever the
+// size, rms of V^dag V - 1 4e-15 ... 6e-15; double-float's grows with the rows per sum,
+// n / nsplit: 3.7e-15 at 375 rows (10^3 x 18, 40 columns), 4.6e-15 at 1263 (20^3 x 8, 48),
+// 5.9e-15 at 1365 (16^3 x 16, 64), 9.3e-15 at 3072 (16^3 x 32, 64), either side of 5e-15
+// between 860 and 1270.  From 4e9 multiply-adds on always.
+static bool tc_products(int n, int m, int Tn, int nsplit) {
+  const double macs = (double)n * m * m * Tn;
+  return macs >= 4.0e9 || (macs >= 5.0e7 && n >= 1300 * nsplit);
+}
 
 static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, double* lam_out,
                              Cx<double>** Xres, int* m_out, int* iters_out, PhaseTimer* pt) {
@@ -1081,9 +1089,8 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   // The FP64 blocks' Gram matrices and rotations run in double-float on the FP32
   // units when the tolerance leaves room for its ~2^-46 rounding.
   E.df = ctx->df_eigs && tol >= 1e-11;
-  // (and from kTcWork multiply-adds per product on the tensor cores; DLMA_EIGS_TC=1 / 0
-  // forces either)
-  E.tc = E.df && (double)E.n * E.m * E.m * E.Tn >= kTcWork;
+  // (and large ones on the tensor cores; DLMA_EIGS_TC=1 / 0 forces either)
+  E.tc = E.df && tc_products(E.n, E.m, E.Tn, E.nsplit);
   // the rotation's digits (every row of the block) have to fit a memory cap
   if (ctx->memcap && tc_min_bytes(E.n, E.m, E.Tn) > ctx->memcap) E.tc = 0;
   if (const char* e = getenv("DLMA_EIGS_TC")) E.tc = E.df && atoi(e) == 1;
