@@ -249,6 +249,7 @@ dlma_status set_err(dlma_ctx* ctx, dlma_status st, const char* fmt, ...);
 
 // work buffer of at least `bytes` in slot `slot` (contents not preserved on growth)
 dlma_status work(dlma_ctx* ctx, int slot, size_t bytes, void** out);
+void work_free(dlma_ctx* ctx, int slot);
 template <class T> dlma_status workT(dlma_ctx* ctx, int slot, size_t count, T** out) {
   void* p;
   dlma_status s = work(ctx, slot, count * sizeof(T), &p);
@@ -369,6 +370,7 @@ dlma_status solve_fields(dlma_ctx* ctx, const double* b_dev, double* x_dev, int 
 dlma_status project_tc(dlma_ctx* ctx, const double2* VT, int N, int Tsel, const double* psi, size_t stride_sites,
                        int site_t0, int nrhs, double2* coeff);
 size_t tc_min_bytes(int R, int N, int T);
+size_t tc_block_bytes(const dlma_ctx* ctx, int n, int m, int T);
 // sum over kappa of conj(B_k) A_r per timeslice on the tensor cores (tcproj.cu):
 // omode 1 writes out[t][k][r], omode 2 out[t][r][k]
 dlma_status tc_block_product(dlma_ctx* ctx, int omode, const double2* a_src, size_t a_st, size_t a_sr, size_t a_sk,

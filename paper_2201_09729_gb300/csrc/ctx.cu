@@ -43,6 +43,15 @@ dlma_status work(dlma_ctx* ctx, int slot, size_t bytes, void** out) {
   return DLMA_OK;
 }
 
+// give a work buffer back (its users on the stream have to be done)
+void work_free(dlma_ctx* ctx, int slot) {
+  DevBuf& b = ctx->wb[slot];
+  if (b.p) cudaFree(b.p);
+  ctx->work_bytes -= b.bytes;
+  b.p = nullptr;
+  b.bytes = 0;
+}
+
 dlma_status field_alloc(dlma_ctx* ctx, int slot, int prec, int nrhs, Field* f) {
   size_t per = field_bytes_per_rhs(prec, ctx->g.Vh);
   void* p;
@@ -498,12 +507,7 @@ extern "C" dlma_status dlma_release_workspace(dlma_ctx* ctx) {
   if (!ctx) return DLMA_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaStreamSynchronize(ctx->stream);
-  for (int i = 0; i < WS_COUNT; i++) {
-    if (ctx->wb[i].p) cudaFree(ctx->wb[i].p);
-    ctx->wb[i].p = nullptr;
-    ctx->wb[i].bytes = 0;
-  }
-  ctx->work_bytes = 0;
+  for (int i = 0; i < WS_COUNT; i++) work_free(ctx, i);
   return DLMA_OK;
 }
 

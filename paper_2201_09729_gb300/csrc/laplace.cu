@@ -772,6 +772,16 @@ static dlma_status lap(Eig& E, const Cx<R>* in, const Cx<R>* prev, const Cx<floa
   return DLMA_OK;
 }
 
+// whether a tensor-core product found no memory for its digits: their buffers are given
+// back and double-float takes this product and the following ones
+static bool no_digits(Eig& E, dlma_status st) {
+  if (st != DLMA_ERR_OOM) return false;
+  E.tc = 0;
+  cudaStreamSynchronize(E.ctx->stream);
+  for (int s : {WS_TC_A, WS_TC_B, WS_TC_E, WS_TC_P}) work_free(E.ctx, s);
+  return true;
+}
+
 // out = X^dag Y per timeslice; herm = 1 when the result is hermitian by construction
 template <class R> static dlma_status gram(Eig& E, const Cx<R>* X, const Cx<R>* Y, double2* out, int herm) {
   dlma_ctx* ctx = E.ctx;
@@ -780,9 +790,11 @@ template <class R> static dlma_status gram(Eig& E, const Cx<R>* X, const Cx<R>* 
   phase(E, kPhOrtho);
   const dim3 grid(tiles, E.nsplit, E.Tn);
   if constexpr (sizeof(R) == 8) {
-    if (E.tc)   // G[t][i][j] = sum_k conj(X[k][i]) Y[k][j]: rows = columns of Y, modes = columns of X
-      return tc_block_product(ctx, 1, (const double2*)Y, (size_t)E.n * E.m, 1, (size_t)E.m, E.m,
-                              (const double2*)X, 0, E.m, E.n, E.Tn, out);
+    if (E.tc) {   // G[t][i][j] = sum_k conj(X[k][i]) Y[k][j]: rows = columns of Y, modes = columns of X
+      const dlma_status st = tc_block_product(ctx, 1, (const double2*)Y, (size_t)E.n * E.m, 1, (size_t)E.m, E.m,
+                                              (const double2*)X, 0, E.m, E.n, E.Tn, out);
+      if (!no_digits(E, st)) return st;
+    }
     if (E.df) k_gram<R, df><<<grid, 256, 0, ctx->stream>>>(X, Y, E.n, E.m, E.nsplit, herm, E.part);
     else k_gram<R, R><<<grid, 256, 0, ctx->stream>>>(X, Y, E.n, E.m, E.nsplit, herm, E.part);
   } else {
@@ -804,9 +816,11 @@ template <class R> static dlma_status rotate(Eig& E, const Cx<R>* X, Cx<R>* Z) {
   phase(E, kPhOrtho);
   const dim3 grid((E.n + RT - 1) / RT, (E.m + RT - 1) / RT, E.Tn);
   if constexpr (sizeof(R) == 8) {
-    if (E.tc)   // Z[t][k][j] = sum_l X[k][l] C[l][j]: rows = rows of X, modes = conj of the columns of C
-      return tc_block_product(ctx, 2, (const double2*)X, (size_t)E.n * E.m, (size_t)E.m, 1, E.n, E.C, 1, E.m, E.m,
-                              E.Tn, (double2*)Z);
+    if (E.tc) {   // Z[t][k][j] = sum_l X[k][l] C[l][j]: rows = rows of X, modes = conj of the columns of C
+      const dlma_status st = tc_block_product(ctx, 2, (const double2*)X, (size_t)E.n * E.m, (size_t)E.m, 1, E.n, E.C, 1,
+                                              E.m, E.m, E.Tn, (double2*)Z);
+      if (!no_digits(E, st)) return st;
+    }
     if (E.df) k_rotate<R, df><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
     else k_rotate<R, R><<<grid, 256, 0, ctx->stream>>>(X, E.C, E.n, E.m, Z);
   } else {
@@ -1091,8 +1105,15 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   E.df = ctx->df_eigs && tol >= 1e-11;
   // (and large ones on the tensor cores; DLMA_EIGS_TC=1 / 0 forces either)
   E.tc = E.df && tc_products(E.n, E.m, E.Tn, E.nsplit);
-  // the rotation's digits (every row of the block) have to fit a memory cap
+  // the rotation's digits (every row of the block) have to fit a memory cap, and all of
+  // them (up to 4 GB) the device beside the modes to come (cached, and on their way out)
   if (ctx->memcap && tc_min_bytes(E.n, E.m, E.Tn) > ctx->memcap) E.tc = 0;
+  if (E.tc) {
+    size_t freeb = 0, totb = 0;
+    CU(cudaMemGetInfo(&freeb, &totb));
+    const size_t modes = 2 * (size_t)N * ctx->g.T * E.n * sizeof(double2);
+    if (tc_block_bytes(ctx, E.n, E.m, E.Tn) + modes > freeb - freeb / 64) E.tc = 0;
+  }
   if (const char* e = getenv("DLMA_EIGS_TC")) E.tc = E.df && atoi(e) == 1;
   Cx<double> *X64 = E.D0, *W64 = E.D1, *Y64 = E.D2;
   // phase A's last Ritz pairs were not fetched, or hold refilled (random) columns

@@ -466,33 +466,50 @@ int chunk_split(long tiles, int Q) {
 
 }  // namespace
 
+// How run_products works: chunk groups, blocks per tile and the bytes of its work buffers
+struct Plan {
+  int Q, RT, MB, Qg, ks;
+  size_t a, b, e, p;             // WS_TC_A, WS_TC_B, WS_TC_E, WS_TC_P
+};
+static Plan make_plan(const dlma_ctx* ctx, int T, int R, int N, int K, size_t out_count) {
+  Plan P;
+  P.Q = (K + CK - 1) / CK;
+  P.RT = (R + TM - 1) / TM;
+  P.MB = (N + 31) / 32;
+  // digit bytes per chunk of every timeslice: A (RT tiles of rows) and B (MB tiles of modes)
+  const size_t per_chunk = (size_t)T * NBK * S * ((size_t)P.RT * A_TILE + (size_t)P.MB * B_TILE);
+  size_t budget = (size_t)4 << 30;
+  if (ctx->memcap) budget = std::min(budget, (size_t)ctx->memcap / 4);
+  P.Qg = (int)std::max<size_t>(1, std::min<size_t>((size_t)P.Q, budget / per_chunk));
+  P.Qg = (P.Q + (P.Q + P.Qg - 1) / P.Qg - 1) / ((P.Q + P.Qg - 1) / P.Qg);       // equal groups
+  P.ks = chunk_split((long)T * P.RT * P.MB, P.Qg);
+  // the partial results keep to a quarter of a memory cap, like the digits
+  if (ctx->memcap) P.ks = (int)std::max<size_t>(1, std::min<size_t>(P.ks, ctx->memcap / 4 / (out_count * 16)));
+  P.a = (size_t)T * P.RT * P.Qg * NBK * S * A_TILE;
+  P.b = (size_t)T * P.MB * P.Qg * NBK * S * B_TILE;
+  P.e = (size_t)T * (P.Qg + 1) * (P.RT * TM + P.MB * TN) * sizeof(int);
+  P.p = P.ks > 1 ? (size_t)P.ks * out_count * 16 : 0;
+  return P;
+}
+
 // Shared by the projection and the eigensolver's block products: digit buffers, the
 // chunk groups and the products; slice_a launches the row slicer.
 template <class SliceA>
 static dlma_status run_products(dlma_ctx* ctx, int T, int R, int N, int K, const double2* b_src, int b_conj, int omode,
                                 double2* out, size_t out_count, const char* what, const SliceA& slice_a) {
-  const int Q = (K + CK - 1) / CK;
-  const int RT = (R + TM - 1) / TM, MB = (N + 31) / 32;
-  // digit bytes per chunk of every timeslice: A (RT tiles of rows) and B (MB tiles of modes)
-  const size_t per_chunk = (size_t)T * NBK * S * ((size_t)RT * A_TILE + (size_t)MB * B_TILE);
-  size_t budget = (size_t)4 << 30;
-  if (ctx->memcap) budget = std::min(budget, (size_t)ctx->memcap / 4);
-  int Qg = (int)std::max<size_t>(1, std::min<size_t>((size_t)Q, budget / per_chunk));
-  Qg = (Q + (Q + Qg - 1) / Qg - 1) / ((Q + Qg - 1) / Qg);       // equal groups
-  int ks = chunk_split((long)T * RT * MB, Qg);
-  // the partial results keep to a quarter of a memory cap, like the digits
-  if (ctx->memcap) ks = (int)std::max<size_t>(1, std::min<size_t>(ks, ctx->memcap / 4 / (out_count * 16)));
+  const Plan P = make_plan(ctx, T, R, N, K, out_count);
+  const int Q = P.Q, RT = P.RT, MB = P.MB, Qg = P.Qg, ks = P.ks;
   uint8_t *As, *Bs;
   int *eA, *eB;
-  TRY(workT(ctx, WS_TC_A, (size_t)T * RT * Qg * NBK * S * A_TILE, &As));
-  TRY(workT(ctx, WS_TC_B, (size_t)T * MB * Qg * NBK * S * B_TILE, &Bs));
-  TRY(workT(ctx, WS_TC_E, (size_t)T * (Qg + 1) * (RT * TM + MB * TN), &eA));
+  TRY(workT(ctx, WS_TC_A, P.a, &As));
+  TRY(workT(ctx, WS_TC_B, P.b, &Bs));
+  TRY(workT(ctx, WS_TC_E, P.e / sizeof(int), &eA));
   eB = eA + (size_t)T * Qg * RT * TM;
   int* eAmax = eB + (size_t)T * Qg * MB * TN;
   int* eBmax = eAmax + (size_t)T * RT * TM;
   const size_t nref = (size_t)T * (RT * TM + MB * TN);
   double* parts = (double*)out;
-  if (ks > 1) TRY(workT(ctx, WS_TC_P, (size_t)ks * out_count * 2, &parts));
+  if (ks > 1) TRY(workT(ctx, WS_TC_P, P.p / sizeof(double), &parts));
   int* err = ctx->flag + 8;
   CU(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   static bool attr_set[64] = {false};
@@ -546,6 +563,17 @@ dlma_status project_tc(dlma_ctx* ctx, const double2* VT, int N, int Tsel, const 
 // that run_products works with)
 size_t tc_min_bytes(int R, int N, int T) {
   return (size_t)T * NBK * S * ((size_t)((R + TM - 1) / TM) * A_TILE + (size_t)((N + 31) / 32) * B_TILE);
+}
+
+// device memory that the products below of n x m blocks on T timeslices (Gram matrices and
+// rotations) add to the work buffers held
+size_t tc_block_bytes(const dlma_ctx* ctx, int n, int m, int T) {
+  const Plan G = make_plan(ctx, T, m, m, n, (size_t)T * m * m), Z = make_plan(ctx, T, n, m, m, (size_t)T * n * m);
+  const auto grow = [&](int slot, size_t g, size_t z) {
+    const size_t need = std::max(g, z), held = ctx->wb[slot].bytes;
+    return need > held ? need - held : 0;
+  };
+  return grow(WS_TC_A, G.a, Z.a) + grow(WS_TC_B, G.b, Z.b) + grow(WS_TC_E, G.e, Z.e) + grow(WS_TC_P, G.p, Z.p);
 }
 
 // Block products of the eigensolver's FP64 phase on the tensor cores, with the same
