@@ -149,8 +149,8 @@ struct dlma_ctx {
   // in double-float (dfloat.cuh) for tol >= 1e-11; DLMA_DF_EIGS=0 at context
   // creation keeps FP64 arithmetic
   int df_eigs = 1;
-  // solve batch size per precision, chosen by autotune_batch (valid up to batch_tuned_nb)
-  int batch_rhs[3] = {0, 0, 0}, batch_tuned_nb[3] = {0, 0, 0}, batch_tuned[3] = {0, 0, 0};
+  // solve batch size per field form, chosen by autotune_batch (valid up to batch_tuned_nb)
+  int batch_rhs[4] = {0, 0, 0, 0}, batch_tuned_nb[4] = {0, 0, 0, 0}, batch_tuned[4] = {0, 0, 0, 0};
 
   bool have_gauge = false, have_params = false;
   double m0 = 0, csw = 0;

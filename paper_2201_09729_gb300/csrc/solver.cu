@@ -1526,33 +1526,37 @@ static dlma_status solve_one_batch(dlma_ctx* ctx, const double* b, double* x, in
   return all ? DLMA_OK : set_err(ctx, DLMA_ERR_NOT_CONVERGED, "true residual above tolerance");
 }
 
+// the form of the fields that a batch of n right-hand sides iterates on
+static int solve_form(const dlma_ctx* ctx, dlma_prec prec, int n) {
+  return prec == DLMA_FP32 && ctx->solver == DLMA_SOLVER_BICGSTAB && bicg_pairs(ctx, n) ? kFP32x2 : prec;
+}
+
 // Batch-size autotuner: the stencil's time per right-hand side at the largest
-// batch memory allows (nb) and at nb / 2, nb / 4, measured once per precision on
-// the context's own lattice (the choice is kept until a larger batch fits); the
+// batch memory allows (nb) and at nb / 2, nb / 4, each in the form that a batch of that
+// size iterates on, measured once per form of the largest on the context's own lattice
+// (the choice is kept until a larger batch fits); the
 // solves then run in batches of the cheapest size.  Links and clover are shared
 // by every right-hand side of a batch, so larger batches usually win; the
 // measurement decides where L2 reuse or occupancy says otherwise.
 static dlma_status autotune_batch(dlma_ctx* ctx, dlma_prec prec, int nb, int* out) {
-  if (ctx->batch_tuned[prec] && nb <= ctx->batch_tuned_nb[prec]) {
-    *out = std::min(nb, ctx->batch_rhs[prec]);
+  const int key = solve_form(ctx, prec, nb);
+  if (ctx->batch_tuned[key] && nb <= ctx->batch_tuned_nb[key]) {
+    *out = std::min(nb, ctx->batch_rhs[key]);
     return DLMA_OK;
   }
-  // the fields that the solve iterates on
-  const int fp = prec == DLMA_FP32 && ctx->solver == DLMA_SOLVER_BICGSTAB && bicg_pairs(ctx, nb) ? kFP32x2 : prec;
-  Field in, tmp, res;
-  TRY(field_alloc(ctx, WS_CG_RHS, fp, nb, &in));
-  TRY(field_alloc(ctx, WS_CG_TMP, fp, nb, &tmp));
-  TRY(field_alloc(ctx, WS_CG_Z, fp, nb, &res));
-  CU(cudaMemsetAsync(in.data, 0, field_bytes(fp, ctx->g.Vh, nb), ctx->stream));
-  TRY(autotune_hop(ctx, fp, in, tmp, res));
   cudaEvent_t e0, e1;
   CU(cudaEventCreate(&e0));
   CU(cudaEventCreate(&e1));
   int best_k = nb;
   double best = 1e300;
   for (int k : {nb, ((nb + 1) / 2 + 1) & ~1, ((nb + 3) / 4 + 1) & ~1}) {
-    Field a = in, t = tmp, r = res;
-    a.nrhs = t.nrhs = r.nrhs = k;
+    const int fp = solve_form(ctx, prec, k);
+    Field a, t, r;
+    TRY(field_alloc(ctx, WS_CG_RHS, fp, k, &a));
+    TRY(field_alloc(ctx, WS_CG_TMP, fp, k, &t));
+    TRY(field_alloc(ctx, WS_CG_Z, fp, k, &r));
+    CU(cudaMemsetAsync(a.data, 0, field_bytes(fp, ctx->g.Vh, k), ctx->stream));
+    TRY(autotune_hop(ctx, fp, a, t, r));
     float tmin = 1e30f;
     for (int rep = 0; rep < 3; rep++) {
       CU(cudaEventRecord(e0, ctx->stream));
@@ -1568,9 +1572,9 @@ static dlma_status autotune_batch(dlma_ctx* ctx, dlma_prec prec, int nb, int* ou
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  ctx->batch_rhs[prec] = best_k;
-  ctx->batch_tuned_nb[prec] = nb;
-  ctx->batch_tuned[prec] = 1;
+  ctx->batch_rhs[key] = best_k;
+  ctx->batch_tuned_nb[key] = nb;
+  ctx->batch_tuned[key] = 1;
   *out = std::min(nb, best_k);
   return DLMA_OK;
 }
