@@ -38,10 +38,6 @@
 
 namespace {
 
-template <class R> struct LinkT;
-template <> struct LinkT<double> { typedef double2 T; };
-template <> struct LinkT<float> { typedef float4 T; };
-
 __device__ __forceinline__ void load_link3(const double2* __restrict__ U, int k, size_t s, size_t V, Cx<double> u[3][3]) {
 #pragma unroll
   for (int q = 0; q < 9; q++) {
@@ -730,6 +726,7 @@ struct Eig {
   Cx<double> *D0, *D1, *D2;      // FP64 blocks
   double2 *G, *H, *C, *part, *gwork;
   double *theta, *res, *coef, *scol;
+  const double* plain;           // coefficients of the plain operator: coef slot `degree`
   int* dropped;                  // [0] dropped directions of the last small_rr, [1 + 2t + {0,1}] Jacobi sweeps
   bool refilled = false;         // the last fetch refilled dropped columns
   PhaseTimer* pt = nullptr;      // phases: kPhMatvec, kPhOrtho, kPhHost
@@ -746,28 +743,28 @@ static inline void phase(Eig& E, int p) {
   if (E.pt) E.pt->enter(p);
 }
 
-template <class R> static const typename LinkT<R>::T* links(dlma_ctx* ctx);
-template <> const double2* links<double>(dlma_ctx* ctx) { return ctx->U3; }
-template <> const float4* links<float>(dlma_ctx* ctx) { return ctx->U3f; }
-
-template <class R>
-static dlma_status lap(Eig& E, const Cx<R>* in, const Cx<R>* prev, const Cx<float>* rin, const double* scol,
-                       Cx<R>* out, const double* coef) {
+// one step of the FP32 filter (k_lap_z): out = alpha (A in) + beta in + gamma prev +
+// alpha s rin, two columns per thread (m is even: one 128-bit access per pair)
+static dlma_status lap_filter(Eig& E, const Cx<float>* in, const Cx<float>* prev, const Cx<float>* rin,
+                              const double* scol, Cx<float>* out, const double* coef) {
   dlma_ctx* ctx = E.ctx;
-  const size_t total = (size_t)E.Tn * ctx->g.Vs * E.m;
-  if (total >= (1ull << 31)) return set_err(ctx, DLMA_ERR_INVALID_ARG, "eigensolver block above 2^31 entries");
   phase(E, kPhMatvec);
-  // m is even; FP32: two columns per thread (one 128-bit access per pair, links
-  // rebuilt once per pair); FP64 is bound by its arithmetic and keeps one (a
-  // double-float FP64 matvec, 170 registers and a split of every loaded value, was
-  // slower)
-  if constexpr (sizeof(R) == 4) {
-    const LapTiling t = lap_tiling(ctx->g.L, E.m, E.Tn);
-    k_lap_z<<<dim3((unsigned)(t.nx * t.ny * t.nz * t.groups), E.Tn), 256, 0, ctx->stream>>>(
-        ctx->g, E.t0, E.m, t, links<R>(ctx), in, prev, rin, scol, out, coef);
-  } else {
-    k_lap<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(ctx->g, E.t0, E.Tn, E.m, links<R>(ctx), in, out);
-  }
+  const LapTiling t = lap_tiling(ctx->g.L, E.m, E.Tn);
+  k_lap_z<<<dim3((unsigned)(t.nx * t.ny * t.nz * t.groups), E.Tn), 256, 0, ctx->stream>>>(
+      ctx->g, E.t0, E.m, t, ctx->U3f, in, prev, rin, scol, out, coef);
+  CHECK_LAUNCH();
+  return DLMA_OK;
+}
+// out = A in.  FP32: a filter step with the coefficients of the plain operator.  FP64 is
+// bound by its arithmetic and takes one column per thread (a double-float matvec, 170
+// registers and a split of every loaded value, was slower).
+static dlma_status lap(Eig& E, const Cx<float>* in, Cx<float>* out) {
+  return lap_filter(E, in, nullptr, nullptr, nullptr, out, E.plain);
+}
+static dlma_status lap(Eig& E, const Cx<double>* in, Cx<double>* out) {
+  dlma_ctx* ctx = E.ctx;
+  phase(E, kPhMatvec);
+  k_lap<<<(unsigned)((E.blk / 3 + 255) / 256), 256, 0, ctx->stream>>>(ctx->g, E.t0, E.Tn, E.m, ctx->U3, in, out);
   CHECK_LAUNCH();
   return DLMA_OK;
 }
@@ -869,9 +866,8 @@ template <class R> static dlma_status resid(Eig& E, const Cx<R>* X, const Cx<R>*
 
 // Rayleigh-Ritz of the block Y: W = A Y, then X <- Y C, AX <- W C, residuals (and R = AX - X Theta in FP32)
 template <class R>
-static dlma_status rayleigh_ritz(Eig& E, Cx<R>* Y, Cx<R>* W, Cx<R>* Xout, Cx<R>* AXout, Cx<float>* Rout,
-                                 const double* coef_plain) {
-  TRY(lap<R>(E, Y, nullptr, nullptr, nullptr, W, coef_plain));
+static dlma_status rayleigh_ritz(Eig& E, Cx<R>* Y, Cx<R>* W, Cx<R>* Xout, Cx<R>* AXout, Cx<float>* Rout) {
+  TRY(lap(E, Y, W));
   TRY(gram<R>(E, Y, Y, E.G, 1));
   TRY(gram<R>(E, Y, W, E.H, 1));
   TRY(small_rr<R>(E));
@@ -1056,7 +1052,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   for (int t = 0; t < Tn; t++) hc[(size_t)d * 3 * Tn + 3 * t] = 1.0;
   phase(E, kPhHost);
   CU(cudaMemcpyAsync(E.coef, hc.data(), sizeof(double) * ncoef, cudaMemcpyHostToDevice, ctx->stream));
-  const double* plain = E.coef + (size_t)d * 3 * Tn;
+  E.plain = E.coef + (size_t)d * 3 * Tn;
 
   // ---- phase A: FP32 ----
   phase(E, kPhOrtho);
@@ -1064,7 +1060,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   CHECK_LAUNCH();
   // three FP32 blocks rotate: p3[0] = Ritz vectors X, p3[1], p3[2] free; F3 holds A X
   Cx<float>* p3[3] = {E.F0, E.F1, E.F2};
-  TRY(rayleigh_ritz<float>(E, p3[1], p3[2], p3[0], E.F3, nullptr, plain));
+  TRY(rayleigh_ritz<float>(E, p3[1], p3[2], p3[0], E.F3, nullptr));
   double worst = 1;
   int it = 0;
   const int maxA = 60, maxB = 40;
@@ -1084,16 +1080,16 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
     phase(E, kPhHost);
     CU(cudaMemcpyAsync(E.coef, hc.data(), sizeof(double) * ncoef, cudaMemcpyHostToDevice, ctx->stream));
     Cx<float>*prev = p3[0], *cur = p3[1], *nxt = p3[2];
-    TRY(lap<float>(E, prev, nullptr, nullptr, nullptr, cur, E.coef));
+    TRY(lap_filter(E, prev, nullptr, nullptr, nullptr, cur, E.coef));
     for (int k = 2; k <= dA; k++) {
-      TRY(lap<float>(E, cur, prev, nullptr, nullptr, nxt, E.coef + (size_t)(k - 1) * 3 * Tn));
+      TRY(lap_filter(E, cur, prev, nullptr, nullptr, nxt, E.coef + (size_t)(k - 1) * 3 * Tn));
       Cx<float>* t = prev;
       prev = cur;
       cur = nxt;
       nxt = t;
     }
     // cur holds the filtered block; prev and nxt are free (one of them held X)
-    TRY(rayleigh_ritz<float>(E, cur, prev, nxt, E.F3, nullptr, plain));
+    TRY(rayleigh_ritz<float>(E, cur, prev, nxt, E.F3, nullptr));
     p3[0] = nxt;
     p3[1] = cur;
     p3[2] = prev;
@@ -1135,9 +1131,9 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
   // refill the block is first re-diagonalised in FP64.
   E.drop_rel = 1e-24;
   if (rr_first) {
-    TRY(rayleigh_ritz<double>(E, Y64, W64, X64, Y64, R32, plain));
+    TRY(rayleigh_ritz<double>(E, Y64, W64, X64, Y64, R32));
   } else {
-    TRY(lap<double>(E, X64, nullptr, nullptr, nullptr, Y64, plain));
+    TRY(lap(E, X64, Y64));
     TRY(resid<double>(E, X64, Y64, R32));
   }
   bool conv = false;
@@ -1158,7 +1154,7 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
                                                                              E.blk, ec);
     CHECK_LAUNCH();
     for (int k = 2; k <= dB; k++) {
-      TRY(lap<float>(E, ec, em, R32, E.scol + (size_t)(k - 1) * Tn * m, en, E.coef + (size_t)(k - 1) * 3 * Tn));
+      TRY(lap_filter(E, ec, em, R32, E.scol + (size_t)(k - 1) * Tn * m, en, E.coef + (size_t)(k - 1) * 3 * Tn));
       Cx<float>* t = em ? em : spare;
       em = ec;
       ec = en;
@@ -1170,12 +1166,14 @@ static dlma_status eig_batch(dlma_ctx* ctx, int t0, int Tn, int N, double tol, d
                                                                         (size_t)E.n * m, m, E.blk, Y64);
     CHECK_LAUNCH();
     // Rayleigh-Ritz of Y64: W64 = A Y64; X64 <- Y64 C; AX into W... (use X64 as output: Y64 and W64 are inputs)
-    TRY(lap<double>(E, Y64, nullptr, nullptr, nullptr, W64, plain));
+    TRY(lap(E, Y64, W64));
     TRY(gram<double>(E, Y64, Y64, E.G, 1));
     TRY(gram<double>(E, Y64, W64, E.H, 1));
     TRY(small_rr<double>(E));
     TRY(rotate<double>(E, Y64, X64));
-    TRY(lap<double>(E, X64, nullptr, nullptr, nullptr, Y64, plain));   // A X, fresh (cheaper than W C)
+    // A X afresh in FP64: W C by the same product would add that one's rounding (some 1e-13
+    // of |W|) to the residual (24^3 x 48, 128 columns: 30 ms; a tensor-core product 12 ms)
+    TRY(lap(E, X64, Y64));
     TRY(resid<double>(E, X64, Y64, R32));
   }
   if (!conv) {
