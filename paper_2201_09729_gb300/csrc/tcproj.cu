@@ -16,9 +16,11 @@
 // two values is sum_{i,j} d_i d'_j 2^(ex + ey - 14 - 8 (i + j)); the pairs with
 // i + j <= 5 are kept (21 of 36), grouped by class c = i + j (6 classes).  A class sum
 // over one chunk is an integer below (c + 1) 256 128^2 = (c + 1) 2^22: up to class 3 the
-// tensor core's FP32 accumulation of the bf16 products is exact, and in the last two
-// its rounding weighs less than 2^-56 of the largest term.  Each class is scaled by its
-// power of two and added to a double-float (hi, lo) accumulator.  The result carries
+// tensor core's FP32 accumulation of the bf16 products is exact.  In the last two a sum
+// whose digits are all large and of one sign passes 2^24, where an accumulation loses up
+// to 2 units: in class 4 (units of 2^-32) the last 16 of 80, 2^-49 of the largest chunk sum
+// 2^22, in class 5 (units of 2^-40) the last 32 of 96, 2^-56 of it.  Each class is scaled by
+// its power of two and added to a double-float (hi, lo) accumulator.  The result carries
 // about 47 bits: relative to max |x| of a chunk the digits lose 2^-48.
 // (Digits of 6 bits, 8 per value, need 36 products and a third more digit traffic.)
 //
