@@ -691,7 +691,9 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   const bool cgu = op.cg_x != nullptr && op.hop;
   const bool epi = op.dot_part != nullptr && op.hop && op.own == 2 && !op.kout && !op.g5_hop;
   const bool bis = epi && op.bis_r != nullptr, dot = epi && !bis;
-  if (bis && (op.norm_part || (P != DLMA_FP32 && P != kFP32x2)))
+  // the forms that are compiled: both epilogues in FP32, DOT with |out|^2 and BIS without,
+  // and the CG update on single vectors
+  if ((epi && ((P != DLMA_FP32 && P != kFP32x2) || bis == (op.norm_part != nullptr))) || (cgu && P == kFP32x2))
     return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil epilogue");
   const int nr = (P == DLMA_FP32 && !cgu && !epi) ? ctx->hop_nr[P] : 1;
   a.site0 = op.nsites >= 0 ? op.site0 : 0;
@@ -706,14 +708,10 @@ dlma_status launch_hop(dlma_ctx* ctx, const HopOp& op, const Field& in, const Fi
   if (nblocks_out) *nblocks_out = a.ntiles;
   cudaStream_t st = ctx->stream;
   if (dot) {
-    // Schur step B with the DOT epilogue (and |out|^2 when norm_part is set)
-    const bool nrm = op.norm_part != nullptr;
-#define LD(PP, NRR, LL) \
-  (nrm ? k_hop<PP, NRR, false, false, 2, false, true, true, LL, false, true><<<grid, blk, 0, st>>>(a) \
-       : k_hop<PP, NRR, false, false, 2, false, true, false, LL, false, true><<<grid, blk, 0, st>>>(a))
-    if (P == DLMA_FP32) { if (a.l18) LD(DLMA_FP32, 1, true); else LD(DLMA_FP32, 1, false); }
-    else if (P == kFP32x2) { if (a.l18) LD(kFP32x2, 1, true); else LD(kFP32x2, 1, false); }
-    else return set_err(ctx, DLMA_ERR_INVALID_ARG, "stencil epilogue");
+    // Schur step B with the DOT epilogue and |out|^2
+#define LD(PP, LL) k_hop<PP, 1, false, false, 2, false, true, true, LL, false, true><<<grid, blk, 0, st>>>(a)
+    if (P == DLMA_FP32) { if (a.l18) LD(DLMA_FP32, true); else LD(DLMA_FP32, false); }
+    else { if (a.l18) LD(kFP32x2, true); else LD(kFP32x2, false); }
 #undef LD
   } else if (bis) {
 #define LB(PP, LL) k_hop<PP, 1, false, false, 2, false, true, false, LL, false, false, true><<<grid, blk, 0, st>>>(a)

@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(256, 2) k_lap_z(Geom g, int t0, int m, LapTili
   if (site >= L.px * L.py || x >= g.L || y >= g.L || 2 * pair >= m) return;
   const int z0 = bz * L.zlen, z1 = min(g.L, z0 + L.zlen);
   const int j0 = 2 * pair, plane = g.L * g.L;
-  const float alpha = (float)coef[3 * tl], beta = (float)coef[3 * tl + 1], gamma = (float)coef[3 * tl + 2];
+  const float alpha = (float)coef[3 * tl], gamma = (float)coef[3 * tl + 2];
   const size_t row0 = (size_t)tl * g.Vs;                   // first site of the block's timeslice
   const size_t s0 = (size_t)(t0 + tl) * g.Vs;              // ... and of the links'
   const int xf = x + 1 == g.L ? 0 : x + 1, xb = x == 0 ? g.L - 1 : x - 1;

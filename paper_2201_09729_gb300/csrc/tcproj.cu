@@ -87,8 +87,6 @@ __device__ __forceinline__ void digits(double x, int e, float (&d)[S]) {
   for (int i = 2; i < S; i++) d[i] = __uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7440 + 5 - i)) - 8388736.f;
 }
 
-__device__ __forceinline__ int warp_max_int(int v) { return __reduce_max_sync(0xffffffffu, v); }
-
 // 2^e as a float (exact for -126 <= e <= 127, 0 below)
 __device__ __forceinline__ float pow2f(int e) {
   return e < -126 ? 0.f : (e > 127 ? __int_as_float(0x7f800000) : __int_as_float((e + 127) << 23));
