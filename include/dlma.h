@@ -184,9 +184,9 @@ dlma_status dlma_solve(dlma_ctx* ctx, const double* b, double* x, int nrhs, doub
  * changes the reported residual by less than 0.05 (tol / 2), an update subtracts the
  * FP32 operator's image of the FP32 solution increment from the last residual instead
  * of applying the FP64 operator to x: the errors of doing so, bounded by
- * |Dhat| (2 eps32 |increment| + eps64 / 2 |x|) and added up since the last FP64
- * evaluation, have to stay within 0.05 (tol / 2) |b| (CGNE with FP32 vectors does the
- * same).  The shadow residual is a fixed random vector.  Two operator
+ * |Dhat| (2 eps32 |increment| + eps64 / 2 |x|), links off SU(3) counted in, and added up
+ * since the last FP64 evaluation, have to stay within 0.05 (tol / 2) |b| (CGNE with FP32
+ * vectors does the same).  The shadow residual is a fixed random vector.  Two operator
  * applications per iteration and about half as many as CGNE needs on these
  * systems.  Right-hand sides it leaves above the tolerance are solved again
  * with CGNE in the same call; their info sums both iteration counts.

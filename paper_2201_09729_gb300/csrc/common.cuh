@@ -154,7 +154,9 @@ struct dlma_ctx {
 
   bool have_gauge = false, have_params = false;
   double m0 = 0, csw = 0;
+  double su3_defect[2] = {0, 0};       // largest |U U^dag - 1| and third-row defect of the links (set_gauge)
   double schur_norm = 0;               // bound of |Dhat| (set_params)
+  double schur_err32 = 0;              // bound of |Dhat x - FP32 Dhat x| / |x|
   int solver = DLMA_SOLVER_BICGSTAB;   // Krylov method of the FP32 inner solves
   // generations of the gauge field and of the cached modes: a checkpoint taken
   // under one generation is stale under the next

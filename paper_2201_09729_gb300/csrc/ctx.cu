@@ -122,10 +122,44 @@ __device__ __forceinline__ M3<double> load_can(const double2* U, int s, int mu) 
   return m;
 }
 
+// *p = max(*p, v) for a non-negative v (those order like their bits; few sites exceed the
+// maximum so far)
+__device__ __forceinline__ void max_to(double v, unsigned long long* p) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  if (b > *(volatile unsigned long long*)p) atomicMax(p, b);
+}
+// largest row sum of |A_ij|: a bound of the hermitian block's norm
+__device__ double row_sum_norm(const Cx<double> A[6][6]) {
+  double m = 0;
+  for (int i = 0; i < 6; i++) {
+    double s = 0;
+    for (int j = 0; j < 6; j++) s += sqrt(norm2(A[i][j]));
+    m = fmax(m, s);
+  }
+  return m;
+}
+// how far a link (rows e[0..2], e[3..5], e[6..8]) is from SU(3): d[0] = |U U^dag - 1|
+// (Frobenius), d[1] = |row 2 - conj(row 0 x row 1)|, which the 12-real forms drop
+__device__ void su3_defect(const double2 e[9], double d[2]) {
+  M3<double> u;
+  for (int k = 0; k < 9; k++) u.a[k / 3][k % 3] = cx<double>(e[k].x, e[k].y);
+  const M3<double> w = mmul(u, mdag(u));
+  double s = 0, t = 0;
+  for (int i = 0; i < 3; i++)
+    for (int j = 0; j < 3; j++) s += norm2(w.a[i][j] - cx<double>(i == j ? 1.0 : 0.0, 0.0));
+  for (int c = 0; c < 3; c++) {
+    const int a = (c + 1) % 3, b = (c + 2) % 3;
+    t += norm2(u.a[2][c] - conj(u.a[0][a] * u.a[1][b] - u.a[0][b] * u.a[1][a]));
+  }
+  d[0] = sqrt(s);
+  d[1] = sqrt(t);
+}
+
 // ---------------------------------------------------------------------------
 // gauge conversion: canonical [V][4][3][3] -> even-odd SoA copies
 __global__ void k_gauge_convert(Geom g, const double2* __restrict__ Ucan, double2* U64, float4* U32, float4* U32f,
-                                uint4* U16a, uint2* U16b, double2* U3, float4* U3f, int* flag) {
+                                uint4* U16a, uint2* U16b, double2* U3, float4* U3f, int* flag,
+                                unsigned long long* defect) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.V) return;
   int x = s % g.L, y = (s / g.L) % g.L, z = (s / (g.L * g.L)) % g.L, t = s / (g.L * g.L * g.L);
@@ -140,6 +174,12 @@ __global__ void k_gauge_convert(Geom g, const double2* __restrict__ Ucan, double
       if (!isfinite(e[k].x) || !isfinite(e[k].y)) bad = true;
     }
     if (bad) atomicOr(flag, 1);
+    else {
+      double d[2];
+      su3_defect(e, d);
+      max_to(d[0], defect);
+      max_to(d[1], defect + 1);
+    }
     size_t base = ((size_t)(p * 4 + mu));
     for (int k = 0; k < 9; k++) U64[(base * 9 + k) * g.Vh + i] = e[k];
     for (int q = 0; q < 3; q++)
@@ -245,19 +285,6 @@ __device__ __forceinline__ void pack_block(Cx<double> A[6][6], double* out) {
     }
 }
 
-// *norm = max(*norm, largest row sum of |A_ij|), a bound of the hermitian block's norm
-// (non-negative doubles order like their bits)
-__device__ void max_row_sum(const Cx<double> A[6][6], unsigned long long* norm) {
-  double m = 0;
-  for (int i = 0; i < 6; i++) {
-    double s = 0;
-    for (int j = 0; j < 6; j++) s += sqrt(norm2(A[i][j]));
-    m = fmax(m, s);
-  }
-  const unsigned long long b = (unsigned long long)__double_as_longlong(m);
-  if (b > *(volatile unsigned long long*)norm) atomicMax(norm, b);      // few sites exceed the maximum so far
-}
-
 __global__ void k_clover(Geom g, const double2* __restrict__ Ucan, SigmaBlocks sb, double m0, double csw,
                          double2* C64, double2* Ci64, float4* C32, float4* Ci32, uint4* C16, uint4* Ci16,
                          int* flag, unsigned long long* norms) {
@@ -292,10 +319,10 @@ __global__ void k_clover(Geom g, const double2* __restrict__ Ucan, SigmaBlocks s
             for (int b = 0; b < 3; b++) A[s1 * 3 + a][s2 * 3 + b] = A[s1 * 3 + a][s2 * 3 + b] + f * F[pl][a][b];
         }
     pack_block(A, packed + 36 * ch);
-    max_row_sum(A, norms);
+    max_to(row_sum_norm(A), norms);
     ok = ok && inv6(A, B);
     pack_block(B, packedi + 36 * ch);
-    if (ok) max_row_sum(B, norms + 1);
+    if (ok) max_to(row_sum_norm(B), norms + 1);
   }
   if (!ok) atomicOr(flag, 2);
   for (int k = 0; k < 36; k++) {
@@ -549,10 +576,11 @@ extern "C" dlma_status dlma_set_gauge(dlma_ctx* ctx, const double* links, dlma_m
   CU(cudaMemsetAsync(ctx->flag, 0, 16 * sizeof(int), ctx->stream));
   int nb = (ctx->g.V + 255) / 256;
   k_gauge_convert<<<nb, 256, 0, ctx->stream>>>(ctx->g, Ucan, ctx->U64, ctx->U32, ctx->U32f, ctx->U16a, ctx->U16b,
-                                               ctx->U3, ctx->U3f, ctx->flag);
+                                               ctx->U3, ctx->U3f, ctx->flag, (unsigned long long*)(ctx->flag + 4));
   CHECK_LAUNCH();
   int h = 0;
   CU(cudaMemcpyAsync(&h, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CU(cudaMemcpyAsync(ctx->su3_defect, ctx->flag + 4, sizeof(ctx->su3_defect), cudaMemcpyDeviceToHost, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   ctx->have_params = false;
   ctx->eig_N = 0;
@@ -589,9 +617,15 @@ extern "C" dlma_status dlma_set_params(dlma_ctx* ctx, double m0, double c_sw) {
   }
   ctx->m0 = m0;
   ctx->csw = c_sw;
-  // Dhat = T - D_eo T^-1 D_oe with |D_eo|, |D_oe| <= 4: half the hop is the sum over mu of
-  // S_mu-translations (S + S^dag - g_mu (S - S^dag)) / 2, each of norm 1
-  ctx->schur_norm = norms[0] + 16.0 * norms[1];
+  // Dhat = T - D_eo T^-1 D_oe with |D_eo|, |D_oe| <= 4 u: half the hop is the sum over mu of
+  // (S + S^dag - g_mu (S - S^dag)) / 2, S a translation with links of norm u
+  const double u2 = 1.0 + ctx->su3_defect[0], u = sqrt(u2), dl = ctx->su3_defect[1];
+  ctx->schur_norm = norms[0] + 16.0 * u2 * norms[1];
+  // rounding of the FP32 form (measured: 0.16 ... 0.53 eps32 |Dhat| over random fields,
+  // smooth ones and solutions, clover coefficients 1 ... 2, masses -0.5 ... 2, bounds of
+  // |Dhat| 8 ... 19, 12- and 18-real links), and what rebuilt third rows change: 8 dl in
+  // D_eo and in D_oe
+  ctx->schur_err32 = 2.0 * 1.1920929e-7 * ctx->schur_norm + 64.0 * dl * (u + dl) * norms[1];
   ctx->have_params = true;
   ctx->dirac_N = 0;     // the Dirac low modes belong to the previous operator
   return DLMA_OK;

@@ -394,14 +394,11 @@ __global__ void k_rowsum(const double* part, int nb, int nrhs, double* out, int 
 
 // Split the rhs paused for a reliable update: lo corrects r64 with the FP32 operator's
 // image of x_l, hi recomputes it with the FP64 operator.  The correction leaves two errors
-// in r64: the image's rounding and that of x64 when x_l was folded into it.  The first is
-// below 2 eps32 norm s |x_l|, norm the bound of |Dhat| that set_params took (measured:
-// 0.16 ... 0.53 eps32 norm |x_l| over random fields, smooth ones and solutions, clover
-// coefficients 1 ... 2, masses -0.5 ... 2, norms 8 ... 19, 12- and 18-real links), the
-// second eps64 / 2 norm |x64|.  lo takes those whose errors, added up since their last
-// FP64 evaluation, stay within `limit` times |b|.
+// in r64, the image's, at most err32 s |x_l|, and the rounding of x64 as x_l was folded
+// into it, at most err64 |x64| (bounds from set_params).  lo takes those whose errors,
+// added up since their last FP64 evaluation, stay within `limit` times |b|.
 __global__ void __launch_bounds__(256) k_split_ru(const double* lpart, const double* xpart, int nb, CgScal sc,
-                                                  double norm, double limit, int* ru_hi, int* ru_lo) {
+                                                  double err32, double err64, double limit, int* ru_hi, int* ru_lo) {
   const int j = blockIdx.x;
   const bool on = sc.ru[j] != 0;
   double n[2] = {0, 0};
@@ -413,8 +410,7 @@ __global__ void __launch_bounds__(256) k_split_ru(const double* lpart, const dou
     block_sums<2, 8>(n);
   }
   if (threadIdx.x) return;
-  const double err =
-      sc.rerr[j] + norm * (2.0 * 1.1920929e-7 * sc.scale[j] * sqrt(n[0]) + 1.1102231e-16 * sqrt(n[1]));
+  const double err = sc.rerr[j] + err32 * sc.scale[j] * sqrt(n[0]) + err64 * sqrt(n[1]);
   const bool lo = on && err <= limit * sc.bnorm[j];
   if (on) sc.rerr[j] = lo ? err : 0.0;
   ru_lo[j] = lo;
@@ -911,8 +907,9 @@ static dlma_status fold_residual(dlma_ctx* ctx, SolveBufs& B, int nrhs, double t
                                                 B.part2);
   CHECK_LAUNCH();
   if constexpr (kCorr) {
-    k_split_ru<<<nrhs, 256, 0, ctx->stream>>>(B.part, B.part2, gv.x, B.sc, ctx->schur_norm, kCorrLimit * tol_target,
-                                              B.ru_hi, B.ru_lo);
+    k_split_ru<<<nrhs, 256, 0, ctx->stream>>>(B.part, B.part2, gv.x, B.sc, ctx->schur_err32,
+                                              1.1102231e-16 * ctx->schur_norm, kCorrLimit * tol_target, B.ru_hi,
+                                              B.ru_lo);
     CHECK_LAUNCH();
     TRY(schur_apply(ctx, B.xl, B.t32, B.q32, 0, B.ru_lo, nullptr));
     hi = B.ru_hi;

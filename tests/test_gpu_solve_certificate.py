@@ -20,17 +20,8 @@ def dl():
     return dl
 
 
-@pytest.mark.parametrize("m0", [0.08, -0.08, -0.082])
-@pytest.mark.parametrize("prec,solver", [("FP32", "SOLVER_BICGSTAB"), ("FP32", "SOLVER_CGNE"), ("FP16S", "SOLVER_CGNE")])
-def test_reported_residual(dl, m0, prec, solver):
-    U = synth.gauge_field(L, T, 0.2, 701)
-    eo = dirac.EvenOdd(U, L, T, m0, CSW)
-    b = synth.gaussian_spinors(NRHS, L ** 3 * T, 702)
-    ctx = dl.Context(L, T, 0, 0)
-    ctx.dlma_set_gauge(U)
-    ctx.dlma_set_params(m0, CSW)
-    ctx.dlma_set_solver(getattr(dl, solver))
-    for tol in (1e-8, 1e-10, 1e-12, 1e-13, 1e-14, 2e-15, 3e-16):
+def check(ctx, dl, eo, b, prec, tols):
+    for tol in tols:
         x, info = ctx.dlma_solve(b, tol, getattr(dl, prec), allow_not_converged=True)
         for j in range(NRHS):
             nb = np.linalg.norm(b[j].ravel())
@@ -42,4 +33,34 @@ def test_reported_residual(dl, m0, prec, solver):
             assert abs(got - r) <= 0.05 * r + 0.025 * tol + noise, (tol, j, got, r, noise)
             if info[j]["converged"]:
                 assert r <= 1.05 * tol + noise, (tol, j, got, r)
+
+
+@pytest.mark.parametrize("m0", [0.08, -0.08, -0.082])
+@pytest.mark.parametrize("prec,solver", [("FP32", "SOLVER_BICGSTAB"), ("FP32", "SOLVER_CGNE"), ("FP16S", "SOLVER_CGNE")])
+def test_reported_residual(dl, m0, prec, solver):
+    U = synth.gauge_field(L, T, 0.2, 701)
+    eo = dirac.EvenOdd(U, L, T, m0, CSW)
+    b = synth.gaussian_spinors(NRHS, L ** 3 * T, 702)
+    ctx = dl.Context(L, T, 0, 0)
+    ctx.dlma_set_gauge(U)
+    ctx.dlma_set_params(m0, CSW)
+    ctx.dlma_set_solver(getattr(dl, solver))
+    check(ctx, dl, eo, b, prec, (1e-8, 1e-10, 1e-12, 1e-13, 1e-14, 2e-15, 3e-16))
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec,solver", [("FP32", "SOLVER_BICGSTAB"), ("FP32", "SOLVER_CGNE"), ("FP16S", "SOLVER_CGNE")])
+def test_links_off_su3(dl, prec, solver, monkeypatch):
+    # third rows 1e-4 off: the 12-real FP32 links rebuild other ones than FP64 reads
+    monkeypatch.setenv("DLMA_FORCE_LINKS", "12")
+    rng = np.random.Generator(np.random.PCG64(703))
+    U = synth.gauge_field(L, T, 0.2, 701)
+    U[..., 2, :] += 1e-4 * (rng.standard_normal(U[..., 2, :].shape) + 1j * rng.standard_normal(U[..., 2, :].shape))
+    eo = dirac.EvenOdd(U, L, T, 0.08, CSW)
+    b = synth.gaussian_spinors(NRHS, L ** 3 * T, 702)
+    ctx = dl.Context(L, T, 0, 0)
+    ctx.dlma_set_gauge(U)
+    ctx.dlma_set_params(0.08, CSW)
+    ctx.dlma_set_solver(getattr(dl, solver))
+    check(ctx, dl, eo, b, prec, (1e-8, 1e-10))
     ctx.close()
