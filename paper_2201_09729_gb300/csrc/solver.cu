@@ -44,7 +44,7 @@ struct CgScal {
   int* iters;      // inner iterations in total
   int* since;      // inner iterations since the last update
   int* nupd;       // reliable updates
-  double* rbest;   // smallest FP64 residual seen at an update
+  double* rbest;   // smallest residual seen at an update
   int* stall;      // consecutive updates without halving rbest
   int* rst;        // restart the search direction at this update (p = r)
   int* cf;         // mask of the final full-lattice residual evaluation
@@ -471,13 +471,13 @@ __global__ void k_mark_exact(int nrhs, CgScal sc) {
 }
 
 // rhs whose reported residual still needs an FP64 evaluation on the full lattice:
-// stopped before converging, or retired without an FP64 residual
+// stopped before converging, or retired without an update's residual
 __global__ void k_final_mask(int nrhs, CgScal sc) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < nrhs) sc.cf[j] = sc.alive[j] || !sc.exact[j];
 }
 
-// after the FP64 residual of the paused rhs: retire the converged, mark the rest for resumption
+// after the update's residual of the paused rhs: retire the converged, mark the rest for resumption
 __global__ void k_ru_check(int nrhs, CgScal sc, double tol) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nrhs || !sc.ru[j]) return;
@@ -926,7 +926,7 @@ static dlma_status fold_residual(dlma_ctx* ctx, SolveBufs& B, int nrhs, double t
   return DLMA_OK;
 }
 
-// Reliable update of the rhs in mask ru: x64 += s x_l, x_l = 0; r64 = bhat - Dhat x64 (FP64);
+// Reliable update of the rhs in mask ru: x64 += s x_l, x_l = 0; r64 = bhat - Dhat x64 (fold_residual);
 // retire the converged ones; for the others r_l = Dhat^dag (r64 / s) and resume.
 // first: the initial update (nothing to fold); restart: also reset p = r (a plain
 // defect-correction restart, used with the FP16 stencil whose rounding makes the
@@ -1198,10 +1198,10 @@ static dlma_status solve_finish(dlma_ctx* ctx, SolveBufs& B, double* x_dev, int 
   }
   TRY(unpack_parity(ctx, B.x64, 1, 0, x_dev));
   TRY(unpack_parity(ctx, B.t64o, 1, 1, x_dev));
-  // reported residual ||b - D x|| / ||b||: for an rhs retired on an FP64 residual it is
-  // that residual, |bhat - Dhat x_e| (x_o above makes the odd rows of b - D x vanish);
-  // the rest (stopped early, or retired on a recursive residual) are evaluated on the
-  // full lattice in FP64 here
+  // reported residual ||b - D x|| / ||b||: for an rhs retired at a reliable update it is
+  // that update's, |bhat - Dhat x_e| (x_o above makes the odd rows of b - D x vanish);
+  // the rest (stopped early, or without an update) are evaluated on the full lattice in
+  // FP64 here
   k_final_mask<<<(nrhs + 127) / 128, 128, 0, ctx->stream>>>(nrhs, B.sc);
   CHECK_LAUNCH();
   const int* fm = B.sc.cf;
@@ -1411,8 +1411,8 @@ static dlma_status bicg_iteration(dlma_ctx* ctx, SolveBufs& B, int nrhs, int max
   return DLMA_OK;
 }
 
-// Reliable update of the paused rhs: x64 += s x_l, x_l = 0, r64 = bhat - Dhat x64 in
-// FP64; the converged retire; the rest continue with r_l = r64 / s and rho = (r0, r_l),
+// Reliable update of the paused rhs: x64 += s x_l, x_l = 0, r64 = bhat - Dhat x64
+// (fold_residual); the converged retire; the rest continue with r_l = r64 / s and rho = (r0, r_l),
 // restarting p = r_l on the first update, after a breakdown or on stagnation.
 template <int P>
 static dlma_status bicg_update(dlma_ctx* ctx, SolveBufs& B, int nrhs, double tol_target, double delta, bool first) {
