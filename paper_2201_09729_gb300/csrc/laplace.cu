@@ -987,7 +987,9 @@ static void cheb_coefficients(Eig& E, int d, std::vector<double>& hc, std::vecto
 // size, rms of V^dag V - 1 4e-15 ... 6e-15; double-float's grows with the rows per sum,
 // n / nsplit: 3.7e-15 at 375 rows (10^3 x 18, 40 columns), 4.6e-15 at 1263 (20^3 x 8, 48),
 // 5.9e-15 at 1365 (16^3 x 16, 64), 9.3e-15 at 3072 (16^3 x 32, 64), either side of 5e-15
-// between 860 and 1270.  From 4e9 multiply-adds on always.
+// between 860 and 1270.  (The eigenvalues come out to an rms of 6e-15 ... 1e-14 with
+// double-float and 2e-15 ... 8e-15 with the digits, both far below any tol.)  From 4e9
+// multiply-adds on always.
 static bool tc_products(int n, int m, int Tn, int nsplit) {
   const double macs = (double)n * m * m * Tn;
   return macs >= 4.0e9 || (macs >= 5.0e7 && n >= 1300 * nsplit);
